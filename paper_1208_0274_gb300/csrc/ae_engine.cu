@@ -467,6 +467,8 @@ struct Search {
     int64_t nhits = 0;        // point hits accumulated in w->hkey/hscore
     double batch_hint = -1;   // expected sweep hit records of the current batch (< 0: no hints)
     ae_stats stats;
+    // the frontier's nodes and entries (its arenas may also hold unused ends of regions)
+    int64_t live_nodes = 0, live_ent = 0;
     int64_t dna_nodes = 0, dna_entries = 0, dna_retries = 0;   // DNA int16x2 route (counted on the host)
     double dna_ratio[5] = {0, 0, 0, 0, 0};   // the last DNA level's outputs per input, by arena kind
     bool dna_ratio_ok = false;
@@ -618,6 +620,8 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
     ensure(w->totals, 64, st);
     ensure(w->ctr, sizeof(LevelCounters), st);
     CU(cudaMemsetAsync(w->ctr.p, 0, sizeof(LevelCounters), st));   // clears the sticky overflow flag
+    live_nodes = F;
+    live_ent = cur_ent;
     bool root_level = d0 < 1;   // the first level of a walk from the root has implicit rows
     while (F > 0 && depth <= L_max_all) {
         if (i16 && (int64_t)(depth + 1) * sc.gmax > opt.int16_limit) {
@@ -651,6 +655,7 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
         ca.items = d_items;
         ca.nodes = ptr<Node>(w->nodes[cur]);
         ca.nnodes = F;
+        ca.live = live_nodes;
         ca.nseg = ptr<uint32_t>(w->cnt[0]);
         ca.ntrip = ptr<uint32_t>(w->cnt[1]);
         ca.stats = ptr<DevStats>(w->stats);
@@ -779,8 +784,8 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
         lf_node_base += lf_node;
         rh_base += hits;
         cur = nxt;
-        F = fr_node;
-        cur_ent = fr_ent;
+        F = live_nodes = fr_node;
+        cur_ent = live_ent = fr_ent;
         ++depth;
         stats.levels++;
         if (i16) stats.levels_int16++;
@@ -828,10 +833,20 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 #define AE_WIDE_ROW_AVG 512
 #endif
 
-// Average parent-row length up to which a level's rows are walked one lane per
-// (node, child) rather than spread one entry per lane (per level on the 100 Mbp
-// text with queries of 10 kbp to 1 Mbp, the walk was the faster layout up to
-// rows of about 250 entries and the spread one from about 270)
+// Average parent-row length up to which a level's rows are packed over the
+// lanes; longer rows are spread one entry per lane.  Per level of the 100 Mbp
+// text with queries of 10 kbp to 1 Mbp (packed against the walk it replaces):
+// rows of 158 entries 2.4 ms against 6.3, 57: 3.3 / 6.2, 59 (2.0 M nodes):
+// 8.3 / 10.7, 30: 10.6 / 11.8, 13: 20.2 / 15.8, 7.2: 26.2 / 38.8, 5.0: 41.8 /
+// 56.5, 2.3: 13.8 / 26.9, 1.5: 3.5 / 7.3; rows of 441 stay with the spread
+// layout (3.1 ms)
+#ifndef AE_PACK_ROW_AVG
+#define AE_PACK_ROW_AVG 300
+#endif
+
+// Average parent-row length up to which the walk layout is taken instead of
+// the spread one where rows are not packed: inside the fixed arena of the
+// no-allocation entry point, whose room the regions' unused ends would take
 #ifndef AE_SEQ_ROW_AVG
 #define AE_SEQ_ROW_AVG 256
 #endif
@@ -848,14 +863,17 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
     const int nxt = cur ^ 1;
     // nodes per task: 32 (one per lane) unless the level is too small to give
     // every resident warp a few tasks
-    const int64_t warps = (int64_t)num_sms * ae_rows_dna_blocks_per_sm() * ae_rows_dna_warps_per_block();
-    const int npt = (int)std::max<int64_t>(1, std::min<int64_t>(32, F / (warps * 4)));
+    const bool packed = opt.row_layout == 0 && !g_arena && live_ent <= AE_PACK_ROW_AVG * live_nodes;
+    const int64_t warps = packed ? (int64_t)num_sms * ae_rows_pack_blocks_per_sm() * ae_rows_pack_warps_per_block()
+                                 : (int64_t)num_sms * ae_rows_dna_blocks_per_sm() * ae_rows_dna_warps_per_block();
+    const int npt = (int)std::max<int64_t>(1, std::min<int64_t>(packed ? ae_rows_pack_nodes() : 32, F / (warps * 4)));
 
     // expected outputs: per kind (frontier entries, leaf entries, frontier
     // nodes, leaf nodes, hits) the previous level's ratio to its input, plus a
     // fifth; the first level of a batch assumes four children per node
     static const double first_ratio[5] = {8.0, 1.0, 4.0, 1.0, 0.25};
-    const double in[5] = {(double)cur_ent, (double)cur_ent, (double)F, (double)F, (double)cur_ent};
+    const double in[5] = {(double)live_ent, (double)live_ent, (double)live_nodes, (double)live_nodes,
+                          (double)live_ent};
     int64_t want[5];
     for (int q = 0; q < 5; ++q) {
         double r = dna_ratio_ok ? dna_ratio[q] * 1.2 : first_ratio[q];
@@ -867,8 +885,18 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
         if (r * in[q] > (double)(1 << 28)) r = std::min(r, 1.5);
         want[q] = (int64_t)(r * in[q]) + 256;
     }
-    want[2] = std::min<int64_t>(want[2], 4 * F);   // a node has at most four children
-    want[3] = std::min<int64_t>(want[3], 4 * F);
+    want[2] = std::min<int64_t>(want[2], 4 * live_nodes);   // a node has at most four children
+    want[3] = std::min<int64_t>(want[3], 4 * live_nodes);
+    // packed layout: a warp takes its frontier space in regions of a sixteenth (entries, per
+    // child index) or an eighth (node records) of what it is expected to write, so that their
+    // unused ends stay a few per cent; node records of small levels are reserved exactly
+    uint32_t region_ent = 0, region_node = 0;
+    if (packed) {
+        region_ent = (uint32_t)std::max<int64_t>(64, std::min<int64_t>(want[0] / (16 * warps), 2048));
+        const int64_t rn = want[2] / (8 * warps);
+        if (rn >= 32) region_node = (uint32_t)std::min<int64_t>(rn, 1024);
+    }
+    const int64_t slack_ent = 4 * warps * (int64_t)region_ent, slack_node = warps * (int64_t)region_node;
     // grow ahead only outside the fixed arena, and only as far as memory allows:
     // a capacity that falls short costs one more run of the level
     auto grow = [&](int64_t fe, int64_t le, int64_t fn, int64_t ln, int64_t h, bool exact) {
@@ -899,7 +927,7 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
                         st);
         });
     };
-    grow(want[0], want[1], want[2], want[3], want[4], false);
+    grow(want[0] + slack_ent, want[1], want[2] + slack_node, want[3], want[4], false);
 
     DnaRowsArgs da;
     memset(&da, 0, sizeof(da));
@@ -908,6 +936,8 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
     da.qv = qv;
     da.nnodes = F;
     da.nodes_per_task = npt;
+    da.region_ent = region_ent;
+    da.region_node = region_node;
     da.leaf_delay = opt.leaf_delay;
     {
         const uint64_t u = (uint64_t)(-(int64_t)sc.ss);
@@ -915,10 +945,11 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
     }
     // short parent rows are walked one lane per (node, child); long rows spread
     // over the lanes (a lone long row would hold its warp alone)
-    da.sequential = (opt.row_layout == 1) || (opt.row_layout == 0 && cur_ent <= AE_SEQ_ROW_AVG * F) ? 1 : 0;
+    da.sequential = (opt.row_layout == 1) || (opt.row_layout == 0 && live_ent <= AE_SEQ_ROW_AVG * live_nodes) ? 1 : 0;
     // a level of few nodes with long rows: one block per node
-    if (opt.row_layout == 3 || (opt.row_layout == 0 && F <= AE_WIDE_NODES && cur_ent >= AE_WIDE_ROW_AVG * F))
+    if (opt.row_layout == 3 || (opt.row_layout == 0 && live_nodes <= AE_WIDE_NODES && live_ent >= AE_WIDE_ROW_AVG * live_nodes))
         da.sequential = 2;
+    if (packed) da.sequential = 3;
     // the walk layout keeps its count phase's rows for the write phase (outside the
     // fixed arena of the no-allocation entry point; without room, rows are computed twice)
     da.stage = nullptr;
@@ -964,7 +995,7 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
         da.hit_cap = cap(w->rhits, sizeof(RangeHit), 1);
         da.ctr = ptr<LevelCounters>(w->ctr);
         prof.mark(K_ROWS);
-        ae_rows_dna(da, num_sms * ae_rows_dna_blocks_per_sm(), st);
+        ae_rows_dna(da, num_sms * (packed ? ae_rows_pack_blocks_per_sm() : ae_rows_dna_blocks_per_sm()), st);
         prof.mark(K_ROWS);
         CU(cudaMemcpyAsync(tot(), w->ctr.p, sizeof(hc), cudaMemcpyDeviceToHost, st));
         sync();
@@ -972,40 +1003,45 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
         if (hc.overflow) throw ae_error{AE_ECUDA};   // the two phases of a task disagreed
     };
     run();
-    int64_t fr_ent = (int64_t)hc.fr_ent, fr_node = (int64_t)hc.fr_node;
     int64_t lf_ent = (int64_t)hc.lf_ent - lf_ent_base, lf_node = (int64_t)hc.lf_node - lf_node_base;
     int64_t hits = (int64_t)hc.hits - rh_base;
+    const int64_t n_ent = (int64_t)(packed ? hc.n_ent : hc.fr_ent), n_node = (int64_t)(packed ? hc.n_node : hc.fr_node);
     const bool retried = hc.retry != 0;
-    if (retried) {
+    for (int again = 1; hc.retry; ++again) {
+        // how the packed layout's regions fall differs a little from run to run
+        if (again > (packed ? 4 : 1)) throw ae_error{AE_ECUDA};
         ++dna_retries;
-        grow(fr_ent, lf_ent, fr_node, lf_node, hits, true);
+        grow((int64_t)hc.fr_ent + again * slack_ent, lf_ent, (int64_t)hc.fr_node + again * slack_node, lf_node, hits, true);
         run();
-        if (hc.retry || (int64_t)hc.fr_ent != fr_ent || (int64_t)hc.fr_node != fr_node ||
+        if ((int64_t)(packed ? hc.n_ent : hc.fr_ent) != n_ent || (int64_t)(packed ? hc.n_node : hc.fr_node) != n_node ||
             (int64_t)hc.lf_ent - lf_ent_base != lf_ent || (int64_t)hc.lf_node - lf_node_base != lf_node ||
             (int64_t)hc.hits - rh_base != hits)
             throw ae_error{AE_ECUDA};   // the same level gave other totals
     }
+    const int64_t fr_ent = (int64_t)hc.fr_ent, fr_node = (int64_t)hc.fr_node;   // extents of the frontier's arenas
     stats.triples += (int64_t)hc.triples;
-    dna_nodes += F;
-    dna_entries += fr_ent + lf_ent;
+    dna_nodes += live_nodes;
+    dna_entries += n_ent + lf_ent;
     {
-        const double out[5] = {(double)fr_ent, (double)lf_ent, (double)fr_node, (double)lf_node, (double)hits};
+        const double out[5] = {(double)n_ent, (double)lf_ent, (double)n_node, (double)lf_node, (double)hits};
         for (int q = 0; q < 5; ++q) dna_ratio[q] = in[q] > 0 ? out[q] / in[q] : 0.0;
         dna_ratio_ok = true;
     }
     if (trace()) {
         fprintf(stderr, "[ae level] dna %s nodes %lld (per task %d) entries %lld triples %lld -> frontier %lld nodes %lld, "
                         "leaf %lld rows %lld%s; %.3f ms\n",
-                da.sequential == 2 ? "block" : da.sequential ? "walk" : "spread", (long long)F, npt, (long long)cur_ent,
-                (long long)hc.triples,
-                (long long)fr_ent, (long long)fr_node, (long long)lf_ent, (long long)lf_node,
+                da.sequential == 3 ? "packed" : da.sequential == 2 ? "block" : da.sequential ? "walk" : "spread",
+                (long long)live_nodes, npt, (long long)live_ent, (long long)hc.triples, (long long)n_ent,
+                (long long)n_node, (long long)lf_ent, (long long)lf_node,
                 retried ? " (run again at exact sizes)" : "", ms_since(t_level));
     }
     lf_ent_base += lf_ent;
     lf_node_base += lf_node;
     rh_base += hits;
-    F = fr_node;
+    F = n_node > 0 ? fr_node : 0;
     cur_ent = fr_ent;
+    live_nodes = n_node;
+    live_ent = n_ent;
 }
 
 // Reduce the hits [from, nhits) of the batch just finished to one record per

@@ -72,6 +72,7 @@ struct ChildrenArgs {
     const WorkItem *items;
     const Node *nodes;
     int64_t nnodes;
+    int64_t live;                         // nodes with a row (the others are empty records), for the statistics
     uint32_t *nseg, *ntrip;               // per node: non-empty children, triples
     DevStats *stats;
 };
@@ -110,6 +111,8 @@ struct LevelCounters {
     unsigned long long overflow, task_c, task_w, wide;   // wide: a task total passed 2^32 - 1
     unsigned long long triples;   // DNA int16x2 route: (child, parent entry) pairs of the level
     unsigned long long retry;     // DNA int16x2 route: a reservation passed an arena's capacity
+    unsigned long long n_ent, n_node;   // packed layout: frontier entries and nodes written (its cursors
+                                        // fr_ent and fr_node also count unused ends of regions)
 };
 
 struct RowsArgs {
@@ -171,8 +174,9 @@ struct DnaRowsArgs {
     int32_t nodes_per_task;
     int32_t leaf_delay;
     uint64_t urec;                        // ceil(2^32 / u), u = -s_s: gap-run lengths without division
-    int32_t sequential;                   // 1: one lane per (node, child) walking the parent row in order
-                                          // (short rows); 0: one lane per parent entry (long rows)
+    int32_t sequential;                   // row layout: 3 rows packed over a warp's lanes, 1 one lane per (node,
+                                          // child) walking the parent row in order, 0 one lane per parent entry,
+                                          // 2 one block per node
     const int32_t *pj;                    // parent arena: column, packed (M | G_a << 16)
     const uint32_t *pmg;
     int32_t *fj;                          // next-level arena (packed rows)
@@ -191,10 +195,16 @@ struct DnaRowsArgs {
     // every row is computed twice
     uint2 *stage;
     int32_t stage_cap;
+    // packed layout: entries and node records a warp takes of the frontier arenas at a
+    // time (0: exactly what it writes)
+    uint32_t region_ent, region_node;
 };
 void ae_rows_dna(const DnaRowsArgs &a, int blocks, cudaStream_t st);
 int ae_rows_dna_blocks_per_sm();
 int ae_rows_dna_warps_per_block();
+int ae_rows_pack_blocks_per_sm();
+int ae_rows_pack_warps_per_block();
+int ae_rows_pack_nodes();   // nodes per task at most
 struct LeafArgs {
     IndexView ix;
     ScoreView sc;

@@ -126,6 +126,12 @@ __device__ __forceinline__ uint64_t reduce_add_u64(uint32_t v) {
     return ((uint64_t)hi << 16) + lo;
 }
 
+__device__ __forceinline__ uint64_t reduce_add_u64_wide(uint64_t v) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(FULL, v, d);
+    return v;
+}
+
 __device__ __forceinline__ uint32_t excl_scan_u32(uint32_t v) {
     const int lane = threadIdx.x & 31;
     uint32_t x = v;
@@ -878,6 +884,515 @@ __global__ void __launch_bounds__(DW * 32, AE_DNA_MINB) k_rows_dna(DnaRowsArgs a
     if (lane == 0 && trip_mine) atomicAdd(&a.ctr->triples, (unsigned long long)trip_mine);
 }
 
+// ---- the packed layout: a task's rows laid end to end over a warp's lanes, one
+// parent entry per lane
+//
+// A task is up to PK_N frontier nodes.  Its prologue puts them into shared
+// memory with an order by their number of children (nodes with four first,
+// single occurrences last), so that the nodes met together have about the same
+// number.  The entries of all rows then pass through the warp 32 at a time: a
+// chunk reads its entries once and computes the rows of the nodes' first
+// children, then of their second ones and so on.  A row lies in consecutive
+// lanes, so the horizontal gap is a max-plus scan segmented by node, as long
+// as the chunk's longest row part, and an output's place is a warp-wide rank.
+// A row that goes on in the next chunk carries its gap key along.
+//
+// Nothing is counted ahead and no row is computed twice: a warp writes the
+// i-th children's rows one after the other into its own i-th region of the
+// frontier arena (region_ent entries at a time, one atomic per region).  A row
+// that does not fit the rest of its region moves to the next one, the part
+// already written with it.  Node records are written at the end of their rows
+// into the warp's node region (or, with region_node 0, into exactly reserved
+// places); its unused end is closed with empty records, which the next level
+// skips.  Rows that leave for the text-position sweep are copied from the
+// region to the leaf arena when complete; they and the range hits are few and
+// reserved exactly.  A reservation past an arena's capacity raises `retry` and
+// is not written; the cursors keep counting.
+constexpr int PK_W = 4;           // warps per block
+#ifndef AE_PACK_ROUNDS
+#define AE_PACK_ROUNDS 2
+#endif
+constexpr int PK_R = AE_PACK_ROUNDS;
+constexpr int PK_N = 32 * PK_R;   // nodes per task at most
+#ifndef AE_PACK_MINB
+#define AE_PACK_MINB 7
+#endif
+
+struct __align__(16) PackRegion {
+    uint64_t pos;    // next free entry
+    uint32_t rem;    // what is left of the region
+    uint32_t part;   // entries written of the row that the last chunk left open
+};
+
+struct PackWarp {
+    PackRegion reg[4];           // the frontier regions by child index
+    int32_t carry[4];            // the open row's horizontal-gap key (0: none)
+    uint64_t off[PK_N];          // the node's row
+    uint32_t cum[PK_N + 1];      // first entry of the k-th node in order; the task's entries
+    uint32_t len[PK_N];          // row length
+    uint32_t item[PK_N];         // query | levels as a single occurrence << 24
+    uint32_t kid[PK_N];          // child letters (2 bits each, in order), 1 << 8: stays (per child), count << 12
+    uint32_t lo[4][PK_N], hi[4][PK_N];   // children's SA ranges, by child index
+    int32_t m[PK_N], H[PK_N];
+    uint32_t qoff[PK_N];
+    uint8_t ord[PK_N];           // the nodes in order
+};
+
+// The parent entry of a lane and what its children's rows take from it: slot A
+// (column j) and slot B (column j + 1) before the horizontal gap, and their
+// keys for it, for a child letter that differs from the column's query letter
+// ([0]) or equals it ([1]).  Dead values are AE_NEG.  A key is M' + column * u
+// > 0; 0 stands for none, since a gap value from key 0 is never positive.
+struct PackEntry {
+    int32_t j, jn, traw, ju, H, m;   // threshold of column x (Theorem 2): max(traw + (x - j) g, 0)
+    int32_t A[2], B[2], kA[2], kB[2];
+    uint32_t gapw;                   // G_a as stored: the high halfword of slot A's word
+    int pA, pB;                      // query letters at j and j + 1
+    bool hasB;                       // slot B exists: j + 1 is a query column and not the next entry's
+};
+
+// One child's outputs of a lane's entry: slot A at j, slot B at j + 1, then a
+// run of run_len columns from rs on whose values fall by u from V0
+struct PackSlot {
+    int32_t MA, MB, rs, V0, run_len, run_hits;
+    bool aliveA, aliveB;
+};
+
+__device__ __forceinline__ void pack_entry(const DnaRowsArgs &a, bool valid, int32_t j, int32_t M, int32_t Ga, int32_t jn,
+                                           int32_t pj, int32_t pM, int pA, int pB, int32_t m, int32_t H, PackEntry &e) {
+    const ScoreView &sc = a.sc;
+    const int32_t strong = -(sc.sg + sc.ss);   // a gap opened from M' lives only if M' > |s_g + s_s| (Eq. 3)
+    e.j = j;
+    e.jn = jn;
+    e.m = m;
+    e.H = H;
+    e.traw = H - 1 - (m - 1 - j) * sc.gmax;
+    e.ju = -j * sc.ss;
+    const int32_t tA = max(e.traw, 0), tB = max(e.traw + sc.gmax, 0);
+    // the vertical gap, max(G_a + s_s, M + s_g + s_s); a dead state (AE_DEAD16) stays below the threshold
+    int32_t gap = max(Ga + sc.ss, M - strong);
+    gap = valid && gap > tA ? gap : AE_NEG;
+    e.gapw = (uint32_t)(gap > 0 ? gap : AE_DEAD16) << 16;
+    const bool adj = valid && pj + 1 == j && pM > 0;
+    e.hasB = valid && j + 1 < m && j + 1 != jn;
+    e.pA = pA;
+    e.pB = pB;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int32_t d = q ? sc.sa : sc.sb;
+        e.A[q] = max(adj && pM + d > tA ? pM + d : AE_NEG, gap);
+        e.B[q] = e.hasB && M + d > tB ? M + d : AE_NEG;
+        e.kA[q] = e.A[q] > strong ? e.A[q] + e.ju : 0;
+        e.kB[q] = e.B[q] > strong ? e.B[q] + e.ju - sc.ss : 0;
+    }
+}
+
+// The horizontal gap at the slots (excl: the keys before this entry) and the
+// run after them (incl: this entry's keys included); o.MA and o.MB hold the
+// slots before it.  Lanes without the child (has false) have no keys before them.
+__device__ __forceinline__ void pack_finish(const DnaRowsArgs &a, const PackEntry &e, bool has, int32_t keyA,
+                                            int32_t excl, int32_t incl, PackSlot &o) {
+    const ScoreView &sc = a.sc;
+    const int32_t u = -sc.ss, base = sc.sg - e.ju;
+    o.MA = max(o.MA, base + excl);
+    o.aliveA = has && o.MA > max(e.traw, 0);
+    o.MB = max(o.MB, base - u + max(excl, keyA));
+    o.aliveB = has && e.hasB && o.MB > max(e.traw + sc.gmax, 0);
+    o.rs = e.hasB ? e.j + 2 : e.j + 1;
+    o.V0 = base - (e.hasB ? 2 * u : u) + incl;
+    if (has && o.V0 > 0 && o.rs < e.jn) {
+        const int32_t rl = min((int32_t)div_small((uint32_t)(o.V0 - 1), a.urec) + 1, e.jn - o.rs);
+        if (e.traw + (o.rs + rl - 1 - e.j) * sc.gmax <= 0) {   // threshold 0 over the whole run
+            o.run_len = rl;
+            if (o.V0 >= e.H) o.run_hits = min(rl, (int32_t)div_small((uint32_t)(o.V0 - e.H), a.urec) + 1);
+        } else {
+            run_of(o.rs, e.jn, incl, sc, e.m, e.H, u, o.run_len, o.run_hits);
+        }
+    }
+}
+
+__device__ __forceinline__ uint32_t pack_hits_of(const PackSlot &o, int32_t H) {
+    return (uint32_t)(o.aliveA && o.MA >= H) + (uint32_t)(o.aliveB && o.MB >= H) + (uint32_t)o.run_hits;
+}
+
+// A lane's live outputs of one child in column order: f(column, M, packed word)
+template <typename F>
+__device__ __forceinline__ void pack_each(const DnaRowsArgs &a, const PackEntry &e, const PackSlot &o, F f) {
+    const uint32_t dead = (uint32_t)AE_DEAD16 << 16;
+    if (o.aliveA) f(e.j, o.MA, ((uint32_t)o.MA & 0xFFFFu) | e.gapw);
+    if (o.aliveB) f(e.j + 1, o.MB, ((uint32_t)o.MB & 0xFFFFu) | dead);
+    for (int32_t r = 0; r < o.run_len; ++r) {
+        const int32_t v = o.V0 + r * a.sc.ss;
+        f(o.rs + r, v, ((uint32_t)v & 0xFFFFu) | dead);
+    }
+}
+
+// A warp's output state besides its entry regions (all values warp-uniform)
+struct PackOut {
+    uint64_t npos;          // next free node record of the warp's region
+    uint32_t nrem;          // what is left of it
+    bool efull, nfull;      // an arena's capacity was passed: nothing is written to it any more
+    uint32_t ents, nodes;   // written to the frontier since the counts were last added up
+};
+
+// Slots of `n` for a warp on one of the level's cursors; ok = within `cap`
+__device__ __forceinline__ uint64_t pack_take(const DnaRowsArgs &a, unsigned long long *cursor, uint64_t n, uint64_t cap,
+                                              int lane, bool &ok) {
+    unsigned long long b = 0;
+    if (lane == 0) b = atomicAdd(cursor, (unsigned long long)n);
+    b = __shfl_sync(FULL, b, 0);
+    ok = b + n <= cap;
+    if (!ok && lane == 0) atomicExch(&a.ctr->retry, 1ull);
+    return b;
+}
+
+// A new region with room for the open row's `part` entries and `need` more; the
+// open row moves with it
+__device__ __forceinline__ void pack_new_region(const DnaRowsArgs &a, PackOut &o, int lane, PackRegion &g, uint32_t part,
+                                                uint32_t need) {
+    const uint64_t old = g.pos - part;
+    // an open row may still grow: twice the room, so that a long row moves a few times only
+    const uint32_t n = max(a.region_ent, part ? 2 * (part + need) : need);
+    const bool had = !o.efull;
+    bool ok;
+    const uint64_t b = pack_take(a, &a.ctr->fr_ent, n, a.fr_ent_cap, lane, ok);
+    if (!ok) o.efull = true;
+    __syncwarp();   // the part written so far is complete
+    if (had && ok)
+        for (uint32_t x = lane; x < part; x += 32) {
+            a.fj[b + x] = a.fj[old + x];
+            a.fmg[b + x] = a.fmg[old + x];
+        }
+    g.pos = b + part;
+    g.rem = n - part;
+}
+
+// Places of `need` node records: the first `room` of them at `at`, the others
+// in a new region, which starts at npos
+struct PackPlace {
+    uint64_t at;
+    uint32_t room;
+};
+
+__device__ __forceinline__ PackPlace pack_node_room(const DnaRowsArgs &a, PackOut &o, int lane, uint32_t need) {
+    PackPlace p = {o.npos, min(need, o.nrem)};
+    o.npos += p.room;
+    o.nrem -= p.room;
+    if (p.room < need) {
+        const uint32_t n = max(a.region_node, need - p.room);
+        bool ok;
+        o.npos = pack_take(a, &a.ctr->fr_node, n, a.fr_node_cap, lane, ok);
+        o.nrem = n;
+        if (!ok) o.nfull = true;
+    }
+    o.nodes += need;
+    return p;
+}
+
+__device__ __forceinline__ void pack_put_node(const DnaRowsArgs &a, uint64_t at, uint32_t lo, uint32_t hi,
+                                              uint32_t item, uint32_t cnt, uint64_t off) {
+    const uint32_t uq = hi - lo == 1 ? (item & 0xFF000000u) + (1u << 24) : 0u;   // levels as a single occurrence
+    uint64_t *d = reinterpret_cast<uint64_t *>(a.fnodes + at);
+    d[0] = (uint64_t)lo | ((uint64_t)hi << 32);
+    d[1] = (uint64_t)((item & 0xFFFFFFu) | uq) | ((uint64_t)cnt << 32);
+    d[2] = off;
+}
+
+// The rows of the task's n nodes
+__device__ __forceinline__ void pack_rows(const DnaRowsArgs &a, PackWarp &w, PackOut &out, int lane, int n) {
+    const unsigned le = lane == 31 ? 0xffffffffu : (1u << (lane + 1)) - 1u, lt = le >> 1;
+    const uint32_t total = w.cum[n];
+    int32_t prev_j = -2, prev_M = 0;   // the last chunk's last entry and the letter after it
+    int prev_p = 255;
+    int sc = 0;                        // the node of the chunk's first entry
+    bool may_hit = false;
+#pragma unroll 1
+    for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+        // ---- which node each lane's entry belongs to
+        const bool cont_in = w.cum[sc] < t0;          // the first row started in an earlier chunk
+        const int x = sc + 1 + lane;
+        const uint32_t start = x < n ? w.cum[x] - t0 : 32u;
+        const unsigned heads = __reduce_or_sync(FULL, start < 32u ? 1u << start : 0u);   // rows starting past lane 0
+        const int si = sc + __popc(heads & le);
+        const int s = w.ord[si];
+        const int first = (heads & le) ? 31 - __clz(heads & le) : 0;   // the row's first lane in this chunk
+        const bool open0 = first == 0 && cont_in;                      // the row goes on from the last chunk
+        const bool in = t0 + lane < total;
+        bool valid = in;
+        const uint32_t k = t0 + lane - w.cum[si];
+        const bool last = in && t0 + lane + 1 == w.cum[si + 1];
+        sc += __popc(heads);
+        if (w.cum[sc + 1] <= t0 + 32) ++sc;
+        const bool cont_out = t0 + 32 < total && w.cum[sc] < t0 + 32;  // the last row goes on
+        const uint32_t kid = w.kid[s];
+        const int32_t m = w.m[s], H = w.H[s];
+        int32_t j = m, jn = m;
+        uint32_t mg = 0;
+        if (valid) {
+            const uint64_t e = w.off[s] + k;
+            j = a.pj[e];
+            mg = a.pmg[e];
+            if (lane == 31 && !last) jn = a.pj[e + 1];
+        }
+        {
+            const int32_t d = __shfl_down_sync(FULL, j, 1);
+            if (lane < 31 && !last) jn = d;
+        }
+        if (valid && ((uint32_t)j >= (uint32_t)m || jn <= j || jn > m)) {   // not a sorted row in [0, m): reported
+            atomicExch(&a.ctr->overflow, 1ull);
+            valid = false;
+        }
+        int pB = 255;
+        if (valid && j + 1 < m) pB = a.qv.codes[w.qoff[s] + (uint32_t)j + 1u];
+        const int32_t M0 = (int32_t)(int16_t)(mg & 0xFFFFu);
+        int pA = __shfl_up_sync(FULL, pB, 1);   // read only when the previous entry is in the previous column
+        int32_t pj = __shfl_up_sync(FULL, j, 1), pM = __shfl_up_sync(FULL, M0, 1);
+        if (lane == 0) {
+            pA = prev_p;
+            pj = prev_j;
+            pM = prev_M;
+        }
+        if (lane == first && !open0) pj = -2;
+        prev_j = __shfl_sync(FULL, j, 31);
+        prev_M = __shfl_sync(FULL, M0, 31);
+        prev_p = __shfl_sync(FULL, pB, 31);
+        PackEntry e;
+        pack_entry(a, valid, j, M0, (int32_t)(int16_t)(mg >> 16), jn, pj, pM, pA, pB, m, H, e);
+        const int nk = in ? (int)(kid >> 12) : 0;
+        const int nkmax = (int)__reduce_max_sync(FULL, (unsigned)nk);
+        const int longest = (int)__reduce_max_sync(FULL, (unsigned)(lane - first)) + 1;
+        // a child's values exceed the largest of its parent's row by at most g (the open
+        // row may carry a gap from the chunk before)
+        may_hit = __any_sync(FULL, valid && M0 + a.sc.gmax >= H) || (cont_in && may_hit);
+        const bool may_leave = __any_sync(FULL, in && ((kid >> 8) & 15u) != (1u << nk) - 1u);
+#pragma unroll 1
+        for (int i = 0; i < nkmax; ++i) {
+            const bool has = valid && i < nk;
+            const int c = (int)((kid >> (2 * i)) & 3u);
+            const bool mA = c == e.pA, mB = c == e.pB;
+            PackSlot o;
+            o.MA = has ? (mA ? e.A[1] : e.A[0]) : AE_NEG;
+            o.MB = has ? (mB ? e.B[1] : e.B[0]) : AE_NEG;
+            o.run_len = o.run_hits = 0;
+            const int32_t keyA = mA ? e.kA[1] : e.kA[0];
+            int32_t incl = has ? max(keyA, mB ? e.kB[1] : e.kB[0]) : 0;
+            const int32_t cin = cont_in ? w.carry[i] : 0;
+            PackRegion g = w.reg[i];
+            const uint32_t part = cont_in ? g.part : 0u;
+            // ---- places: ranks over the warp, one row after the other
+            uint32_t cnt, ci, tot;
+            if (__any_sync(FULL, incl != 0) || cin) {   // some horizontal gap is alive
+                int32_t excl;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    if (d >= longest) break;   // warp-uniform
+                    const int32_t y = __shfl_up_sync(FULL, incl, d);
+                    if (lane - d >= first) incl = max(incl, y);
+                }
+                excl = __shfl_up_sync(FULL, incl, 1);
+                if (lane == first) excl = 0;
+                if (open0) {
+                    incl = max(incl, cin);
+                    excl = max(excl, cin);
+                }
+                pack_finish(a, e, has, keyA, excl, incl, o);
+                cnt = (uint32_t)o.aliveA + (uint32_t)o.aliveB + (uint32_t)o.run_len;
+                if (__any_sync(FULL, cnt > 3u)) {
+                    ci = warp_incl_sum(cnt);
+                    tot = __shfl_sync(FULL, ci, 31);
+                } else {   // counts of two bits
+                    const unsigned b0 = __ballot_sync(FULL, cnt & 1u), b1 = __ballot_sync(FULL, cnt & 2u);
+                    ci = __popc(b0 & le) + 2 * __popc(b1 & le);
+                    tot = __popc(b0) + 2 * __popc(b1);
+                }
+            } else {
+                o.aliveA = o.MA > 0;
+                o.aliveB = o.MB > 0;
+                const unsigned b0 = __ballot_sync(FULL, o.aliveA), b1 = __ballot_sync(FULL, o.aliveB);
+                cnt = (uint32_t)o.aliveA + (uint32_t)o.aliveB;
+                ci = __popc(b0 & le) + __popc(b1 & le);
+                tot = __popc(b0) + __popc(b1);
+            }
+            if (tot + part == 0 && !cont_out) continue;   // warp-uniform: nothing here or from before
+            if (g.rem < tot) pack_new_region(a, out, lane, g, part, tot);
+            const uint64_t epos = g.pos;
+            const uint32_t ex = ci - cnt;
+            if (cnt && !out.efull) {
+                int32_t *dj = a.fj + (epos + ex);
+                uint32_t *dm = a.fmg + (epos + ex);
+                pack_each(a, e, o, [&](int32_t col, int32_t, uint32_t word) {
+                    *dj++ = col;
+                    *dm++ = word;
+                });
+            }
+            // ---- rows that end here: their node records
+            const uint32_t row0 = __shfl_sync(FULL, ex, first);
+            const uint32_t before = open0 ? part : 0u;
+            const uint32_t cells = ci - row0 + before;
+            const bool done = last && has && cells > 0;
+            const bool go = may_leave && has && !((kid >> (8 + i)) & 1u);   // to the sweep
+            out.ents += tot;
+            const unsigned be = __ballot_sync(FULL, done && !go);
+            if (be) {
+                const uint32_t nn = __popc(be);
+                const PackPlace np = pack_node_room(a, out, lane, nn);
+                if (done && !go && !out.nfull) {
+                    const uint32_t r = __popc(be & lt);
+                    pack_put_node(a, r < np.room ? np.at + r : out.npos + (r - np.room), w.lo[i][s], w.hi[i][s],
+                                  w.item[s], cells, epos + row0 - before);
+                }
+                out.npos += nn - np.room;
+                out.nrem -= nn - np.room;
+            }
+            // ---- range hits of the rows that stay
+            if (may_hit) {
+                const uint32_t hc = go ? 0u : pack_hits_of(o, H);
+                if (__any_sync(FULL, hc)) {
+                    const uint32_t hi = warp_incl_sum(hc);
+                    bool ok;
+                    uint64_t h = pack_take(a, &a.ctr->hits, __shfl_sync(FULL, hi, 31), a.hit_cap, lane, ok) + (hi - hc);
+                    if (ok && hc)
+                        pack_each(a, e, o, [&](int32_t col, int32_t M, uint32_t) {
+                            if (M >= H)
+                                a.rhits[h++] = RangeHit{w.lo[i][s], w.hi[i][s], (int32_t)(w.item[s] & 0xFFFFFFu), col, M, 0};
+                        });
+                }
+            }
+            // ---- complete rows that leave for the text-position sweep
+            if (may_leave) {
+                const unsigned bl = __ballot_sync(FULL, done && go);
+                if (bl) {
+                    const uint32_t c = done && go ? cells : 0u, li = warp_incl_sum(c);
+                    const uint32_t lt_ent = __shfl_sync(FULL, li, 31);
+                    bool ok, nok;
+                    const uint64_t b = pack_take(a, &a.ctr->lf_ent, lt_ent, a.lf_ent_cap, lane, ok) + (li - c);
+                    const uint64_t y = pack_take(a, &a.ctr->lf_node, __popc(bl), a.lf_node_cap, lane, nok);
+                    out.ents -= lt_ent;
+                    __syncwarp();   // the rows are complete
+                    if (ok && !out.efull) {
+                        const uint64_t src = epos + row0 - before;
+                        for (uint32_t r = 0; r < c; ++r) {
+                            const uint32_t word = a.fmg[src + r];
+                            a.lj[b + r] = a.fj[src + r];
+                            a.lM[b + r] = mg_lo(word);
+                            a.lGa[b + r] = mg_hi(word);
+                        }
+                    }
+                    if (nok && done && go)
+                        a.inj[y + __popc(bl & lt)] =
+                            Inject{(int32_t)(w.item[s] & 0xFFFFFFu), a.ix.tend[w.lo[i][s]], cells, 0, b};
+                }
+            }
+            // ---- the region after this step, the row left open by this chunk
+            __syncwarp();
+            if (lane == 31) {
+                g.pos = epos + tot;
+                g.rem -= tot;
+                g.part = cont_out ? cells : 0u;
+                w.reg[i] = g;
+                if (cont_out) w.carry[i] = incl;
+            }
+            __syncwarp();
+        }
+    }
+}
+
+__global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsArgs a) {
+    __shared__ PackWarp smem[PK_W];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    PackWarp &w = smem[threadIdx.x >> 5];
+    const int npt = a.nodes_per_task;
+    const uint64_t ntask = (uint64_t)((a.nnodes + npt - 1) / npt);
+    uint64_t trip = 0, ents = 0, nodes = 0;   // (child, parent entry) pairs of this lane; entries and nodes written
+    PackOut out;
+    out.npos = 0;
+    out.nrem = out.ents = out.nodes = 0;
+    out.efull = out.nfull = false;
+    if (lane < 4) {
+        w.reg[lane] = PackRegion{0, 0, 0};
+        w.carry[lane] = 0;
+    }
+    for (;;) {
+        unsigned long long task = 0;
+        if (lane == 0) task = atomicAdd(&a.ctr->task_c, 1ull);
+        task = __shfl_sync(FULL, task, 0);
+        if (task >= ntask) break;
+        // ---- prologue: child ranges, PK_R nodes per lane, then their order
+        Node nd[PK_R];
+        unsigned km[PK_R];
+#pragma unroll
+        for (int r = 0; r < PK_R; ++r) {
+            const int64_t v = (int64_t)task * npt + r * 32 + lane;
+            nd[r] = Node{0, 0, 0, 0, 0};
+            if (r * 32 + lane < npt && v < a.nnodes) nd[r] = a.nodes[v];
+        }
+#pragma unroll
+        for (int r = 0; r < PK_R; ++r) {
+            uint32_t clo[4], chi[4];
+            km[r] = nd[r].cnt ? kids4(a.ix, nd[r].lo, nd[r].hi, clo, chi) : 0u;
+            trip += (uint64_t)__popc(km[r]) * nd[r].cnt;
+            if (!km[r]) continue;
+            const int s = r * 32 + lane;
+            // a child stays in the walk while it has several occurrences, or for
+            // the first leaf_delay levels after it became a single one
+            const bool young = (int)((uint32_t)nd[r].item >> 24) + 1 <= a.leaf_delay;
+            uint32_t kid = (uint32_t)__popc(km[r]) << 12;
+            int i = 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if ((km[r] >> c) & 1u) {
+                    kid |= (uint32_t)c << (2 * i);
+                    if (young || chi[c] - clo[c] >= 2) kid |= 256u << i;
+                    w.lo[i][s] = clo[c];
+                    w.hi[i][s] = chi[c];
+                    ++i;
+                }
+            const int32_t qid = nd[r].item & 0xFFFFFF;
+            w.kid[s] = kid;
+            w.off[s] = nd[r].off;
+            w.len[s] = nd[r].cnt;
+            w.item[s] = (uint32_t)nd[r].item;
+            w.m[s] = a.qv.m[qid];
+            w.H[s] = a.qv.H[qid];
+            w.qoff[s] = (uint32_t)a.qv.off[qid];
+        }
+        int n = 0;
+#pragma unroll
+        for (int k = 4; k > 0; --k) {
+#pragma unroll
+            for (int r = 0; r < PK_R; ++r) {
+                const bool mine = __popc(km[r]) == k;
+                const unsigned b = __ballot_sync(FULL, mine);
+                if (mine) w.ord[n + __popc(b & lt)] = (uint8_t)(r * 32 + lane);
+                n += __popc(b);
+            }
+        }
+        __syncwarp();
+        uint32_t sum = 0;
+#pragma unroll 1
+        for (int b = 0; b < n; b += 32) {
+            const uint32_t ln = b + lane < n ? w.len[w.ord[b + lane]] : 0u, li = warp_incl_sum(ln);
+            if (b + lane < n) w.cum[b + lane] = sum + li - ln;
+            sum += __shfl_sync(FULL, li, 31);
+        }
+        if (lane == 0) w.cum[n] = sum;
+        __syncwarp();
+        if (n) pack_rows(a, w, out, lane, n);
+        ents += out.ents;
+        nodes += out.nodes;
+        out.ents = out.nodes = 0;
+        __syncwarp();
+    }
+    if (!out.nfull)   // the rest of the node region holds empty records
+        for (uint32_t i = lane; i < out.nrem; i += 32) a.fnodes[out.npos + i] = Node{0, 0, 0, 0, 0};
+    trip = reduce_add_u64_wide(trip);
+    if (lane == 0) {
+        if (trip) atomicAdd(&a.ctr->triples, (unsigned long long)trip);
+        if (ents) atomicAdd(&a.ctr->n_ent, (unsigned long long)ents);
+        if (nodes) atomicAdd(&a.ctr->n_node, (unsigned long long)nodes);
+    }
+}
 
 // ---- levels of few nodes with long rows: one block per node
 //
@@ -1215,11 +1730,16 @@ __global__ void __launch_bounds__(WB_T) k_rows_dna_wide(DnaRowsArgs a) {
 
 int ae_rows_dna_blocks_per_sm() { return AE_DNA_MINB; }
 int ae_rows_dna_warps_per_block() { return DW; }
+int ae_rows_pack_blocks_per_sm() { return AE_PACK_MINB; }
+int ae_rows_pack_warps_per_block() { return PK_W; }
+int ae_rows_pack_nodes() { return PK_N; }
 
 void ae_rows_dna(const DnaRowsArgs &a, int blocks, cudaStream_t st) {
     if (a.nnodes <= 0) return;
     ++g_launches;
-    if (a.sequential == 2) {   // one block per node
+    if (a.sequential == 3) {   // rows packed over the lanes
+        k_rows_pack<<<blocks, PK_W * 32, 0, st>>>(a);
+    } else if (a.sequential == 2) {   // one block per node
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

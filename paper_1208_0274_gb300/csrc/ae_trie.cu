@@ -65,7 +65,7 @@ __global__ void k_children(ChildrenArgs a) {
         a.nseg[v] = len ? nseg : 0u;
         a.ntrip[v] = len ? nseg * len : 0u;
     }
-    if (a.stats && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&a.stats->nodes, (unsigned long long)a.nnodes);
+    if (a.stats && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&a.stats->nodes, (unsigned long long)a.live);
 }
 
 // Per node: write its non-empty children as segments at the scanned offsets.
