@@ -190,8 +190,8 @@ void ae_options_default(ae_options *opt);
  * in T of the substrings whose reverse prefixes suffix h), and the forward
  * text (Section 2.3 and Section 5 (1)-(3)).  The suffix array is built on the
  * current CUDA device (ae_suffix_array_device, about 33 bytes of device memory
- * per letter while it runs).  The occurrence blocks are filled from it on the
- * host, and the index is then copied once to the device.
+ * per letter while it runs, beside the index's own 5.5), and the arrays are
+ * filled from it there; the host keeps no copy.
  * Errors: AE_EINVAL (n < 1, unknown letter, bad alphabet), AE_EUNSUPPORTED
  * (n >= 2^31 - 1), AE_ENOMEM, AE_ECUDA. */
 ae_status ae_index_build(const uint8_t *text, int64_t n, int32_t alphabet, ae_index **out);
@@ -211,8 +211,9 @@ ae_status ae_index_build(const uint8_t *text, int64_t n, int32_t alphabet, ae_in
 ae_status ae_index_build_collection(const uint8_t *text, int64_t n, const int64_t *starts, int32_t nseq,
                                    int32_t alphabet, ae_index **out);
 
-/* Write / read an index file (versioned header + checksum).  Load copies to
- * the current device.  Errors: AE_EIO, AE_ENOMEM, AE_ECUDA. */
+/* Write / read an index file (versioned header + checksum).  Save copies the
+ * arrays from the device while it writes; load copies to the current device.
+ * Errors: AE_EIO, AE_ENOMEM, AE_ECUDA. */
 ae_status ae_index_save(const ae_index *idx, const char *path);
 ae_status ae_index_load(const char *path, ae_index **out);
 

@@ -1,4 +1,4 @@
-"""Build libae.so in-tree: seven translation units compiled in parallel for
+"""Build libae.so in-tree: eight translation units compiled in parallel for
 sm_103a, then linked into one shared library next to this file.
 
     python -m paper_1208_0274_gb300.build [--force]
@@ -13,7 +13,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libae.so")
 BUILD = os.path.join(HERE, "_build")
-SOURCES = ["ae_index.cpp", "ae_kernels.cu", "ae_trie.cu", "ae_engine.cu", "ae_mlp.cu", "ae_peak.cu", "ae_rows_dna.cu"]
+SOURCES = ["ae_index.cpp", "ae_kernels.cu", "ae_trie.cu", "ae_engine.cu", "ae_mlp.cu", "ae_peak.cu", "ae_rows_dna.cu",
+           "ae_build.cu"]
 HEADERS = ["ae_internal.h", "ae_kernels.h", "ae_device.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -38,7 +39,7 @@ def build(force=False, verbose=False):
         return OUT
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
-    common = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
+    common = ["-O3", "-std=c++20", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
     common += os.environ.get("AE_NVCC_EXTRA", "").split()   # extra defines for tuning builds
 
     def compile_one(src):

@@ -331,27 +331,26 @@ const uint32_t *dom_table(const ae_index *cidx, int d0, cudaStream_t st) {
     return t;
 }
 
-ae_status upload_index(ae_index *idx) {
-    HostIndex &h = idx->host;
-    size_t occ_b = sizeof(uint32_t) * (size_t)(h.nblocks * h.block_words);
-    size_t tend_b = sizeof(int32_t) * (size_t)h.rows;
-    size_t text_b = (size_t)h.n;
-    size_t sep_b = h.nseq ? sizeof(uint32_t) * (size_t)(h.nblocks * AE_SEP_BLOCK_WORDS) : 0;
-    size_t ends_b = h.nseq ? sizeof(uint32_t) * (size_t)((h.n + 31) / 32) : 0;
+// Device memory of the index's arrays, sized by idx->host
+ae_status alloc_index(ae_index *idx) {
+    const HostIndex &h = idx->host;
+    void **const d[5] = {&idx->d_occ, &idx->d_tend, &idx->d_text, &idx->d_sep, &idx->d_ends};
     if (cudaGetDevice(&idx->device) != cudaSuccess) return AE_ECUDA;
-    if (cudaMalloc(&idx->d_occ, occ_b) != cudaSuccess || cudaMalloc(&idx->d_tend, tend_b) != cudaSuccess ||
-        cudaMalloc(&idx->d_text, text_b) != cudaSuccess ||
-        (h.nseq && (cudaMalloc(&idx->d_sep, sep_b) != cudaSuccess || cudaMalloc(&idx->d_ends, ends_b) != cudaSuccess))) {
-        cudaGetLastError();
-        return AE_ENOMEM;
+    idx->device_bytes = 0;
+    for (int k = 0; k < 5; ++k) {
+        if (!h.bytes(k)) continue;
+        if (cudaMalloc(d[k], h.bytes(k)) != cudaSuccess) {
+            cudaGetLastError();
+            return AE_ENOMEM;
+        }
+        idx->device_bytes += (int64_t)h.bytes(k);
     }
-    if (cudaMemcpy(idx->d_occ, h.occ, occ_b, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(idx->d_tend, h.tend, tend_b, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(idx->d_text, h.text, text_b, cudaMemcpyHostToDevice) != cudaSuccess ||
-        (h.nseq && (cudaMemcpy(idx->d_sep, h.sep, sep_b, cudaMemcpyHostToDevice) != cudaSuccess ||
-                    cudaMemcpy(idx->d_ends, h.ends, ends_b, cudaMemcpyHostToDevice) != cudaSuccess)))
-        return AE_ECUDA;
-    idx->device_bytes = (int64_t)(occ_b + tend_b + text_b + sep_b + ends_b);
+    return AE_OK;
+}
+
+// The device view, once the arrays and idx->host's counts are complete
+void set_view(ae_index *idx) {
+    const HostIndex &h = idx->host;
     IndexView &v = idx->view;
     memset(&v, 0, sizeof(v));
     v.occ = (const uint32_t *)idx->d_occ;
@@ -365,6 +364,18 @@ ae_status upload_index(ae_index *idx) {
     v.rows = h.rows;
     v.sep = (const uint32_t *)idx->d_sep;
     v.ends = (const uint32_t *)idx->d_ends;
+}
+
+// A loaded index to the device; the host arrays are released
+ae_status upload_index(ae_index *idx) {
+    HostIndex &h = idx->host;
+    ae_status st = alloc_index(idx);
+    if (st != AE_OK) return st;
+    void *const d[5] = {idx->d_occ, idx->d_tend, idx->d_text, idx->d_sep, idx->d_ends};
+    for (int k = 0; k < 5; ++k)
+        if (h.bytes(k) && cudaMemcpy(d[k], h.array(k), h.bytes(k), cudaMemcpyHostToDevice) != cudaSuccess) return AE_ECUDA;
+    ae_host_index_free(&h);
+    set_view(idx);
     return AE_OK;
 }
 
@@ -1473,68 +1484,117 @@ ae_status search_core(const ae_index *idx, Workspace *w, const int64_t *offsets,
 
 namespace {
 
-// Section 5 (1)-(2): the suffix array of the reversed text on the device
-// (prefix doubling), the occurrence blocks and text-end array filled from it
-// on the host, then the upload.
-ae_status build_index(ae_index *idx, const uint8_t *codes, int64_t n, int32_t alphabet,
-                      const int64_t *starts = nullptr, int32_t nseq = 0) {
-    // a collection is indexed as its sequences joined by separators (code 0,
-    // letters shifted up by one for the suffix array)
-    std::vector<uint8_t> joined;
-    const uint8_t *sa_codes = codes;
-    int64_t J = n;
-    int sa_sigma = ae_alphabet_sigma(alphabet);
-    if (nseq > 0) {
-        J = n + nseq - 1;
-        try {
-            joined.resize((size_t)J);
-        } catch (...) {
-            return AE_ENOMEM;
-        }
-        int64_t q = 0;
-        for (int32_t k = 0; k < nseq; ++k) {
-            const int64_t b = starts[k], e = k + 1 < nseq ? starts[k + 1] : n;
-            if (k > 0) joined[q++] = 0;
-            for (int64_t p = b; p < e; ++p) joined[q++] = (uint8_t)(codes[p] + 1);
-        }
-        sa_codes = joined.data();
-        sa_sigma += 1;
-    }
-    const int64_t N = J + 1;
-    std::vector<int32_t> sa;
-    try {
-        sa.resize((size_t)N);
-    } catch (...) {
-        return AE_ENOMEM;
-    }
+// Section 5 (1)-(2), all on the device: letter codes, the suffix array of the
+// reversed text (prefix doubling), and the index's arrays filled from it.  A
+// collection is indexed as its sequences joined by separators (code 0, letters
+// shifted up by one for the suffix array).
+ae_status build_index(ae_index *idx, const uint8_t *text, int64_t n, int32_t alphabet, const int64_t *starts,
+                      int32_t nseq) {
+    HostIndex &h = idx->host;
+    memset(&h, 0, sizeof(h));
+    const int sigma = ae_alphabet_sigma(alphabet);
+    const int64_t J = n + (nseq > 0 ? nseq - 1 : 0), N = J + 1;
+    h.alphabet = alphabet;
+    h.sigma = sigma;
+    h.n = n;
+    h.rows = N;
+    h.nseq = nseq;
+    h.block_words = alphabet == AE_DNA ? AE_DNA_BLOCK_WORDS : AE_PROT_BLOCK_WORDS;
+    h.nblocks = (N + AE_ROWS_PER_BLOCK - 1) / AE_ROWS_PER_BLOCK + 1;
     cudaStream_t st = nullptr;
     if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         return AE_ECUDA;
     }
-    uint8_t *d_codes = nullptr;
-    int32_t *d_sa = nullptr;
+    std::vector<void *> bufs;
+    auto alloc = [&](size_t bytes) -> void * {
+        void *p = nullptr;
+        bufs.reserve(bufs.size() + 1);
+        if (cudaMalloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess) {
+            cudaGetLastError();
+            throw ae_error{AE_ENOMEM};
+        }
+        bufs.push_back(p);
+        return p;
+    };
     ae_status res = AE_OK;
-    if (cudaMalloc(&d_codes, (size_t)J) != cudaSuccess || cudaMalloc(&d_sa, sizeof(int32_t) * (size_t)N) != cudaSuccess) {
-        cudaGetLastError();
+    try {
+        res = alloc_index(idx);
+        if (res != AE_OK) throw ae_error{res};
+        // letters (the ASCII text goes through the text-end array's memory)
+        uint8_t *ascii = (uint8_t *)idx->d_tend, *codes = (uint8_t *)idx->d_text;
+        struct Small {
+            uint64_t totals[AE_MAX_SIGMA + 5];
+            int64_t dollar;
+            int bad, bad_sa;
+        } hs;
+        Small *ds = (Small *)alloc(sizeof(Small));
+        CU(cudaMemsetAsync(ds, 0, sizeof(Small), st));
+        CU(cudaMemcpyAsync(ascii, text, (size_t)n, cudaMemcpyHostToDevice, st));
+        ae_encode_queries(ascii, codes, n, alphabet, &ds->bad, st);
+        CU(cudaMemcpyAsync(&hs, ds, sizeof(Small), cudaMemcpyDeviceToHost, st));
+        CU(cudaStreamSynchronize(st));
+        if (hs.bad) throw ae_error{AE_EINVAL};
+        const uint8_t *s = codes;
+        int64_t *d_starts = nullptr;
+        if (nseq > 0) {
+            uint8_t *joined = (uint8_t *)alloc((size_t)J);
+            d_starts = (int64_t *)alloc(sizeof(int64_t) * (size_t)nseq);
+            CU(cudaMemsetAsync(joined, 0, (size_t)J, st));
+            CU(cudaMemsetAsync(idx->d_ends, 0, h.bytes(4), st));
+            CU(cudaMemsetAsync(idx->d_sep, 0, h.bytes(3), st));
+            CU(cudaMemcpyAsync(d_starts, starts, sizeof(int64_t) * (size_t)nseq, cudaMemcpyHostToDevice, st));
+            ae_join_sequences(codes, n, d_starts, nseq, joined, (uint32_t *)idx->d_ends, st);
+            s = joined;
+        }
+        int32_t *sa = (int32_t *)alloc(sizeof(int32_t) * (size_t)N);
+        res = ae_sa_doubling(s, J, sigma + (nseq > 0 ? 1 : 0), 1, sa, nullptr, st);
+        if (res != AE_OK) throw ae_error{res};
+        uint32_t *cnt = (uint32_t *)alloc(sizeof(uint32_t) * (size_t)(sigma + 1) * (size_t)h.nblocks);
+        uint64_t *tmp = (uint64_t *)alloc(8 * (size_t)ae_fill_tmp_words(h.nblocks));
+        CU(cudaMemsetAsync(idx->d_occ, 0, h.bytes(0), st));
+        ae_fill_index(sigma, s, sa, J, d_starts, nseq, (uint32_t *)idx->d_occ, (uint32_t *)idx->d_sep,
+                      (int32_t *)idx->d_tend, h.nblocks, cnt, tmp, ds->totals, &ds->dollar, &ds->bad_sa, st);
+        CU(cudaGetLastError());
+        CU(cudaMemcpyAsync(&hs, ds, sizeof(Small), cudaMemcpyDeviceToHost, st));
+        CU(cudaStreamSynchronize(st));
+        if (hs.bad_sa) throw ae_error{AE_ECUDA};
+        h.dollar_row = hs.dollar;
+        h.C[0] = (uint32_t)(1 + J - n);
+        for (int c = 0; c < sigma; ++c) h.C[c + 1] = h.C[c] + (uint32_t)hs.totals[c];
+        set_view(idx);
+    } catch (const ae_error &err) {
+        res = err.st;
+    } catch (const std::bad_alloc &) {
         res = AE_ENOMEM;
     }
-    if (res == AE_OK && cudaMemcpyAsync(d_codes, sa_codes, (size_t)J, cudaMemcpyHostToDevice, st) != cudaSuccess)
-        res = AE_ECUDA;
-    if (res == AE_OK) res = ae_sa_doubling(d_codes, J, sa_sigma, 1, d_sa, nullptr, st);
-    if (res == AE_OK && (cudaMemcpyAsync(sa.data(), d_sa, sizeof(int32_t) * (size_t)N, cudaMemcpyDeviceToHost, st) !=
-                             cudaSuccess ||
-                         cudaStreamSynchronize(st) != cudaSuccess))
-        res = AE_ECUDA;
     cudaStreamSynchronize(st);
-    if (d_codes) cudaFree(d_codes);
-    if (d_sa) cudaFree(d_sa);
+    cudaGetLastError();
+    for (void *p : bufs) cudaFree(p);
     cudaStreamDestroy(st);
-    if (res == AE_OK)
-        res = nseq > 0 ? ae_host_index_fill_collection(codes, n, starts, nseq, alphabet, sa.data(), &idx->host)
-                       : ae_host_index_fill(codes, n, alphabet, sa.data(), &idx->host);
-    if (res == AE_OK) res = upload_index(idx);
     return res;
+}
+
+// The checks and the build of both entry points
+ae_status new_index(const uint8_t *text, int64_t n, int32_t alphabet, const int64_t *starts, int32_t nseq,
+                    ae_index **out) {
+    ae_index *idx = new (std::nothrow) ae_index();
+    if (!idx) return AE_ENOMEM;
+    ae_status st = build_index(idx, text, n, alphabet, starts, nseq);
+    if (st == AE_OK) {
+        *out = idx;
+        return AE_OK;
+    }
+    delete idx;
+    if (st != AE_EINVAL) {
+        // a letter outside the alphabet is reported as such also where the device
+        // could not be used
+        uint8_t lut[256];
+        ae_letter_lut(alphabet, lut);
+        for (int64_t i = 0; i < n; ++i)
+            if (lut[text[i]] == 255) return AE_EINVAL;
+    }
+    return st;
 }
 
 }  // namespace
@@ -1588,22 +1648,7 @@ ae_status ae_index_build(const uint8_t *text, int64_t n, int32_t alphabet, ae_in
     *out = nullptr;
     if (!text || n < 1 || !ae_alphabet_sigma(alphabet)) return AE_EINVAL;
     if (n + 1 >= INT32_MAX) return AE_EUNSUPPORTED;
-    std::vector<uint8_t> codes;
-    try {
-        codes.resize((size_t)n);
-    } catch (...) {
-        return AE_ENOMEM;
-    }
-    if (ae_encode_letters(text, n, alphabet, codes.data()) != 0) return AE_EINVAL;
-    ae_index *idx = new (std::nothrow) ae_index();
-    if (!idx) return AE_ENOMEM;
-    ae_status st = build_index(idx, codes.data(), n, alphabet);
-    if (st != AE_OK) {
-        delete idx;
-        return st;
-    }
-    *out = idx;
-    return AE_OK;
+    return new_index(text, n, alphabet, nullptr, 0, out);
 }
 
 ae_status ae_index_build_collection(const uint8_t *text, int64_t n, const int64_t *starts, int32_t nseq,
@@ -1614,27 +1659,62 @@ ae_status ae_index_build_collection(const uint8_t *text, int64_t n, const int64_
     for (int32_t k = 1; k < nseq; ++k)
         if (starts[k] < starts[k - 1] || starts[k] > n) return AE_EINVAL;
     if (n + nseq >= INT32_MAX) return AE_EUNSUPPORTED;
-    std::vector<uint8_t> codes;
-    try {
-        codes.resize((size_t)n);
-    } catch (...) {
-        return AE_ENOMEM;
-    }
-    if (ae_encode_letters(text, n, alphabet, codes.data()) != 0) return AE_EINVAL;
-    ae_index *idx = new (std::nothrow) ae_index();
-    if (!idx) return AE_ENOMEM;
-    ae_status st = build_index(idx, codes.data(), n, alphabet, starts, nseq);
-    if (st != AE_OK) {
-        delete idx;
-        return st;
-    }
-    *out = idx;
-    return AE_OK;
+    return new_index(text, n, alphabet, starts, nseq, out);
 }
 
 ae_status ae_index_save(const ae_index *idx, const char *path) {
     if (!idx || !path) return AE_EINVAL;
-    return ae_host_index_save(&idx->host, path);
+    // the arrays are copied from the device by a second thread, one ahead of the
+    // checksum and the writing
+    HostIndex h = idx->host;
+    void *const d[5] = {idx->d_occ, idx->d_tend, idx->d_text, idx->d_sep, idx->d_ends};
+    h.occ = (uint32_t *)malloc(h.bytes(0));
+    h.tend = (int32_t *)malloc(h.bytes(1));
+    h.text = (uint8_t *)malloc(h.bytes(2));
+    if (h.nseq) {
+        h.sep = (uint32_t *)malloc(h.bytes(3));
+        h.ends = (uint32_t *)malloc(h.bytes(4));
+    }
+    ae_status res = AE_OK;
+    for (int k = 0; k < 5; ++k)
+        if (h.bytes(k) && !h.array(k)) res = AE_ENOMEM;
+    if (res == AE_OK) {
+        std::atomic<int> have{0};   // arrays copied; -1: a copy failed
+        const int device = idx->device, arrays = h.nseq ? 5 : 3;
+        auto fetch = [&] {
+            bool ok = cudaSetDevice(device) == cudaSuccess;
+            for (int k = 0; ok && k < arrays; ++k) {
+                ok = cudaMemcpy(h.array(k), d[k], h.bytes(k), cudaMemcpyDeviceToHost) == cudaSuccess;
+                if (ok) have.fetch_add(1);
+                have.notify_all();
+            }
+            if (!ok) {
+                have.store(-1);
+                have.notify_all();
+            }
+        };
+        auto ready = [&](int k) {
+            for (int v = have.load(); v >= 0 && v <= k; v = have.load()) have.wait(v);
+            return have.load() >= 0;
+        };
+        std::thread th;
+        try {
+            th = std::thread(fetch);
+        } catch (const std::system_error &) {
+            int dev = 0;
+            cudaGetDevice(&dev);
+            fetch();
+            cudaSetDevice(dev);
+        }
+        res = ae_host_index_save(&h, path, ready);
+        if (th.joinable()) th.join();
+        if (have.load() < 0) {
+            cudaGetLastError();
+            res = AE_ECUDA;
+        }
+    }
+    ae_host_index_free(&h);
+    return res;
 }
 
 ae_status ae_index_load(const char *path, ae_index **out) {

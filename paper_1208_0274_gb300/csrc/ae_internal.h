@@ -5,6 +5,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <functional>
+
 #include "ae.h"
 
 #ifdef __CUDACC__
@@ -126,6 +128,8 @@ struct DevStats {
 };
 
 // ---------------------------------------------------------------- host index
+// Sizes and letter counts of an index; its arrays are on the host only while a
+// file is read or written.
 struct HostIndex {
     int32_t alphabet, sigma;
     int64_t n;
@@ -140,20 +144,26 @@ struct HostIndex {
     int32_t nseq;      // sequences of a collection (0: a single text)
     uint32_t *sep;     // collections: nblocks * AE_SEP_BLOCK_WORDS
     uint32_t *ends;    // collections: (n + 31) / 32 words
+
+    // the arrays in file order (0 occ, 1 tend, 2 text, 3 sep, 4 ends) and their sizes
+    void *array(int k) const {
+        void *const a[5] = {occ, tend, text, sep, ends};
+        return a[k];
+    }
+    size_t bytes(int k) const {
+        const size_t b[5] = {sizeof(uint32_t) * (size_t)(nblocks * block_words), sizeof(int32_t) * (size_t)rows, (size_t)n,
+                             nseq ? sizeof(uint32_t) * (size_t)(nblocks * AE_SEP_BLOCK_WORDS) : 0,
+                             nseq ? sizeof(uint32_t) * (size_t)((n + 31) / 32) : 0};
+        return b[k];
+    }
 };
 
 int ae_alphabet_sigma(int32_t alphabet);
 int ae_encode_letters(const uint8_t *ascii, int64_t n, int32_t alphabet, uint8_t *codes);
 void ae_letter_lut(int32_t alphabet, uint8_t lut[256]);
-ae_status ae_host_index_fill(const uint8_t *codes, int64_t n, int32_t alphabet, const int32_t *sa, HostIndex *out);
-// The index of a collection: codes[0..n) are the sequences back to back,
-// starts[0..nseq) their first positions (starts[0] = 0, non-decreasing); sa is
-// the suffix array of the reversed joined text (nseq - 1 separators of code 0,
-// letters shifted up by one) followed by the sentinel.
-ae_status ae_host_index_fill_collection(const uint8_t *codes, int64_t n, const int64_t *starts, int32_t nseq,
-                                        int32_t alphabet, const int32_t *sa, HostIndex *out);
 void ae_host_index_free(HostIndex *h);
-ae_status ae_host_index_save(const HostIndex *h, const char *path);
+// ready(k) waits until array k is there (false: it could not be had)
+ae_status ae_host_index_save(const HostIndex *h, const char *path, const std::function<bool(int)> &ready);
 ae_status ae_host_index_load(const char *path, HostIndex *h);
 
 // Device view of a built index (pointers into the index's device memory).

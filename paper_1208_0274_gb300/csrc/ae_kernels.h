@@ -31,6 +31,20 @@ int ae_radix_sort(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_
 ae_status ae_sa_doubling(const uint8_t *d_codes, int64_t n, int sigma, int reversed, int32_t *d_sa, int *rounds,
                          cudaStream_t st);
 
+// Index build (ae_build.cu).  ae_join_sequences: the collection's codes joined by
+// separators (code 0, letters + 1; `joined` zeroed, n + nseq - 1 bytes) and the
+// bitmap of sequence ends (zeroed).  ae_fill_index: occurrence blocks (zeroed),
+// text ends and separator records (zeroed, NULL for one text) from the suffix
+// array `sa` of s[0..J) reversed; totals[0..sigma] receive the letters' and the
+// separators' numbers (room for sigma + 5), *dollar the sentinel's row, *bad 2 on
+// an entry out of range.  cnt: (sigma + 1) x nblocks words, tmp: ae_fill_tmp_words.
+void ae_join_sequences(const uint8_t *codes, int64_t n, const int64_t *starts, int32_t nseq, uint8_t *joined,
+                       uint32_t *ends, cudaStream_t st);
+int64_t ae_fill_tmp_words(int64_t nblocks);
+void ae_fill_index(int sigma, const uint8_t *s, const int32_t *sa, int64_t J, const int64_t *starts, int32_t nseq,
+                   uint32_t *occ, uint32_t *sep, int32_t *tend, int64_t nblocks, uint32_t *cnt, uint64_t *tmp,
+                   uint64_t *totals, int64_t *dollar, int *bad, cudaStream_t st);
+
 // Query letters -> codes; sets *bad (device int) on an unknown letter.
 void ae_encode_queries(const uint8_t *ascii, uint8_t *codes, int64_t total, int alphabet, int *bad,
                        cudaStream_t st);
