@@ -172,8 +172,9 @@ typedef struct {
     int32_t fork_part;
     int32_t leaf_wide_rows;   /* a walk of the text-position sweep whose row grows past this many
                                  entries continues on a whole thread block (each step spread over
-                                 its threads) instead of one warp; 0: never.  Default 128.  The
-                                 results are the same */
+                                 its threads) instead of one warp; 0: never.  Default 128; values
+                                 from 128 to 1,024 count as 1,024 where rows are injected at most
+                                 text positions.  The results are the same */
 } ae_options;
 
 /* Fill *opt with the defaults: qprefix_seed 1, leaf_segment 0, item_columns

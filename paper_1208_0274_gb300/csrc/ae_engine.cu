@@ -173,12 +173,12 @@ struct Workspace {
     // point hits of the whole search
     DevBuf hkey, hscore, hcount, hk1, hv1;
     // leaf sweep scratch; walks handed on to blocks (state, count, row buffers)
-    DevBuf scratch, next_seg, esc, esc_count, esc_rows;
+    DevBuf scratch, next_seg, esc, esc_count, esc_pool, wide_rows;
     // walk layout of the DNA row kernel: per warp and lane, the count phase's child rows
     DevBuf stage;
     // output
     DevBuf uniq, uflags, uoff, qcount;
-    DevBuf stats, segs, ctr, seg_cnt, seg_hit, task_first, task_tot, task_off, task_tmp, task_sum, res, res_key;
+    DevBuf stats, stats_keep, segs, ctr, seg_cnt, seg_hit, task_first, task_tot, task_off, task_tmp, task_sum, res, res_key;
     double fr_ratio = 1.2, lf_ratio = 0.6, hit_ratio = 0.5;
     // pinned host staging
     uint64_t *h_tot = nullptr;
@@ -192,7 +192,7 @@ struct Workspace {
     std::vector<cudaStream_t> out_st;
     std::vector<cudaEvent_t> out_ev;
     cudaEvent_t out_ready = nullptr;
-    int32_t leaf_cap = 0;
+    int32_t leaf_cap = 0, wide_cap = 0;   // row capacity of the sweep's warps and blocks
     std::mutex busy;              // one search at a time per workspace (per stream)
 
     int64_t device_bytes() {
@@ -207,7 +207,7 @@ struct Workspace {
                 &aM[1], &aGa[0], &aGa[1], &nodes[0], &nodes[1], &cnt[0], &cnt[1], &cnt[2], &cnt[3],
                 &cnt[4], &off[0], &off[1], &off[2], &off[3], &off[4], &totals, &scan_tmp, &lj, &lM,
                 &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hkey, &hscore, &hcount, &hk1,
-                &hv1, &scratch, &next_seg, &esc, &esc_count, &esc_rows, &stage, &uniq, &uflags, &uoff, &qcount, &stats, &segs, &ctr, &seg_cnt, &seg_hit,
+                &hv1, &scratch, &next_seg, &esc, &esc_count, &esc_pool, &wide_rows, &stage, &uniq, &uflags, &uoff, &qcount, &stats, &stats_keep, &segs, &ctr, &seg_cnt, &seg_hit,
                 &task_first, &task_tot, &task_off, &task_tmp, &task_sum, &res, &res_key};
     }
 
@@ -230,7 +230,7 @@ struct Workspace {
     void trim_batch() {
         DevBuf *drop[] = {&aj[0], &aj[1], &aM[0], &aM[1], &aGa[0], &aGa[1], &nodes[0], &nodes[1], &cnt[0], &cnt[1],
                           &cnt[2], &cnt[3], &cnt[4], &off[0], &off[1], &off[2], &off[3], &off[4], &scan_tmp, &lj,
-                          &lM, &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hk1, &hv1, &scratch, &esc_rows,
+                          &lM, &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hk1, &hv1, &scratch, &esc_pool, &wide_rows,
                           &uniq,
                           &uflags, &uoff, &segs, &seg_cnt, &seg_hit, &task_first, &task_tot, &task_off, &task_tmp,
                           &res, &res_key};
@@ -241,7 +241,7 @@ struct Workspace {
                 b->p = nullptr;
                 b->bytes = 0;
             }
-        leaf_cap = 0;
+        leaf_cap = wide_cap = 0;
     }
 
     // Forget every carved buffer (the next static call carves them again).
@@ -476,6 +476,7 @@ struct Search {
     int be, bj, bq;
     int d0;
     int64_t nhits = 0;        // point hits accumulated in w->hkey/hscore
+    int64_t batch_queries = 1; // work items of the current batch
     double batch_hint = -1;   // expected sweep hit records of the current batch (< 0: no hints)
     ae_stats stats;
     // the frontier's nodes and entries (its arenas may also hold unused ends of regions)
@@ -519,6 +520,7 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
     }
     const int sigma = ix.sigma;
     const int64_t batch_hits0 = nhits;
+    batch_queries = (int64_t)items.size();
     const int nitems = (int)items.size();
     ensure(w->items, sizeof(WorkItem) * items.size(), st);
     CU(cudaMemcpyAsync(w->items.p, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, st));
@@ -829,10 +831,23 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 #define AE_STAGE_ROWS 256
 #endif
 
-// Slots for sweep walks handed on to thread blocks (12 row buffers of the
-// sweep's row capacity each; a walk that finds no free slot stays on its warp)
+// Slots for sweep walks handed on to thread blocks and the entries of the pool
+// their rows wait in (a walk that finds no room stays on its warp)
 #ifndef AE_LEAF_WIDE_SLOTS
-#define AE_LEAF_WIDE_SLOTS 512
+#define AE_LEAF_WIDE_SLOTS 16384
+#endif
+#ifndef AE_LEAF_WIDE_POOL
+#define AE_LEAF_WIDE_POOL (1 << 22)
+#endif
+
+// Sweep tasks are cut at gaps of more than AE_LEAF_GAP text positions between
+// injections, as long as a query's injections lie at least half that far apart
+// on average over the text (denser ones leave too few gaps to cut at).  Cut at
+// multiples of 32 injections instead, each part of a homologous region walked on
+// to the region's end beside the others: 13 times the cells and hit records on
+// six homologous reads (sweep 100 ms against 17)
+#ifndef AE_LEAF_GAP
+#define AE_LEAF_GAP 64
 #endif
 
 // Levels of at most AE_WIDE_NODES nodes whose rows average AE_WIDE_ROW_AVG
@@ -1146,32 +1161,51 @@ void Search::leaf_phase(int64_t ninj) {
                               ptr<uint64_t>(w->sort_tmp), st);
     prof.mark(K_SORT);
     const uint32_t *order = which ? ptr<uint32_t>(w->sv1) : ptr<uint32_t>(w->sv0);
+    const uint64_t *keys = which ? ptr<uint64_t>(w->sk1) : ptr<uint64_t>(w->sk0);
 
     const int threads = 128;
     const int blocks = num_sms * (g_arena ? 2 : 12);
     const int nwarps = blocks * threads / 32;
     if (w->leaf_cap < opt.leaf_capacity) w->leaf_cap = opt.leaf_capacity;
+    w->wide_cap = std::max(w->wide_cap, opt.leaf_capacity);
+    const int wide_blocks = num_sms * ae_leaf_wide_blocks_per_sm();
     ensure(w->next_seg, 8, st);
     ensure(w->hcount, 8, st);
     int64_t hit_cap = std::max<int64_t>(1 << 20, batch_hint >= 0 ? (int64_t)(1.25 * batch_hint) + 65536
                                                                  : (int64_t)(ninj * w->hit_ratio) + 4096);
     // wide walks move to blocks (not inside the fixed arena of the no-allocation
     // entry point, nor when entries are counted by tier, which only the warp walk does)
-    const int32_t esc_min = (g_arena || opt.tier_stats) ? 0 : opt.leaf_wide_rows;
+    const bool sparse = (double)ninj * (AE_LEAF_GAP / 2) <= (double)ix.n * batch_queries;
+    // (where injections are dense every task walks a wide row and warps are the better
+    // use of the chip: 1 M residues, BLOSUM62: blocks from rows of 128 entries on 153 ms,
+    // 512: 173, 1,024: 91, never: 103)
+    const int32_t esc_min = (g_arena || opt.tier_stats || opt.leaf_wide_rows == 0) ? 0
+                            : sparse || opt.leaf_wide_rows < 128                 ? opt.leaf_wide_rows
+                                                                                 : std::max(opt.leaf_wide_rows, 1024);
     const int32_t esc_max = esc_min > 0 ? AE_LEAF_WIDE_SLOTS : 0;
+    // the counters before the sweep: one that is run again counts once
+    ensure(w->stats_keep, sizeof(DevStats), st);
+    CU(cudaMemcpyAsync(w->stats_keep.p, w->stats.p, sizeof(DevStats), cudaMemcpyDeviceToDevice, st));
     for (int attempt = 0; attempt < 12; ++attempt) {
+        if (attempt) CU(cudaMemcpyAsync(w->stats.p, w->stats_keep.p, sizeof(DevStats), cudaMemcpyDeviceToDevice, st));
         ensure(w->scratch, (size_t)ae_leaf_scratch_words(w->leaf_cap, nwarps) * 4, st);
         if (esc_max > 0) {
             ensure(w->esc, (size_t)esc_max * sizeof(EscWalk), st);
-            ensure(w->esc_count, 8, st);
-            ensure(w->esc_rows, (size_t)esc_max * 12 * (size_t)w->leaf_cap * 4, st);
-            CU(cudaMemsetAsync(w->esc_count.p, 0, 8, st));
+            ensure(w->esc_count, 24, st);
+            ensure(w->esc_pool, (size_t)AE_LEAF_WIDE_POOL * 12, st);
+            ensure(w->wide_rows, (size_t)wide_blocks * 12 * (size_t)w->wide_cap * 4, st);
+            CU(cudaMemsetAsync(w->esc_count.p, 0, 24, st));
         }
         hits_reserve(hit_cap);
+        // all of the buffers' room is used (a search that wrote many hits once finds them
+        // large enough the next time)
+        hit_cap = std::max(hit_cap, (int64_t)std::min(w->hkey.bytes / sizeof(uint64_t), w->hscore.bytes / sizeof(int32_t)) -
+                                        nhits);
         CU(cudaMemsetAsync(w->next_seg.p, 0, 8, st));
         unsigned long long base = (unsigned long long)nhits;
         CU(cudaMemcpyAsync(w->hcount.p, &base, 8, cudaMemcpyHostToDevice, st));
         CU(cudaMemsetAsync((char *)w->stats.p + offsetof(DevStats, leaf_overflow), 0, 16, st));
+        CU(cudaMemsetAsync((char *)w->stats.p + offsetof(DevStats, wide_overflow), 0, 8, st));
         LeafArgs la;
         memset(&la, 0, sizeof(la));
         la.ix = ix;
@@ -1207,8 +1241,14 @@ void Search::leaf_phase(int64_t ninj) {
         if (esc_max > 0) {
             la.esc_count = ptr<unsigned long long>(w->esc_count);
             la.esc = ptr<EscWalk>(w->esc);
-            la.esc_rows = ptr<int32_t>(w->esc_rows);
+            la.esc_pool = ptr<int32_t>(w->esc_pool);
+            la.esc_pool_cap = AE_LEAF_WIDE_POOL;
+            la.wide_rows = ptr<int32_t>(w->wide_rows);
+            la.wide_cap = w->wide_cap;
+            la.wide_blocks = wide_blocks;
         }
+        la.keys = keys;
+        la.gap = sparse ? AE_LEAF_GAP : 0;
         prof.mark(K_LEAF);
         ++stats.leaf_sweeps;
         const auto t_sweep = std::chrono::steady_clock::now();
@@ -1220,6 +1260,8 @@ void Search::leaf_phase(int64_t ninj) {
         CU(cudaMemcpyAsync(tot() + 1, (char *)w->stats.p + offsetof(DevStats, leaf_overflow), 16,
                            cudaMemcpyDeviceToHost, st));
         if (esc_max > 0) CU(cudaMemcpyAsync(tot() + 3, w->esc_count.p, 8, cudaMemcpyDeviceToHost, st));
+        CU(cudaMemcpyAsync(tot() + 4, (char *)w->stats.p + offsetof(DevStats, wide_overflow), 8, cudaMemcpyDeviceToHost,
+                           st));
         sync();
         hdr[0] = tot()[0];
         hdr[1] = tot()[1];
@@ -1229,6 +1271,11 @@ void Search::leaf_phase(int64_t ninj) {
             fprintf(stderr, "[ae leaf] injections %lld (tasks %lld of %d) attempt %d: %.2f ms, hits %llu (cap %lld), row overflow %llu, hit overflow %llu, cap %d\n",
                     (long long)ninj, (long long)la.nseg, la.seg, attempt, ms_since(t_sweep),
                     hdr[0] - (unsigned long long)nhits, (long long)hit_cap, hdr[1], hdr[2], w->leaf_cap);
+        if (tot()[4] != 0) {        // a row outgrew the blocks' buffers: retry larger
+            if (w->wide_cap >= (1 << 28)) throw ae_error{AE_ENOMEM};
+            w->wide_cap *= 4;
+            continue;
+        }
         if (hdr[1] != 0) {          // a row outgrew the scratch: retry larger
             // a sweep row holds at most two entries per query column plus gap runs, so
             // a capacity past 2^28 entries means something else is wrong: stop

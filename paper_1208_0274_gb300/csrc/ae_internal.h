@@ -124,7 +124,7 @@ struct DevStats {
     unsigned long long reused;            // sweep: injected entries absorbed by a walked row at their position
     unsigned long long cand, pruned_nonpos, pruned_reach;   // tier_stats: slot candidates of the trie
                                                             // levels and those the filters dropped
-    unsigned long long pad;
+    unsigned long long wide_overflow;     // sweep: a row outgrew a block's buffers
 };
 
 // ---------------------------------------------------------------- host index

@@ -26,6 +26,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 
 #include "ae_device.cuh"
@@ -615,6 +616,31 @@ __device__ __forceinline__ void leaf_merge(const LeafArgs &a, int lane, int32_t 
     }
 }
 
+// First injection of task s.  Rows injected close to each other, as along a
+// homologous region, belong to one walk: cut apart, each part's walk would run
+// on to the region's end beside the others, over the same cells.  So a task
+// starts where the injections leave a gap.  A stretch of TASK_REACH injections
+// without one is cut at the multiple of seg.  The result depends on s alone and
+// does not decrease.
+constexpr int64_t TASK_REACH = 65536;
+__device__ __forceinline__ int64_t task_start(const LeafArgs &a, int lane, int64_t s) {
+    const int64_t k0 = s * a.seg;
+    if (k0 >= a.ninj) return a.ninj;
+    if (s == 0 || a.gap == 0) return k0;
+    const int64_t end = min(k0 + TASK_REACH, a.ninj);
+    for (int64_t k = k0; k < end; k += 32) {
+        const int64_t x = k + lane;
+        bool cut = false;
+        if (x < end) {
+            const uint64_t y = a.keys[x], z = a.keys[x - 1];
+            cut = (y >> 32) != (z >> 32) || (uint32_t)y - (uint32_t)z > a.gap;
+        }
+        const unsigned b = __ballot_sync(FULL, cut);
+        if (b) return k + __ffs(b) - 1;
+    }
+    return end == a.ninj ? a.ninj : k0;
+}
+
 #ifndef AE_LEAF_E
 #define AE_LEAF_E 2
 #endif
@@ -663,8 +689,9 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
         s = __shfl_sync(FULL, s, 0);
         if (s >= (unsigned long long)a.nseg) break;
         if (*(volatile unsigned long long *)&a.stats->leaf_overflow) break;
-        int64_t k = (int64_t)s * a.seg;
-        const int64_t kend = min(k + (int64_t)a.seg, a.ninj);
+        int64_t k = task_start(a, lane, (int64_t)s);
+        const int64_t kend = task_start(a, lane, (int64_t)s + 1);
+        if (k >= kend) continue;
         int64_t rlen = 0;
         int32_t p = -1, qid = -1, m = 0, H = 0;
         const uint8_t *P = nullptr;
@@ -1089,15 +1116,28 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
             if (a.esc_min > 0 && rlen > a.esc_min) {
                 // a wide row goes on on a whole block (k_leaf_wide), with the rest of
                 // this task's injections; the warp takes its next task
-                unsigned long long slot = 0;
-                if (lane == 0) slot = atomicAdd(a.esc_count, 1ull);
+                unsigned long long slot = 0, at = 0;
+                if (lane == 0) {
+                    // (a walk that finds no room leaves the counters past their ends; they are
+                    // read first so that they cannot wrap)
+                    slot = *(volatile unsigned long long *)a.esc_count;
+                    at = *(volatile unsigned long long *)(a.esc_count + 1);
+                    if (slot < (unsigned long long)a.esc_max && at + rlen <= (unsigned long long)a.esc_pool_cap) {
+                        at = atomicAdd(a.esc_count + 1, (unsigned long long)rlen);
+                        slot = at + rlen <= (unsigned long long)a.esc_pool_cap ? atomicAdd(a.esc_count, 1ull)
+                                                                               : (unsigned long long)a.esc_max;
+                    } else {
+                        slot = (unsigned long long)a.esc_max;
+                    }
+                }
                 slot = __shfl_sync(FULL, slot, 0);
+                at = __shfl_sync(FULL, at, 0);
                 if (slot < (unsigned long long)a.esc_max) {
-                    int32_t *eb = a.esc_rows + (int64_t)slot * 12 * cap;
                     for (int64_t i = lane; i < rlen; i += 32) {
-                        eb[i] = R.j[i];
-                        eb[cap + i] = R.M[i];
-                        eb[2 * cap + i] = R.Ga[i];
+                        int32_t *x = a.esc_pool + 3 * ((int64_t)at + i);
+                        x[0] = R.j[i];
+                        x[1] = R.M[i];
+                        x[2] = R.Ga[i];
                     }
                     if (lane == 0) {
                         EscWalk e;
@@ -1106,6 +1146,7 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
                         e.rlen = rlen;
                         e.k = k;
                         e.kend = kend;
+                        e.row = (int64_t)at;
                         a.esc[slot] = e;
                     }
                     __syncwarp();
@@ -1153,264 +1194,545 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
 // ------------------------------------------------------------------ wide sweep walks
 //
 // A walk whose row has grown wide is continued by a whole block: each step's
-// entries are spread over LEAF_WIDE_THREADS threads (LEAF_E consecutive
-// entries each), the horizontal-gap keys and the output counts are block-wide
-// scans, and the merges of injected rows run on the first warp.  The values
-// are those of the warp walk of k_leaf (the same make_slots / slot_finish per
-// entry, the same merge); only the time per step differs.
-constexpr int LEAF_WIDE_THREADS = 512;
-constexpr int LEAF_WIDE_WARPS = LEAF_WIDE_THREADS / 32;
-constexpr int LEAF_WIDE_HS = 128;   // hit records staged per warp of the block
+// entries are spread over the block's threads (WIDE_E consecutive entries
+// each), the horizontal-gap keys and the output counts are block-wide scans.
+// The values are those of the warp walk of k_leaf (the same make_slots /
+// slot_finish per entry, the same merge); only the time per step differs.
+//
+// A walk is a chain of steps, one per text position, and a search waits for
+// its longest one (thousands of positions along a homolog), so a step is built
+// for latency: the two rows live in shared memory, a row of up to 512 entries
+// is stepped one entry per thread, hits collect in a block-wide stage, and the
+// next injections wait with their rows in a ring.  The rows injected at a
+// position are looked up in the walked row by a warp each; those it dominates
+// (nearly all along a homolog) are done with that, the others are merged by
+// the whole block.  A row too long for shared memory moves to the block's
+// buffers in global memory and back.  About 7,500 cycles a step at rows of 1,300
+// entries, 4,500 at 200, where the warp walk takes 40,000 at 1,300 (in
+// instructions: the slots and the finish, three scans, the look-up); more
+// threads or more entries per thread spill registers and are slower.
+#ifndef AE_WIDE_T
+#define AE_WIDE_T 512
+#endif
+constexpr int WIDE_T = AE_WIDE_T;     // threads
+constexpr int WIDE_W = WIDE_T / 32;
+constexpr int WIDE_E = 2;             // consecutive entries per thread at most
+constexpr int WIDE_ROW = 6144;        // entries of a row in shared memory
+constexpr int WIDE_HITS = 4096;       // staged hits
+constexpr int WIDE_RING = 32;         // injections looked up ahead
+constexpr int WIDE_RE = 8;            // entries of their rows held in the ring
+constexpr int WIDE_HS = 64;           // hits staged by the merging warp
 
-__device__ __forceinline__ int32_t block_excl_max(int32_t v, int32_t *sw, int32_t &total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int32_t incl = warp_incl_max(v);
-    if (lane == 31) sw[w] = incl;
-    __syncthreads();
-    int32_t pre = AE_KNEG, all = AE_KNEG;
-#pragma unroll
-    for (int x = 0; x < LEAF_WIDE_WARPS; ++x) {
-        const int32_t y = sw[x];
-        if (x < w) pre = max(pre, y);
-        all = max(all, y);
-    }
-    int32_t ex = __shfl_up_sync(FULL, incl, 1);
-    if (lane == 0) ex = AE_KNEG;
-    total = all;
-    __syncthreads();
-    return max(pre, ex);
-}
-
-__device__ __forceinline__ uint32_t block_excl_sum(uint32_t v, uint32_t *sw, uint32_t &total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t incl = warp_incl_sum(v);
-    if (lane == 31) sw[w] = incl;
-    __syncthreads();
-    uint32_t pre = 0, all = 0;
-#pragma unroll
-    for (int x = 0; x < LEAF_WIDE_WARPS; ++x) {
-        const uint32_t y = sw[x];
-        if (x < w) pre += y;
-        all += y;
-    }
-    total = all;
-    __syncthreads();
-    return pre + incl - v;
-}
-
-struct WideState {
-    int64_t rlen, k;
-    int32_t p, qid, m, H;
-    int32_t buf[4];   // the slot's buffers serving as R, Rn, Cb, C2
-    int32_t overflow;
+struct __align__(16) WideSmem {
+    int32_t j[2][WIDE_ROW], M[2][WIDE_ROW], G[2][WIDE_ROW];
+    int32_t hp[WIDE_HITS], hj[WIDE_HITS], hs[WIDE_HITS];   // hits: text position, column, score
+    uint64_t mkey[WIDE_HS];
+    int32_t mscore[WIDE_HS];
+    __align__(16) int32_t smax[2][WIDE_W];
+    __align__(16) uint32_t scnt[2][WIDE_W];
+    __align__(16) uint32_t shit[2][WIDE_W];
+    uint64_t roff[WIDE_RING];
+    uint32_t rcnt[WIDE_RING];
+    int32_t rqid[WIDE_RING], rpos[WIDE_RING];
+    int32_t rj[WIDE_RING][WIDE_RE], rM[WIDE_RING][WIDE_RE], rG[WIDE_RING][WIDE_RE];
+    int32_t dom[WIDE_RING];              // the walked row dominates the injected one
+    int32_t mq[32], mM[32], mG[32];      // a merge: place in the row (new entries: ~place), values
+    unsigned long long walk, hbase;
+    int64_t nlen;
+    int32_t swapped, overflow;
+    int8_t mat[AE_MAX_SIGMA * AE_MAX_SIGMA];
 };
 
-__global__ void __launch_bounds__(LEAF_WIDE_THREADS) k_leaf_wide(LeafArgs a) {
-    __shared__ int8_t smat[AE_MAX_SIGMA * AE_MAX_SIGMA];
-    __shared__ uint64_t s_hkey[LEAF_WIDE_WARPS][LEAF_WIDE_HS];
-    __shared__ int32_t s_hscore[LEAF_WIDE_WARPS][LEAF_WIDE_HS];
-    __shared__ uint32_t s_scan[LEAF_WIDE_WARPS];
-    __shared__ WideState ws;
-    load_matrix(a.sc, smat);
-    const unsigned long long nesc = min(*(volatile unsigned long long *)a.esc_count, (unsigned long long)a.esc_max);
-    if ((unsigned long long)blockIdx.x >= nesc) return;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    HitStage hstage = {s_hkey[wid], s_hscore[wid], 0u, (uint32_t)LEAF_WIDE_HS};
-    const ScoreView &sc = a.sc;
-    const int32_t u = -sc.ss, oe = sc.sg + sc.ss, g = sc.gmax;
-    const int64_t cap = a.cap;
-    const uint64_t jmask = (1ull << a.bj) - 1ull;
-    int32_t *eb = a.esc_rows + (int64_t)blockIdx.x * 12 * cap;
-    Buf B[4];
-#pragma unroll
-    for (int x = 0; x < 4; ++x) B[x] = Buf{eb + 3 * x * cap, eb + (3 * x + 1) * cap, eb + (3 * x + 2) * cap};
-    const EscWalk e0 = a.esc[blockIdx.x];
-    const int64_t kend = e0.kend;
-    if (threadIdx.x == 0) {
-        ws.rlen = e0.rlen;
-        ws.k = e0.k;
-        ws.p = e0.p;
-        ws.qid = e0.qid;
-        ws.m = a.qv.m[e0.qid];
-        ws.H = a.qv.H[e0.qid];
-        for (int x = 0; x < 4; ++x) ws.buf[x] = x;
-        ws.overflow = 0;
+// Over the values of the block's warps in sw: of those before warp w, and of all
+__device__ __forceinline__ void wide_max(const int32_t *sw, int w, int32_t &pre, int32_t &all) {
+    const int lane = threadIdx.x & 31;
+    const int32_t v = lane < WIDE_W ? sw[lane] : AE_KNEG;
+    pre = __reduce_max_sync(FULL, lane < w ? v : AE_KNEG);
+    all = __reduce_max_sync(FULL, v);
+}
+__device__ __forceinline__ void wide_sum(const uint32_t *sw, int w, uint32_t &pre, uint32_t &all) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t v = lane < WIDE_W ? sw[lane] : 0u;
+    pre = __reduce_add_sync(FULL, lane < w ? v : 0u);
+    all = __reduce_add_sync(FULL, v);
+}
+
+// The staged hits go out (all threads; hn is block-uniform)
+__device__ __forceinline__ void wide_flush(const LeafArgs &a, WideSmem &s, int32_t qid, uint32_t &hn) {
+    if (!hn) return;
+    __syncthreads();
+    if (threadIdx.x == 0) s.hbase = atomicAdd(a.hit_count, (unsigned long long)hn);
+    __syncthreads();
+    const uint64_t b = s.hbase;
+    if (b + hn <= a.hit_cap) {
+        const uint64_t kq = (uint64_t)qid << (a.be + a.bj);
+        for (uint32_t i = threadIdx.x; i < hn; i += WIDE_T) {
+            a.hit_key[b + i] = kq | ((uint64_t)(uint32_t)s.hp[i] << a.bj) | (uint64_t)(uint32_t)s.hj[i];
+            a.hit_score[b + i] = s.hs[i];
+        }
+    } else if (threadIdx.x == 0) {
+        atomicAdd(&a.stats->hit_overflow, 1ull);
     }
     __syncthreads();
-    unsigned long long st_rows = 0, st_ent = 0, st_reused = 0, st_t0 = 0, steps = 0, width = 0;
+    hn = 0;
+}
+
+__device__ __forceinline__ void wide_copy(const Buf &d, const Buf &r, int64_t n) {
+    for (int64_t i = threadIdx.x; i < n; i += WIDE_T) {
+        d.j[i] = r.j[i];
+        d.M[i] = r.M[i];
+        d.Ga[i] = r.Ga[i];
+    }
+}
+
+__global__ void __launch_bounds__(WIDE_T, 1) k_leaf_wide(LeafArgs a) {
+    extern __shared__ __align__(16) unsigned char wide_smem[];
+    WideSmem &s = *reinterpret_cast<WideSmem *>(wide_smem);
+    load_matrix(a.sc, s.mat);
+    const unsigned long long nesc = min(*(volatile unsigned long long *)a.esc_count, (unsigned long long)a.esc_max);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    HitStage mstage = {s.mkey, s.mscore, 0u, (uint32_t)WIDE_HS};   // of the merging warp
+    const ScoreView &sc = a.sc;
+    const int32_t u = -sc.ss, oe = sc.sg + sc.ss, g = sc.gmax;
+    const uint64_t jmask = (1ull << a.bj) - 1ull;
+    int32_t *eb = a.wide_rows + (int64_t)blockIdx.x * 12 * a.wide_cap;
+    // buffers 0 and 1: the rows in shared memory; 2 to 5: in global memory
+    auto buf = [&](int x) {
+        if (x < 2) return Buf{s.j[x], s.M[x], s.G[x]};
+        int32_t *b = eb + (int64_t)(x - 2) * 3 * a.wide_cap;
+        return Buf{b, b + a.wide_cap, b + 2 * (int64_t)a.wide_cap};
+    };
+    unsigned long long st_rows = 0, st_ent = 0, st_reused = 0, st_t0 = 0, width = 0;
     const long long t_start = clock64();
-    while (true) {
-        const int64_t rlen = ws.rlen;
-        int64_t k = ws.k;
-        int32_t p = ws.p, qid = ws.qid, m = ws.m, H = ws.H;
-        const int ib[4] = {ws.buf[0], ws.buf[1], ws.buf[2], ws.buf[3]};
-        __syncthreads();   // every thread has the state before thread 0 changes it
-        Buf R = B[ib[0]], Rn = B[ib[1]], Cb = B[ib[2]], C2 = B[ib[3]];
-        int64_t nlen = 0;
-        if (rlen == 0) {
-            if (k >= kend) break;
-            // a new walk: the row at p is the union of the rows injected there
-            const Inject I0 = a.inj[a.order[k]];
-            p = I0.e;
-            qid = I0.qid;
-            m = a.qv.m[qid];
-            H = a.qv.H[qid];
-        } else {
-            if (p + 1 >= a.ix.n || seq_end(a.ix, p)) {   // the walk ends with the text or its sequence
-                if (threadIdx.x == 0) ws.rlen = 0;
-                __syncthreads();
-                continue;
-            }
-            ++p;
-            const int c = (int)a.ix.text[p];
-            const uint8_t *P = a.qv.codes + a.qv.off[qid];
-            int32_t carry = AE_KNEG;
-            bool ovf = false;
-            for (int64_t base = 0; base < rlen; base += (int64_t)LEAF_WIDE_THREADS * LEAF_E) {
-                const int64_t i0 = base + (int64_t)threadIdx.x * LEAF_E;
-                int32_t jj[LEAF_E], MM[LEAF_E], GG[LEAF_E];
-#pragma unroll
-                for (int e = 0; e < LEAF_E; ++e) {
-                    const bool v = i0 + e < rlen;
-                    jj[e] = v ? R.j[i0 + e] : m;
-                    MM[e] = v ? R.M[i0 + e] : AE_NEG;
-                    GG[e] = v ? R.Ga[i0 + e] : AE_NEG;
-                }
-                // the entries around this thread's: the next one's column, the previous one
-                const int32_t jnext = i0 + LEAF_E < rlen ? R.j[i0 + LEAF_E] : m;
-                int32_t pj0 = -2, pM0 = AE_NEG;
-                if (i0 > 0 && i0 - 1 < rlen) {
-                    pj0 = R.j[i0 - 1];
-                    pM0 = R.M[i0 - 1];
-                }
-                Slots sl[LEAF_E];
-                int32_t lk[LEAF_E];
-#pragma unroll
-                for (int e = 0; e < LEAF_E; ++e) {
-                    const bool v = i0 + e < rlen;
-                    int32_t jn = (e + 1 < LEAF_E) ? jj[e + 1] : jnext;
-                    if (i0 + e + 1 >= rlen) jn = m;
-                    const int32_t pj = e ? jj[e - 1] : pj0, pM = e ? MM[e - 1] : pM0;
-                    make_slots(sc, smat, c, P, m, H, g, oe, v, jj[e], MM[e], GG[e], pj, pM, jn, sl[e]);
-                    const int32_t keyA = sl[e].MpA > AE_NEG ? sl[e].MpA + sl[e].colA * u : AE_KNEG;
-                    const int32_t keyB = sl[e].MpB > AE_NEG ? sl[e].MpB + (sl[e].colA + 1) * u : AE_KNEG;
-                    lk[e] = max(e ? lk[e - 1] : AE_KNEG, max(keyA, keyB));
-                }
-                int32_t kall;
-                int32_t lexcl = block_excl_max(lk[LEAF_E - 1], (int32_t *)s_scan, kall);
-                lexcl = max(lexcl, carry);
-                carry = max(carry, kall);
-                SlotOut o[LEAF_E];
-                uint32_t cl = 0, hl = 0;
-                int32_t ik[LEAF_E];
-#pragma unroll
-                for (int e = 0; e < LEAF_E; ++e) {
-                    const int32_t ex = e ? max(lexcl, lk[e - 1]) : lexcl;
-                    ik[e] = max(lexcl, lk[e]);
-                    slot_finish(sl[e].colA, sl[e].MpA, sl[e].hasB, sl[e].MpB, sl[e].next_col, ex, ik[e], sc, m, H, u,
-                                i0 + e < rlen, o[e]);
-                    cl += (uint32_t)o[e].aliveA + (uint32_t)o[e].aliveB + (uint32_t)o[e].run_len;
-                    hl += (uint32_t)(o[e].aliveA && o[e].MA >= H) + (uint32_t)(o[e].aliveB && o[e].MB >= H) +
-                          (uint32_t)o[e].run_hits;
-                }
-                uint32_t ctot;
-                const uint32_t cex = block_excl_sum(cl, s_scan, ctot);
-                if (nlen + (int64_t)ctot > cap) {   // block-uniform
-                    ovf = true;
-                    break;
-                }
-                // hits: each warp reserves its own in its stage
-                const uint32_t hi = warp_incl_sum(hl);
-                const uint32_t htot = __shfl_sync(FULL, hi, 31);
-                bool staged = true, hok = true;
-                uint64_t hbase = 0;
-                if (htot) hbase = stage_reserve(hstage, a, lane, htot, staged, hok);
-                const uint64_t kq = ((uint64_t)qid << (a.be + a.bj)) | ((uint64_t)(uint32_t)p << a.bj);
-                int64_t eo = nlen + (int64_t)cex;
-                uint64_t ho = hbase + hi - hl;
-#pragma unroll
-                for (int e = 0; e < LEAF_E; ++e) {
-                    const int32_t colA = sl[e].colA;
-                    const bool hA = o[e].aliveA && o[e].MA >= H, hB = o[e].aliveB && o[e].MB >= H;
-                    if (o[e].aliveA) {
-                        Rn.j[eo] = colA;
-                        Rn.M[eo] = o[e].MA;
-                        Rn.Ga[eo] = sl[e].GaA;
-                        ++eo;
-                        if (hA && hok) hit_put(hstage, a, staged, ho, kq | ((uint64_t)colA & jmask), o[e].MA);
-                        ho += hA;
-                    }
-                    if (o[e].aliveB) {
-                        Rn.j[eo] = colA + 1;
-                        Rn.M[eo] = o[e].MB;
-                        Rn.Ga[eo] = AE_NEG;
-                        ++eo;
-                        if (hB && hok) hit_put(hstage, a, staged, ho, kq | ((uint64_t)(colA + 1) & jmask), o[e].MB);
-                        ho += hB;
-                    }
-                    for (int32_t r = 0; r < o[e].run_len; ++r) {
-                        const int32_t cc = o[e].run_start + r;
-                        const int32_t v = sc.sg - cc * u + ik[e];
-                        Rn.j[eo] = cc;
-                        Rn.M[eo] = v;
-                        Rn.Ga[eo] = AE_NEG;
-                        ++eo;
-                        if (r < o[e].run_hits) {
-                            if (hok) hit_put(hstage, a, staged, ho, kq | ((uint64_t)cc & jmask), v);
-                            ++ho;
-                        }
-                    }
-                }
-                nlen += (int64_t)ctot;
-            }
-            if (ovf) {
-                if (threadIdx.x == 0) ws.overflow = 1;
-                __syncthreads();
-                break;
-            }
-            st_ent += (unsigned long long)nlen;
-            __syncthreads();   // the step's row is complete before the merge reads it
-        }
-        // ---- the rows injected at (qid, p), merged by the first warp
-        if (wid == 0) {
-            bool ovf = false;
-            leaf_merge(a, lane, qid, p, H, jmask, k, kend, Rn, Cb, C2, nlen, cap, ovf, hstage, st_ent, st_reused,
-                       st_t0);
-            if (lane == 0) {
-                int nr = ib[1], nc = ib[2];   // the merge may have exchanged Rn and Cb
-                if (Rn.j != B[ib[1]].j) {
-                    nr = ib[2];
-                    nc = ib[1];
-                }
-                ws.buf[0] = nr;   // the finished row at p
-                ws.buf[1] = ib[0];
-                ws.buf[2] = nc;
-                ws.buf[3] = ib[3];
-                ws.rlen = nlen;
-                ws.k = k;
-                ws.p = p;
-                ws.qid = qid;
-                ws.m = m;
-                ws.H = H;
-                if (ovf) ws.overflow = 1;
-            }
+    bool stop = false;
+    while (!stop) {
+        // ---- the next walk handed on
+        if (threadIdx.x == 0) {
+            s.walk = *(volatile unsigned long long *)&a.stats->wide_overflow ? nesc : atomicAdd(a.esc_count + 2, 1ull);
+            s.overflow = 0;
         }
         __syncthreads();
-        if (ws.overflow) break;
-        ++st_rows;
-        ++steps;
-        width = max(width, (unsigned long long)ws.rlen);
+        if (s.walk >= nesc) break;
+        const EscWalk e0 = a.esc[s.walk];
+        const int64_t kend = e0.kend;
+        int64_t k = e0.k, rlen = e0.rlen, ring = k;   // ring: first injection the ring holds
+        int32_t p = e0.p;
+        int32_t qid = e0.qid, m = a.qv.m[qid], H = a.qv.H[qid];
+        const uint8_t *P = a.qv.codes + a.qv.off[qid];
+        int cur = 0;                 // the row's buffer
+        uint32_t hn = 0;             // staged hits
+        if (rlen > WIDE_ROW) cur = 2;
+        if (rlen > (cur ? (int64_t)a.wide_cap : (int64_t)WIDE_ROW)) {
+            stop = true;
+            break;
+        }
+        {
+            const Buf B = buf(cur);
+            for (int64_t i = threadIdx.x; i < rlen; i += WIDE_T) {
+                const int32_t *x = a.esc_pool + 3 * (e0.row + i);
+                B.j[i] = x[0];
+                B.M[i] = x[1];
+                B.Ga[i] = x[2];
+            }
+        }
+        auto fill_ring = [&]() {     // injections [ring, ring + WIDE_RING)
+            if (threadIdx.x < WIDE_RING) {
+                const int64_t x = ring + threadIdx.x;
+                s.rqid[threadIdx.x] = -1;
+                if (x < kend) {
+                    const Inject I = a.inj[a.order[x]];
+                    s.rqid[threadIdx.x] = I.qid;
+                    s.rpos[threadIdx.x] = I.e;
+                    s.rcnt[threadIdx.x] = I.cnt;
+                    s.roff[threadIdx.x] = I.off;
+                }
+            }
+            __syncthreads();
+            if (threadIdx.x < WIDE_RING * WIDE_RE) {
+                const int r = threadIdx.x / WIDE_RE, x = threadIdx.x % WIDE_RE;
+                if (s.rqid[r] >= 0 && (uint32_t)x < s.rcnt[r]) {
+                    const uint64_t o = s.roff[r] + x;
+                    s.rj[r][x] = a.lj[o];
+                    s.rM[r][x] = a.lM[o];
+                    s.rG[r][x] = a.lGa[o];
+                }
+            }
+            __syncthreads();
+        };
+        // entry x of ring row r
+        auto inj_entry = [&](int r, uint32_t x, int32_t &y, int32_t &M, int32_t &G) {
+            if (x < WIDE_RE) {
+                y = s.rj[r][x];
+                M = s.rM[r][x];
+                G = s.rG[r][x];
+            } else {
+                const uint64_t o = s.roff[r] + x;
+                y = a.lj[o];
+                M = a.lM[o];
+                G = a.lGa[o];
+            }
+        };
+        fill_ring();
+        unsigned long long steps = 0;
+        int ph = 0;                  // the scans' buffers alternate
+        int c_next = p + 1 < a.ix.n ? (int)a.ix.text[p + 1] : 0;
+        bool again = false;          // a step repeated in global memory
+        while (true) {
+            int64_t nlen = 0;
+            int nxt = cur ^ 1;
+            if (rlen == 0) {
+                // a new walk: the row at p is the union of the rows injected there
+                if (k >= kend) break;
+                if (k >= ring + WIDE_RING) {
+                    __syncthreads();
+                    ring = k;
+                    fill_ring();
+                }
+                p = s.rpos[k - ring];
+                if (s.rqid[k - ring] != qid) {
+                    wide_flush(a, s, qid, hn);   // staged hits are of one query
+                    qid = s.rqid[k - ring];
+                    m = a.qv.m[qid];
+                    H = a.qv.H[qid];
+                    P = a.qv.codes + a.qv.off[qid];
+                }
+                nxt = 0;
+                c_next = p + 1 < a.ix.n ? (int)a.ix.text[p + 1] : 0;
+            } else {
+                if (!again) {
+                    if (p + 1 >= a.ix.n || seq_end(a.ix, p)) {   // the walk ends with the text or its sequence
+                        rlen = 0;
+                        continue;
+                    }
+                    ++p;
+                }
+                again = false;
+                const int c = c_next;
+                const int c_after = p + 1 < a.ix.n ? (int)a.ix.text[p + 1] : 0;   // used one step on
+                const Buf R = buf(cur), Rn = buf(nxt);
+                const int64_t cap = cur < 2 ? (int64_t)WIDE_ROW : (int64_t)a.wide_cap;
+                int32_t carry = AE_KNEG;
+                bool full = false;
+                // one chunk of the row: T * E entries from `base` on
+                auto chunk = [&](int64_t base, auto ec) {
+                    constexpr int E = decltype(ec)::value;
+                    const int64_t i0 = base + (int64_t)threadIdx.x * E;
+                    int32_t jj[E], MM[E], GG[E];
+                    int32_t jnext = m, pj0 = -2, pM0 = AE_NEG;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        jj[e] = m;
+                        MM[e] = GG[e] = AE_NEG;
+                    }
+                    if (i0 < rlen) {
+#pragma unroll
+                        for (int e = 0; e < E; ++e)
+                            if (i0 + e < rlen) {
+                                jj[e] = R.j[i0 + e];
+                                MM[e] = R.M[i0 + e];
+                                GG[e] = R.Ga[i0 + e];
+                            }
+                        if (i0 + E < rlen) jnext = R.j[i0 + E];
+                        if (i0 > 0) {
+                            pj0 = R.j[i0 - 1];
+                            pM0 = R.M[i0 - 1];
+                        }
+                    }
+                    // warps past the row only take part in the scans
+                    const bool active = base + (int64_t)wid * 32 * E < rlen;
+                    Slots sl[E];
+                    int32_t lk[E];
+#pragma unroll
+                    for (int e = 0; e < E; ++e) lk[e] = AE_KNEG;
+                    if (active)
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const int32_t jn = (e + 1 < E) ? jj[e + 1] : jnext;
+                        const int32_t pj = e ? jj[e - 1] : pj0, pM = e ? MM[e - 1] : pM0;
+                        make_slots(sc, s.mat, c, P, m, H, g, oe, i0 + e < rlen, jj[e], MM[e], GG[e], pj, pM, jn, sl[e]);
+                        const int32_t keyA = sl[e].MpA > AE_NEG ? sl[e].MpA + sl[e].colA * u : AE_KNEG;
+                        const int32_t keyB = sl[e].MpB > AE_NEG ? sl[e].MpB + (sl[e].colA + 1) * u : AE_KNEG;
+                        lk[e] = max(e ? lk[e - 1] : AE_KNEG, max(keyA, keyB));
+                    }
+                    const int32_t kincl = active ? warp_incl_max(lk[E - 1]) : AE_KNEG;
+                    if (lane == 31) s.smax[ph][wid] = kincl;
+                    int32_t lexcl = __shfl_up_sync(FULL, kincl, 1);
+                    if (lane == 0) lexcl = AE_KNEG;
+                    __syncthreads();
+                    {
+                        int32_t pre, all;
+                        wide_max(s.smax[ph], wid, pre, all);
+                        lexcl = max(max(lexcl, pre), carry);
+                        carry = max(carry, all);
+                    }
+                    SlotOut o[E];
+                    uint32_t cl = 0, hl = 0;
+                    int32_t ik[E];
+                    if (active)
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const int32_t ex = e ? max(lexcl, lk[e - 1]) : lexcl;
+                        ik[e] = max(lexcl, lk[e]);
+                        slot_finish(sl[e].colA, sl[e].MpA, sl[e].hasB, sl[e].MpB, sl[e].next_col, ex, ik[e], sc, m, H, u,
+                                    i0 + e < rlen, o[e]);
+                        cl += (uint32_t)o[e].aliveA + (uint32_t)o[e].aliveB + (uint32_t)o[e].run_len;
+                        hl += (uint32_t)(o[e].aliveA && o[e].MA >= H) + (uint32_t)(o[e].aliveB && o[e].MB >= H) +
+                              (uint32_t)o[e].run_hits;
+                    }
+                    uint32_t ci = 0, hi = 0;
+                    if (active) {
+                        ci = warp_incl_sum(cl);
+                        hi = warp_incl_sum(hl);
+                    }
+                    if (lane == 31) {
+                        s.scnt[ph][wid] = ci;
+                        s.shit[ph][wid] = hi;
+                    }
+                    __syncthreads();
+                    uint32_t cpre, ctot, hpre, htot;
+                    wide_sum(s.scnt[ph], wid, cpre, ctot);
+                    wide_sum(s.shit[ph], wid, hpre, htot);
+                    ph ^= 1;
+                    if (nlen + (int64_t)ctot > cap) {   // block-uniform
+                        full = true;
+                        return;
+                    }
+                    // hits: to the stage, or straight out where one chunk has more than it holds
+                    if (hn + htot > WIDE_HITS) wide_flush(a, s, qid, hn);
+                    const bool direct = htot > WIDE_HITS;
+                    uint64_t ho = hn + hpre + hi - hl;
+                    bool hok = true;
+                    if (direct) {
+                        if (threadIdx.x == 0) s.hbase = atomicAdd(a.hit_count, (unsigned long long)htot);
+                        __syncthreads();
+                        ho += s.hbase;
+                        hok = s.hbase + htot <= a.hit_cap;
+                        if (!hok && threadIdx.x == 0) atomicAdd(&a.stats->hit_overflow, 1ull);
+                        __syncthreads();
+                    } else {
+                        hn += htot;
+                    }
+                    const uint64_t kq = ((uint64_t)qid << (a.be + a.bj)) | ((uint64_t)(uint32_t)p << a.bj);
+                    auto put = [&](int32_t col, int32_t v) {
+                        if (!direct) {
+                            s.hp[ho] = p;
+                            s.hj[ho] = col;
+                            s.hs[ho] = v;
+                        } else if (hok) {
+                            a.hit_key[ho] = kq | ((uint64_t)col & jmask);
+                            a.hit_score[ho] = v;
+                        }
+                        ++ho;
+                    };
+                    int64_t eo = nlen + (int64_t)(cpre + ci - cl);
+                    if (active)
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const int32_t colA = sl[e].colA;
+                        if (o[e].aliveA) {
+                            Rn.j[eo] = colA;
+                            Rn.M[eo] = o[e].MA;
+                            Rn.Ga[eo] = sl[e].GaA;
+                            ++eo;
+                            if (o[e].MA >= H) put(colA, o[e].MA);
+                        }
+                        if (o[e].aliveB) {
+                            Rn.j[eo] = colA + 1;
+                            Rn.M[eo] = o[e].MB;
+                            Rn.Ga[eo] = AE_NEG;
+                            ++eo;
+                            if (o[e].MB >= H) put(colA + 1, o[e].MB);
+                        }
+                        for (int32_t r = 0; r < o[e].run_len; ++r) {
+                            const int32_t cc = o[e].run_start + r;
+                            const int32_t v = sc.sg - cc * u + ik[e];
+                            Rn.j[eo] = cc;
+                            Rn.M[eo] = v;
+                            Rn.Ga[eo] = AE_NEG;
+                            ++eo;
+                            if (r < o[e].run_hits) put(cc, v);
+                        }
+                    }
+                    nlen += (int64_t)ctot;
+                };
+                if (rlen <= WIDE_T) {
+                    chunk(0, std::integral_constant<int, 1>());
+                } else {
+                    for (int64_t base = 0; base < rlen && !full; base += WIDE_T * WIDE_E)
+                        chunk(base, std::integral_constant<int, WIDE_E>());
+                }
+                if (full) {
+                    // past shared memory: the step is done again in global memory (hits it
+                    // staged already are reported twice, which the per-cell maximum removes);
+                    // past the block's buffers there: reported, the host runs the sweep again
+                    if (cur >= 2 || rlen > a.wide_cap) {
+                        stop = true;
+                        break;
+                    }
+                    __syncthreads();
+                    wide_copy(buf(2), buf(cur), rlen);
+                    cur = 2;
+                    again = true;
+                    __syncthreads();
+                    continue;
+                }
+                c_next = c_after;
+                if (threadIdx.x == 0) st_ent += (unsigned long long)nlen;
+                __syncthreads();   // the step's row is complete
+            }
+            // ---- the rows injected at (qid, p): those of the ring at once
+            while (k < kend && !stop) {
+                if (k >= ring + WIDE_RING) {
+                    __syncthreads();
+                    ring = k;
+                    fill_ring();
+                }
+                const int r0 = (int)(k - ring);
+                const bool here = r0 + lane < WIDE_RING && s.rqid[r0 + lane] == qid && s.rpos[r0 + lane] == p;
+                const int nin = __ffs(~__ballot_sync(FULL, here)) - 1 < 0 ? 32 : __ffs(~__ballot_sync(FULL, here)) - 1;
+                if (nin == 0) break;
+                // an injected row whose every entry the walked row already has with M and G_a
+                // at least as large changes nothing
+                {
+                    const Buf Rn = buf(nxt);
+                    for (int r = r0 + wid; r < r0 + nin; r += WIDE_W) {
+                        bool ok = nlen > 0;
+                        for (uint32_t x = lane; x < s.rcnt[r] && ok; x += 32) {
+                            int32_t y, M, G;
+                            inj_entry(r, x, y, M, G);
+                            // along a homolog the row's columns are consecutive: look there first
+                            int64_t q = (int64_t)y - Rn.j[0];
+                            if (q < 0 || q >= nlen || Rn.j[q] != y) q = lower_bound_g(Rn.j, nlen, y);
+                            ok = q < nlen && Rn.j[q] == y && Rn.M[q] >= M && Rn.Ga[q] >= G;
+                        }
+                        ok = __all_sync(FULL, ok);
+                        if (lane == 0) s.dom[r] = ok;
+                    }
+                }
+                __syncthreads();
+                for (int r = r0; r < r0 + nin && !stop; ++r, ++k) {
+                    const uint32_t icnt = s.rcnt[r];
+                    if (s.dom[r]) {
+                        if (threadIdx.x == 0) st_reused += icnt;
+                        continue;
+                    }
+                    if (icnt <= 32 && nxt < 2 && nlen + (int64_t)icnt <= WIDE_ROW) {
+                        // ---- the union by maximum, into the other row buffer
+                        if (hn + 32 > WIDE_HITS) wide_flush(a, s, qid, hn);
+                        const Buf A = buf(nxt), D = buf(nxt ^ 1);
+                        int32_t y = 0, M = AE_NEG, G = AE_NEG;
+                        int64_t q = 0;
+                        bool fresh = false, hit = false;
+                        if ((uint32_t)lane < icnt) {
+                            inj_entry(r, lane, y, M, G);
+                            q = lower_bound_g(A.j, nlen, y);
+                            fresh = !(q < nlen && A.j[q] == y);
+                            hit = M >= H && (fresh || M > A.M[q]);
+                        }
+                        const unsigned bf = __ballot_sync(FULL, fresh), bh = __ballot_sync(FULL, hit);
+                        const unsigned lt = (1u << lane) - 1u;
+                        if (wid == 0) {
+                            if ((uint32_t)lane < icnt) {
+                                s.mq[lane] = fresh ? ~(int32_t)q : (int32_t)q;
+                                s.mM[lane] = M;
+                                s.mG[lane] = G;
+                                if (fresh) {
+                                    const int64_t d = q + __popc(bf & lt);
+                                    D.j[d] = y;
+                                    D.M[d] = M;
+                                    D.Ga[d] = G;
+                                }
+                            }
+                            if (hit) {
+                                const uint32_t h = hn + __popc(bh & lt);
+                                s.hp[h] = p;
+                                s.hj[h] = y;
+                                s.hs[h] = M;
+                            }
+                        }
+                        hn += __popc(bh);
+                        __syncthreads();
+                        for (int64_t x = threadIdx.x; x < nlen; x += WIDE_T) {
+                            int32_t Mx = A.M[x], Gx = A.Ga[x];
+                            int64_t d = x;
+                            for (uint32_t l = 0; l < icnt; ++l) {
+                                const int32_t z = s.mq[l];
+                                if (z < 0) {
+                                    d += ~z <= x ? 1 : 0;   // a new entry goes before this one
+                                } else if (z == x) {
+                                    Mx = max(Mx, s.mM[l]);
+                                    Gx = max(Gx, s.mG[l]);
+                                }
+                            }
+                            D.j[d] = A.j[x];
+                            D.M[d] = Mx;
+                            D.Ga[d] = Gx;
+                        }
+                        nlen += __popc(bf);
+                        if (threadIdx.x == 0) {
+                            st_ent += __popc(bf);
+                            st_reused += icnt - __popc(bf);
+                        }
+                        nxt ^= 1;
+                        __syncthreads();
+                        continue;
+                    }
+                    // long rows: the first warp merges, through the block's buffers in global memory
+                    if (nxt < 2 && nlen <= a.wide_cap) {
+                        wide_copy(buf(2), buf(nxt), nlen);
+                        nxt = 2;
+                        __syncthreads();
+                    }
+                    if (wid == 0) {
+                        Buf A = buf(nxt), Cb = buf(4), C2 = buf(5);
+                        int32_t *const was = A.j;
+                        bool ovf = nxt < 2;   // longer than the buffers: reported
+                        int64_t kk = k, nl = nlen;
+                        if (!ovf)
+                            leaf_merge(a, lane, qid, p, H, jmask, kk, k + 1, A, Cb, C2, nl, (int64_t)a.wide_cap, ovf, mstage,
+                                       st_ent, st_reused, st_t0);
+                        if (lane == 0) {
+                            s.nlen = nl;
+                            s.swapped = A.j != was;
+                            if (ovf) s.overflow = 1;
+                        }
+                    }
+                    __syncthreads();
+                    if (s.overflow) {
+                        stop = true;
+                        break;
+                    }
+                    nlen = s.nlen;
+                    if (s.swapped) wide_copy(buf(nxt), buf(4), nlen);
+                    __syncthreads();
+                }
+                __syncthreads();   // the ring's flags are read before the next group's are written
+            }
+            if (stop) break;
+            cur = nxt;
+            rlen = nlen;
+            if (cur >= 2 && rlen <= WIDE_ROW / 2) {   // back to shared memory
+                wide_copy(buf(0), buf(cur), rlen);
+                cur = 0;
+                __syncthreads();
+            }
+            ++st_rows;
+            ++steps;
+            width = max(width, (unsigned long long)rlen);
+        }
+        wide_flush(a, s, qid, hn);
+        if (threadIdx.x == 0) atomicMax(&a.stats->leaf_max_steps, steps);
+        __syncthreads();
     }
-    stage_flush(hstage, a, lane);
+    if (wid == 0) stage_flush(mstage, a, lane);
     if (threadIdx.x == 0) {
-        if (ws.overflow) atomicAdd(&a.stats->leaf_overflow, 1ull);
+        if (stop) atomicAdd(&a.stats->wide_overflow, 1ull);
         if (st_rows) atomicAdd(&a.stats->leaf_rows, st_rows);
         if (st_ent) {
             atomicAdd(&a.stats->entries, st_ent);
             atomicAdd(&a.stats->entries_leaf, st_ent);
         }
         if (st_reused) atomicAdd(&a.stats->reused, st_reused);
-        atomicMax(&a.stats->leaf_max_steps, steps);
         atomicMax(&a.stats->leaf_max_width, width);
         atomicMax(&a.stats->leaf_max_cycles, (unsigned long long)(clock64() - t_start));
     }
@@ -1610,15 +1932,18 @@ void ae_inject_keys(const Inject *inj, int64_t ninj, uint64_t *keys, uint32_t *v
     k_inject_keys<<<grid_for(ninj, 256), 256, 0, st>>>(inj, ninj, keys, vals);
 }
 
+int ae_leaf_wide_blocks_per_sm() { return 1; }
+
 int64_t ae_leaf_scratch_words(int32_t cap, int32_t nwarps) { return (int64_t)12 * cap * nwarps; }
 
 void ae_leaf_sweep(const LeafArgs &a, int blocks, int threads, cudaStream_t st) {
     if (a.nseg <= 0) return;
     ++g_launches;
     k_leaf<<<blocks, threads, 0, st>>>(a);
-    if (a.esc_min > 0 && a.esc_max > 0) {   // the walks handed on to blocks (a block per slot taken)
+    if (a.esc_min > 0 && a.esc_max > 0) {   // the walks handed on to blocks
         ++g_launches;
-        k_leaf_wide<<<a.esc_max, LEAF_WIDE_THREADS, 0, st>>>(a);
+        cudaFuncSetAttribute(k_leaf_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WideSmem));
+        k_leaf_wide<<<a.wide_blocks, WIDE_T, sizeof(WideSmem), st>>>(a);
     }
 }
 

@@ -241,22 +241,32 @@ struct LeafArgs {
     int32_t tiers;                // 1: count entries by cost tier
     DevStats *stats;
     // walks whose row grows past esc_min entries (0: never) continue on a whole
-    // block (k_leaf_wide) with the rest of their task's injections, in one of
-    // esc_max slots: esc[slot] the walk's state, esc_rows + slot * 12 * cap its
-    // four row buffers; *esc_count counts the slots taken (it may pass esc_max:
-    // a walk that finds no free slot stays on its warp)
+    // block (k_leaf_wide) with the rest of their task's injections: esc[slot] is
+    // the walk's state, its row lies in the pool at esc[slot].row.  esc_count counts
+    // the slots taken, the pool's entries taken and the walks the blocks have
+    // taken; the first two may pass esc_max and esc_pool_cap: a walk that finds no
+    // room stays on its warp.  Each of the wide_blocks blocks has 12 * wide_cap
+    // words of row buffers at wide_rows.
     int32_t esc_min, esc_max;
+    int64_t esc_pool_cap;
     unsigned long long *esc_count;
     struct EscWalk *esc;
-    int32_t *esc_rows;
+    int32_t *esc_pool;
+    int32_t *wide_rows;
+    int32_t wide_cap, wide_blocks;
+    // sorted (query, text end) of the injections; a task starts at the first one past
+    // a multiple of seg that is more than `gap` positions from the one before it
+    const uint64_t *keys;
+    uint32_t gap;
 };
 // A sweep walk handed from a warp to a block: its query, text position, the
-// row at that position (in the slot's first buffer) and its task's remaining
-// injections [k, kend) (indices into the sorted order).
+// row at that position (rlen entries from `row` on in the pool) and its task's
+// remaining injections [k, kend) (indices into the sorted order).
 struct EscWalk {
     int32_t qid, p;
-    int64_t rlen, k, kend;
+    int64_t rlen, k, kend, row;
 };
+int ae_leaf_wide_blocks_per_sm();
 void ae_inject_keys(const Inject *inj, int64_t ninj, uint64_t *keys, uint32_t *vals, cudaStream_t st);
 void ae_leaf_sweep(const LeafArgs &a, int blocks, int threads, cudaStream_t st);
 int64_t ae_leaf_scratch_words(int32_t cap, int32_t nwarps);

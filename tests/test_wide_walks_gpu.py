@@ -1,0 +1,48 @@
+"""Sweep walks continued on a block, where they can go wrong: rows around the
+block's 512 threads and past its shared memory, buffers grown from a small odd
+capacity, several homologs of several queries in one task, injections merged
+into a walked row, and homologs running into the text's or a sequence's end.
+Results must equal those of the warp walks alone."""
+import numpy as np
+import pytest
+
+from workloads import DNA, Scheme, iid_text, mutate
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1208_0274_gb300 import ae  # noqa: E402
+
+P = [0.25] * 4
+
+
+# (homolog lengths, divergence, H, scheme, options)
+@pytest.mark.parametrize("lengths,div,H,scheme,opts", [
+    ((300, 40, 700), 0.08, 30, (1, -3, -5, -2), dict(leaf_wide_rows=20)),
+    ((1_100, 1_000, 1_040), 0.01, 40, (1, -3, -5, -2), dict(leaf_wide_rows=100, leaf_capacity=67)),
+    ((600, 600, 600), 0.04, 60, (1, -3, -2, -2), dict(leaf_wide_rows=33, leaf_segment=500)),
+    ((9_000,), 0.0, 8_000, (1, -3, -5, -2), dict()),
+])
+def test_block_walks_equal_warp_walks(lengths, div, H, scheme, opts):
+    rng = np.random.default_rng(len(lengths) + H)
+    T = iid_text(60_000, DNA, P, rng)
+    qs = []
+    for q in range(2):
+        parts = [iid_text(37, DNA, P, rng)]
+        for k, L in enumerate(lengths):
+            s = T.size - L if k == 0 else int(rng.integers(0, T.size - L))     # the first one ends with the text
+            parts += [mutate(T[s:s + L], DNA, P, div, div / 5, rng), iid_text(50, DNA, P, rng)]
+        qs.append(np.concatenate(parts))
+    cut = int(T.size - lengths[0] // 2)
+    found = 0
+    for idx in (ae.ae_index_build(T, ae.AE_DNA), ae.ae_index_build_collection([T[:cut], T[cut:]], ae.AE_DNA)):
+        want, wc = ae.ae_search(idx, qs, Scheme(*scheme), H, options=ae.make_options(leaf_wide_rows=0))
+        got, gc = ae.ae_search(idx, qs, Scheme(*scheme), H, options=ae.make_options(**opts))
+        assert ae.ae_last_stats()["leaf_wide_walks"] > 0
+        assert np.array_equal(gc, wc) and np.array_equal(got, want)
+        found += want.size
+        idx.close()
+    assert found > 0
