@@ -172,9 +172,10 @@ typedef struct {
     int32_t fork_part;
     int32_t leaf_wide_rows;   /* a walk of the text-position sweep whose row grows past this many
                                  entries continues on a whole thread block (each step spread over
-                                 its threads) instead of one warp; 0: never.  Default 128; values
-                                 from 128 to 1,024 count as 1,024 where rows are injected at most
-                                 text positions.  The results are the same */
+                                 its threads) instead of one warp; 0: never.  The default, 128,
+                                 lets the library choose: 32 where the injected rows leave gaps
+                                 along the text, 1,024 where they lie at most positions.  The
+                                 results are the same */
 } ae_options;
 
 /* Fill *opt with the defaults: qprefix_seed 1, leaf_segment 0, item_columns

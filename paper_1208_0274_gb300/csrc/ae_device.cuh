@@ -179,12 +179,19 @@ struct SlotOut {
     int32_t run_start, run_len, run_hits;
 };
 
+// a / u for a < 2^16 by the reciprocal rec = ceil(2^32 / u): exact, since
+// a * u < 2^32 or the quotient is 0
+__device__ __forceinline__ uint32_t div_small(uint32_t a, uint64_t rec) {
+    return (uint32_t)(((uint64_t)a * rec) >> 32);
+}
+
 // The run of columns [run_start, next_col) after a lane's slots, where only
 // G_b (key K, the inclusive prefix maximum) can be live: its live cells and
 // how many of them reach H.  G_b along the run is v(x) = s_g - x*u + K,
 // decreasing; thr(x) is non-decreasing, so the live cells form a prefix.  Most
-// runs are empty: the first cell is tested before dividing.  All terms fit
-// int32 (the engine checks m * (u + g + 1) < 2^30).
+// runs are empty: the first cell is tested before dividing, and most others
+// start below 2^16 and end where the threshold is 0: their quotients are
+// products.  All terms fit int32 (the engine checks m * (u + g + 1) < 2^30).
 __device__ __forceinline__ void run_of(int32_t run_start, int32_t next_col, int32_t K, const ScoreView &sc,
                                        int32_t m, int32_t H, int32_t u, int32_t &run_len, int32_t &run_hits) {
     run_len = 0;
@@ -193,6 +200,14 @@ __device__ __forceinline__ void run_of(int32_t run_start, int32_t next_col, int3
     const int32_t g = sc.gmax;
     const int32_t v0 = sc.sg - run_start * u + K;
     if (v0 > thr_of(run_start, m, H, g)) {
+        if (v0 < 65536) {
+            const int32_t r = min((int32_t)div_small((uint32_t)(v0 - 1), sc.urec) + 1, next_col - run_start);
+            if (H - 1 - (m - run_start - r) * g <= 0) {
+                run_len = r;
+                if (v0 >= H) run_hits = min(r, (int32_t)div_small((uint32_t)(v0 - H), sc.urec) + 1);
+                return;
+            }
+        }
         const int32_t x1 = floordiv32(sc.sg + K - 1, u);
         const int32_t x2 = floordiv32(sc.sg + K - H + (m - 1) * g, u + g);
         const int32_t xm = min(min(x1, x2), next_col - 1);

@@ -178,7 +178,7 @@ struct Workspace {
     DevBuf stage;
     // output
     DevBuf uniq, uflags, uoff, qcount;
-    DevBuf stats, stats_keep, segs, ctr, seg_cnt, seg_hit, task_first, task_tot, task_off, task_tmp, task_sum, res, res_key;
+    DevBuf stats, stats_keep, segs, ctr, chain, seg_cnt, seg_hit, task_first, task_tot, task_off, task_tmp, task_sum, res, res_key;
     double fr_ratio = 1.2, lf_ratio = 0.6, hit_ratio = 0.5;
     // pinned host staging
     uint64_t *h_tot = nullptr;
@@ -207,7 +207,7 @@ struct Workspace {
                 &aM[1], &aGa[0], &aGa[1], &nodes[0], &nodes[1], &cnt[0], &cnt[1], &cnt[2], &cnt[3],
                 &cnt[4], &off[0], &off[1], &off[2], &off[3], &off[4], &totals, &scan_tmp, &lj, &lM,
                 &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hkey, &hscore, &hcount, &hk1,
-                &hv1, &scratch, &next_seg, &esc, &esc_count, &esc_pool, &wide_rows, &stage, &uniq, &uflags, &uoff, &qcount, &stats, &stats_keep, &segs, &ctr, &seg_cnt, &seg_hit,
+                &hv1, &scratch, &next_seg, &esc, &esc_count, &esc_pool, &wide_rows, &stage, &uniq, &uflags, &uoff, &qcount, &stats, &stats_keep, &segs, &ctr, &chain, &seg_cnt, &seg_hit,
                 &task_first, &task_tot, &task_off, &task_tmp, &task_sum, &res, &res_key};
     }
 
@@ -293,7 +293,7 @@ Workspace *workspace_for(const ae_index *cidx, cudaStream_t st) {
         if (p.first == st) return p.second;
     Workspace *w = new Workspace();
     w->stream = st;
-    if (cudaMallocHost(&w->h_tot, 64 * sizeof(uint64_t)) != cudaSuccess) {
+    if (cudaMallocHost(&w->h_tot, 256 * sizeof(uint64_t)) != cudaSuccess) {
         cudaGetLastError();
         delete w;
         throw ae_error{AE_ENOMEM};
@@ -395,6 +395,8 @@ ae_status make_score(const ae_scoring *s, int sigma, ScoreView &sc) {
     sc.sg = s->gap_open;
     sc.ss = s->gap_extend;
     if (s->gap_open > 0 || s->gap_extend >= 0) return AE_EINVAL;
+    const uint64_t u = (uint64_t)(-(int64_t)s->gap_extend);
+    sc.urec = ((1ull << 32) + u - 1) / u;
     if (s->matrix) {
         sc.use_matrix = 1;
         int gmax = INT32_MIN;
@@ -503,6 +505,10 @@ struct Search {
     }
 
     void run_batch(const std::vector<WorkItem> &items);
+    void dna_args(DnaRowsArgs &da, int cur, int64_t lf_ent_base, int64_t lf_node_base, int64_t rh_base);
+    int chain_levels(int depth, int64_t max_depth) const;
+    void dna_chain(int64_t &F, int &cur, int64_t &cur_ent, int64_t &lf_ent_base, int64_t &lf_node_base,
+                   int64_t &rh_base, int &depth, int levels);
     void dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_base, int64_t &lf_node_base,
                    int64_t &rh_base, const WorkItem *d_items);
     void run_batch_split(const std::vector<WorkItem> &items);
@@ -648,6 +654,11 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
         if (sigma == 4 && i16 && !opt.tier_stats && !root_level && !opt.general_rows && -sc.ss < 65536) {
             // DNA int16x2 route: one lane per parent entry, child ranges taken in
             // the task prologue (no separate children / compaction passes)
+            const int chain = chain_levels(depth, L_max_all);
+            if (chain > 1) {
+                dna_chain(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base, depth, chain);
+                continue;
+            }
             dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base, d_items);
             cur ^= 1;
             ++depth;
@@ -859,6 +870,10 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 #define AE_WIDE_ROW_AVG 512
 #endif
 
+// Levels launched in a row without a read-back, at most (their counters fit the
+// pinned staging words)
+constexpr int AE_CHAIN_MAX = 8;
+
 // Average parent-row length up to which a level's rows are packed over the
 // lanes; longer rows are spread one entry per lane.  Per level of the 100 Mbp
 // text with queries of 10 kbp to 1 Mbp (packed against the walk it replaces):
@@ -877,6 +892,142 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 #define AE_SEQ_ROW_AVG 256
 #endif
 
+// The arenas of one DNA level: parents in `cur`, children in the other one
+void Search::dna_args(DnaRowsArgs &da, int cur, int64_t lf_ent_base, int64_t lf_node_base, int64_t rh_base) {
+    const int nxt = cur ^ 1;
+    da.ix = ix;
+    da.sc = sc;
+    da.qv = qv;
+    da.leaf_delay = opt.leaf_delay;
+    da.base[0] = (uint64_t)lf_ent_base;
+    da.base[1] = (uint64_t)lf_node_base;
+    da.base[2] = (uint64_t)rh_base;
+    // capacities are the buffers' sizes (the leaf and hit arenas keep one spare slot)
+    auto cap = [](const DevBuf &b, size_t elem, int64_t spare) {
+        return (uint64_t)std::max<int64_t>((int64_t)(b.bytes / elem) - spare, 0);
+    };
+    da.nodes = ptr<Node>(w->nodes[cur]);
+    da.pj = ptr<int32_t>(w->aj[cur]);
+    da.pmg = ptr<uint32_t>(w->aM[cur]);
+    da.fj = ptr<int32_t>(w->aj[nxt]);
+    da.fmg = ptr<uint32_t>(w->aM[nxt]);
+    da.fnodes = ptr<Node>(w->nodes[nxt]);
+    da.fr_ent_cap = std::min(cap(w->aj[nxt], 4, 0), cap(w->aM[nxt], 4, 0));
+    da.fr_node_cap = cap(w->nodes[nxt], sizeof(Node), 0);
+    da.lj = ptr<int32_t>(w->lj);
+    da.lM = ptr<int32_t>(w->lM);
+    da.lGa = ptr<int32_t>(w->lGa);
+    da.inj = ptr<Inject>(w->inj);
+    da.lf_ent_cap = std::min({cap(w->lj, 4, 1), cap(w->lM, 4, 1), cap(w->lGa, 4, 1)});
+    da.lf_node_cap = cap(w->inj, sizeof(Inject), 1);
+    da.rhits = ptr<RangeHit>(w->rhits);
+    da.hit_cap = cap(w->rhits, sizeof(RangeHit), 1);
+}
+
+// Levels to launch without a read-back between them (1: run the next one by
+// itself).  A read-back costs a level of a small search far more than its rows
+// (40 us against 15-20 us: 24 levels of a 613 bp query 1.64 ms with a read-back
+// each, 0.73 in chains), and nothing where a level runs for a millisecond.
+// While levels grow, only as many are launched as the arenas
+// will most likely hold.
+int Search::chain_levels(int depth, int64_t max_depth) const {
+    if (opt.row_layout != 0 || g_arena || opt.workspace_limit > 0) return 1;
+    if (live_ent > AE_PACK_ROW_AVG * live_nodes) return 1;
+    const bool growing = !dna_ratio_ok || dna_ratio[0] > 0.9;
+    int64_t k = live_ent <= (1 << 16) ? 8 : live_ent <= (growing ? 1 << 20 : 1 << 22) ? (growing ? 3 : 8) : 1;
+    k = std::min<int64_t>(k, max_depth - depth + 1);
+    k = std::min<int64_t>(k, (int64_t)opt.int16_limit / sc.gmax - depth);   // (depth + k) g_max stays <= the limit
+    return (int)std::max<int64_t>(k, 1);
+}
+
+// `levels` levels of the packed layout in a row: each reads the sizes of its
+// input from the counters of the one before, and the host reads all of them
+// once.  A level whose outputs did not fit stops the chain and is run again by
+// itself (dna_level), the ones after it have done nothing.
+void Search::dna_chain(int64_t &F, int &cur, int64_t &cur_ent, int64_t &lf_ent_base, int64_t &lf_node_base,
+                       int64_t &rh_base, int &depth, int levels) {
+    // room for some growth; a failed allocation only makes the chain stop earlier
+    const int64_t ent = std::max<int64_t>(8 * live_ent, 1 << 22), nod = std::max<int64_t>(4 * live_nodes, 1 << 21);
+    const int64_t leaf = std::max<int64_t>(2 * live_ent, 1 << 19), hit = std::max<int64_t>(live_ent, 1 << 16);
+    try {
+        for (int b = 0; b < 2; ++b) {
+            if (b != cur) {
+                ensure(w->aj[b], (size_t)ent * 4, st);
+                ensure(w->aM[b], (size_t)ent * 4, st);
+                ensure(w->nodes[b], (size_t)nod * sizeof(Node), st);
+            } else {   // the parents' arena keeps them
+                ensure_keep(w->aj[b], (size_t)ent * 4, (size_t)cur_ent * 4, st);
+                ensure_keep(w->aM[b], (size_t)ent * 4, (size_t)cur_ent * 4, st);
+                ensure_keep(w->nodes[b], (size_t)nod * sizeof(Node), (size_t)F * sizeof(Node), st);
+            }
+        }
+        ensure_keep(w->lj, (size_t)(lf_ent_base + leaf + 1) * 4, (size_t)lf_ent_base * 4, st);
+        ensure_keep(w->lM, (size_t)(lf_ent_base + leaf + 1) * 4, (size_t)lf_ent_base * 4, st);
+        ensure_keep(w->lGa, (size_t)(lf_ent_base + leaf + 1) * 4, (size_t)lf_ent_base * 4, st);
+        ensure_keep(w->inj, (size_t)(lf_node_base + leaf + 1) * sizeof(Inject), (size_t)lf_node_base * sizeof(Inject), st);
+        ensure_keep(w->rhits, (size_t)(rh_base + hit + 1) * sizeof(RangeHit), (size_t)rh_base * sizeof(RangeHit), st);
+    } catch (const ae_error &e) {
+        if (e.st != AE_ENOMEM) throw;
+    }
+    ensure(w->chain, sizeof(LevelCounters) * AE_CHAIN_MAX, st);
+    CU(cudaMemsetAsync(w->chain.p, 0, sizeof(LevelCounters) * (size_t)levels, st));
+    const int64_t warps = (int64_t)num_sms * ae_rows_pack_blocks_per_sm() * ae_rows_pack_warps_per_block();
+    prof.mark(K_ROWS);
+    for (int l = 0; l < levels; ++l) {
+        DnaRowsArgs da;
+        memset(&da, 0, sizeof(da));
+        dna_args(da, cur ^ (l & 1), lf_ent_base, lf_node_base, rh_base);
+        da.sequential = 3;
+        da.nnodes = l ? 0 : F;
+        da.nodes_per_task = ae_rows_pack_task_nodes(F, live_nodes, live_ent, warps);
+        da.region_ent = (uint32_t)std::max<int64_t>(64, std::min<int64_t>(live_ent / (8 * warps), 2048));
+        const int64_t rn = F / (4 * warps);
+        da.region_node = rn >= 32 ? (uint32_t)std::min<int64_t>(rn, 1024) : 0;
+        da.chain = ptr<LevelCounters>(w->chain);
+        da.chain_pos = l;
+        da.ctr = ptr<LevelCounters>(w->chain) + l;
+        ae_rows_dna(da, num_sms * ae_rows_pack_blocks_per_sm(), st);
+    }
+    prof.mark(K_ROWS);
+    std::vector<LevelCounters> hc((size_t)levels);
+    CU(cudaMemcpyAsync(tot(), w->chain.p, sizeof(LevelCounters) * (size_t)levels, cudaMemcpyDeviceToHost, st));
+    sync();
+    memcpy(hc.data(), tot(), sizeof(LevelCounters) * (size_t)levels);
+    for (const LevelCounters &c : hc) {
+        if (c.overflow) throw ae_error{AE_ECUDA};
+        if (F <= 0) break;
+        if (c.retry) {
+            dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base, nullptr);
+        } else {
+            if (trace())
+                fprintf(stderr, "[ae level] dna packed nodes %lld (chain) entries %lld triples %lld -> frontier %lld nodes "
+                                "%lld, leaf %llu rows %llu\n",
+                        (long long)live_nodes, (long long)live_ent, (long long)c.triples, (long long)c.n_ent,
+                        (long long)c.n_node, c.lf_ent, c.lf_node);
+            stats.triples += (int64_t)c.triples;
+            dna_nodes += live_nodes;
+            dna_entries += (int64_t)(c.n_ent + c.lf_ent);
+            const double in[5] = {(double)live_ent, (double)live_ent, (double)live_nodes, (double)live_nodes,
+                                  (double)live_ent};
+            const double out[5] = {(double)c.n_ent, (double)c.lf_ent, (double)c.n_node, (double)c.lf_node, (double)c.hits};
+            for (int q = 0; q < 5; ++q) dna_ratio[q] = in[q] > 0 ? out[q] / in[q] : 0.0;
+            dna_ratio_ok = true;
+            lf_ent_base += (int64_t)c.lf_ent;
+            lf_node_base += (int64_t)c.lf_node;
+            rh_base += (int64_t)c.hits;
+            F = c.n_node ? (int64_t)c.fr_node : 0;
+            cur_ent = (int64_t)c.fr_ent;
+            live_nodes = (int64_t)c.n_node;
+            live_ent = (int64_t)c.n_ent;
+        }
+        cur ^= 1;
+        ++depth;
+        stats.levels++;
+        stats.levels_int16++;
+        if (c.retry) break;
+    }
+}
+
 // One trie level of the DNA int16x2 route (ae_rows_dna.cu) in one launch.
 // The output arenas are sized ahead from the previous level's output per input
 // (with headroom); the kernel reserves every task's ranges on the level
@@ -892,7 +1043,8 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
     const bool packed = opt.row_layout == 0 && !g_arena && live_ent <= AE_PACK_ROW_AVG * live_nodes;
     const int64_t warps = packed ? (int64_t)num_sms * ae_rows_pack_blocks_per_sm() * ae_rows_pack_warps_per_block()
                                  : (int64_t)num_sms * ae_rows_dna_blocks_per_sm() * ae_rows_dna_warps_per_block();
-    const int npt = (int)std::max<int64_t>(1, std::min<int64_t>(packed ? ae_rows_pack_nodes() : 32, F / (warps * 4)));
+    const int npt = packed ? ae_rows_pack_task_nodes(F, live_nodes, live_ent, warps)
+                           : (int)std::max<int64_t>(1, std::min<int64_t>(32, F / (warps * 4)));
 
     // expected outputs: per kind (frontier entries, leaf entries, frontier
     // nodes, leaf nodes, hits) the previous level's ratio to its input, plus a
@@ -957,18 +1109,10 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
 
     DnaRowsArgs da;
     memset(&da, 0, sizeof(da));
-    da.ix = ix;
-    da.sc = sc;
-    da.qv = qv;
     da.nnodes = F;
     da.nodes_per_task = npt;
     da.region_ent = region_ent;
     da.region_node = region_node;
-    da.leaf_delay = opt.leaf_delay;
-    {
-        const uint64_t u = (uint64_t)(-(int64_t)sc.ss);
-        da.urec = ((1ull << 32) + u - 1) / u;
-    }
     // short parent rows are walked one lane per (node, child); long rows spread
     // over the lanes (a lone long row would hold its warp alone)
     da.sequential = (opt.row_layout == 1) || (opt.row_layout == 0 && live_ent <= AE_SEQ_ROW_AVG * live_nodes) ? 1 : 0;
@@ -995,30 +1139,13 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
     auto run = [&]() {
         LevelCounters h0;
         memset(&h0, 0, sizeof(h0));
-        h0.lf_ent = (unsigned long long)lf_ent_base;
-        h0.lf_node = (unsigned long long)lf_node_base;
-        h0.hits = (unsigned long long)rh_base;
+        if (!packed) {   // the packed layout counts from zero behind its bases
+            h0.lf_ent = (unsigned long long)lf_ent_base;
+            h0.lf_node = (unsigned long long)lf_node_base;
+            h0.hits = (unsigned long long)rh_base;
+        }
         upload_level_counters(ptr<LevelCounters>(w->ctr), h0, st);
-        // capacities are the buffers' sizes (the leaf and hit arenas keep one spare slot)
-        auto cap = [](const DevBuf &b, size_t elem, int64_t spare) {
-            return (uint64_t)std::max<int64_t>((int64_t)(b.bytes / elem) - spare, 0);
-        };
-        da.nodes = ptr<Node>(w->nodes[cur]);
-        da.pj = ptr<int32_t>(w->aj[cur]);
-        da.pmg = ptr<uint32_t>(w->aM[cur]);
-        da.fj = ptr<int32_t>(w->aj[nxt]);
-        da.fmg = ptr<uint32_t>(w->aM[nxt]);
-        da.fnodes = ptr<Node>(w->nodes[nxt]);
-        da.fr_ent_cap = std::min(cap(w->aj[nxt], 4, 0), cap(w->aM[nxt], 4, 0));
-        da.fr_node_cap = cap(w->nodes[nxt], sizeof(Node), 0);
-        da.lj = ptr<int32_t>(w->lj);
-        da.lM = ptr<int32_t>(w->lM);
-        da.lGa = ptr<int32_t>(w->lGa);
-        da.inj = ptr<Inject>(w->inj);
-        da.lf_ent_cap = std::min({cap(w->lj, 4, 1), cap(w->lM, 4, 1), cap(w->lGa, 4, 1)});
-        da.lf_node_cap = cap(w->inj, sizeof(Inject), 1);
-        da.rhits = ptr<RangeHit>(w->rhits);
-        da.hit_cap = cap(w->rhits, sizeof(RangeHit), 1);
+        dna_args(da, cur, lf_ent_base, lf_node_base, rh_base);
         da.ctr = ptr<LevelCounters>(w->ctr);
         prof.mark(K_ROWS);
         ae_rows_dna(da, num_sms * (packed ? ae_rows_pack_blocks_per_sm() : ae_rows_dna_blocks_per_sm()), st);
@@ -1027,6 +1154,11 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
         sync();
         memcpy(&hc, tot(), sizeof(hc));
         if (hc.overflow) throw ae_error{AE_ECUDA};   // the two phases of a task disagreed
+        if (packed) {
+            hc.lf_ent += (unsigned long long)lf_ent_base;
+            hc.lf_node += (unsigned long long)lf_node_base;
+            hc.hits += (unsigned long long)rh_base;
+        }
     };
     run();
     int64_t lf_ent = (int64_t)hc.lf_ent - lf_ent_base, lf_node = (int64_t)hc.lf_node - lf_node_base;
@@ -1176,12 +1308,14 @@ void Search::leaf_phase(int64_t ninj) {
     // wide walks move to blocks (not inside the fixed arena of the no-allocation
     // entry point, nor when entries are counted by tier, which only the warp walk does)
     const bool sparse = (double)ninj * (AE_LEAF_GAP / 2) <= (double)ix.n * batch_queries;
-    // (where injections are dense every task walks a wide row and warps are the better
-    // use of the chip: 1 M residues, BLOSUM62: blocks from rows of 128 entries on 153 ms,
-    // 512: 173, 1,024: 91, never: 103)
-    const int32_t esc_min = (g_arena || opt.tier_stats || opt.leaf_wide_rows == 0) ? 0
-                            : sparse || opt.leaf_wide_rows < 128                 ? opt.leaf_wide_rows
-                                                                                 : std::max(opt.leaf_wide_rows, 1024);
+    // the default chooses: where injections leave gaps the few wide walks set the
+    // sweep's time, and a step on a block is faster from the first row past a warp's
+    // lanes on (613 bp query: 0.76 ms from 32 entries, 0.79 from 64, 1.09 from 128);
+    // where they are dense every task walks a wide row and warps are the better use of
+    // the chip (1 M residues, BLOSUM62: from 128 entries 153 ms, 512: 173, 1,024: 91,
+    // never: 103)
+    const int32_t wide = opt.leaf_wide_rows != 128 ? opt.leaf_wide_rows : sparse ? 32 : 1024;
+    const int32_t esc_min = (g_arena || opt.tier_stats) ? 0 : wide;
     const int32_t esc_max = esc_min > 0 ? AE_LEAF_WIDE_SLOTS : 0;
     // the counters before the sweep: one that is run again counts once
     ensure(w->stats_keep, sizeof(DevStats), st);

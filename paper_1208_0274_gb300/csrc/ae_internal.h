@@ -63,6 +63,7 @@ struct ScoreView {
     int32_t sa, sb, sg, ss;    // <s_a, s_b, s_g, s_s>
     int32_t use_matrix;
     int32_t gmax;              // largest gain of one query column (s_a or max matrix entry)
+    uint64_t urec;             // ceil(2^32 / -s_s): quotients by -s_s of numerators below 2^16 as products
     int8_t mat[AE_MAX_SIGMA * AE_MAX_SIGMA];   // delta(text letter, query letter)
 };
 

@@ -1207,10 +1207,11 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
 // position are looked up in the walked row by a warp each; those it dominates
 // (nearly all along a homolog) are done with that, the others are merged by
 // the whole block.  A row too long for shared memory moves to the block's
-// buffers in global memory and back.  About 7,500 cycles a step at rows of 1,300
-// entries, 4,500 at 200, where the warp walk takes 40,000 at 1,300 (in
-// instructions: the slots and the finish, three scans, the look-up); more
-// threads or more entries per thread spill registers and are slower.
+// buffers in global memory and back.  A step takes about 6,500 cycles at rows of
+// 1,300 entries (load and slots 1,430, the key scan 820, finish 860, the count
+// scan 1,110, writing 1,120, injected rows 1,100) and 3,800 at 200, where the
+// warp walk takes 40,000 at 1,300; more entries per thread spill registers and
+// are slower.
 #ifndef AE_WIDE_T
 #define AE_WIDE_T 512
 #endif
@@ -1481,8 +1482,14 @@ __global__ void __launch_bounds__(WIDE_T, 1) k_leaf_wide(LeafArgs a) {
                     }
                     uint32_t ci = 0, hi = 0;
                     if (active) {
-                        ci = warp_incl_sum(cl);
-                        hi = warp_incl_sum(hl);
+                        if (__any_sync(FULL, cl > 1023u)) {   // (no lane has more hits than outputs)
+                            ci = warp_incl_sum(cl);
+                            hi = warp_incl_sum(hl);
+                        } else {
+                            const uint32_t x = warp_incl_sum(cl | (hl << 16));
+                            ci = x & 0xFFFFu;
+                            hi = x >> 16;
+                        }
                     }
                     if (lane == 31) {
                         s.scnt[ph][wid] = ci;

@@ -187,7 +187,6 @@ struct DnaRowsArgs {
     int64_t nnodes;
     int32_t nodes_per_task;
     int32_t leaf_delay;
-    uint64_t urec;                        // ceil(2^32 / u), u = -s_s: gap-run lengths without division
     int32_t sequential;                   // row layout: 3 rows packed over a warp's lanes, 1 one lane per (node,
                                           // child) walking the parent row in order, 0 one lane per parent entry,
                                           // 2 one block per node
@@ -212,13 +211,23 @@ struct DnaRowsArgs {
     // packed layout: entries and node records a warp takes of the frontier arenas at a
     // time (0: exactly what it writes)
     uint32_t region_ent, region_node;
+    // packed layout: `ctr` starts at zero and the leaf and hit places it hands out lie
+    // behind base[0..2] (leaf entries, injections, hits).  In a chain of levels launched
+    // without a read-back between them, chain[0..chain_pos) are the counters of the
+    // chain's earlier levels: the level's nodes are those the last one wrote (none after
+    // a level that must be run again), its bases follow all of them, and the task and
+    // region sizes are taken from its own size.
+    uint64_t base[3];
+    const LevelCounters *chain;
+    int32_t chain_pos;
 };
 void ae_rows_dna(const DnaRowsArgs &a, int blocks, cudaStream_t st);
 int ae_rows_dna_blocks_per_sm();
 int ae_rows_dna_warps_per_block();
 int ae_rows_pack_blocks_per_sm();
 int ae_rows_pack_warps_per_block();
-int ae_rows_pack_nodes();   // nodes per task at most
+// nodes per task of a level with `nodes` nodes in `slots` records and `entries` row entries
+int ae_rows_pack_task_nodes(int64_t slots, int64_t nodes, int64_t entries, int64_t warps);
 struct LeafArgs {
     IndexView ix;
     ScoreView sc;

@@ -111,16 +111,6 @@ struct WarpSmem {
     uint64_t base[3];   // write: the task's first slot in the frontier, leaf and hit arenas
 };
 
-// Length of a gap run (Section 2.2: a horizontal gap extended column by column)
-// without a division: the run after a lane's last slot starts at column rs with
-// G_b = V0 > 0 and loses u per column, so away from the query's last columns
-// (threshold 0) its live cells number floor((V0 - 1) / u) + 1.  The quotient is
-// taken as a product with the reciprocal rec = ceil(2^32 / u), exact for
-// numerators below 2^16 (the int16x2 route keeps every state below 2^15).
-__device__ __forceinline__ uint32_t div_small(uint32_t a, uint64_t rec) {
-    return (uint32_t)(((uint64_t)a * rec) >> 32);
-}
-
 __device__ __forceinline__ uint64_t reduce_add_u64(uint32_t v) {
     const uint32_t hi = __reduce_add_sync(FULL, v >> 16), lo = __reduce_add_sync(FULL, v & 0xFFFFu);
     return ((uint64_t)hi << 16) + lo;
@@ -298,10 +288,10 @@ __device__ __forceinline__ void rows_seq(const DnaRowsArgs &a, WarpSmem &sm, int
             const int32_t rs = hasB ? j + 2 : j + 1;
             const int32_t V0 = sc.sg - rs * u + K;
             if (K > AE_KNEG / 2 && rs < jn && V0 > 0) {
-                const int32_t rl = min((int32_t)div_small((uint32_t)(V0 - 1), a.urec) + 1, jn - rs);
+                const int32_t rl = min((int32_t)div_small((uint32_t)(V0 - 1), a.sc.urec) + 1, jn - rs);
                 if (traw + (rs + rl - 1) * g <= 0) {
                     run_len = rl;
-                    if (V0 >= H) run_hits = min(rl, (int32_t)div_small((uint32_t)(V0 - H), a.urec) + 1);
+                    if (V0 >= H) run_hits = min(rl, (int32_t)div_small((uint32_t)(V0 - H), a.sc.urec) + 1);
                 } else {
                     run_of(rs, jn, K, sc, m, H, u, run_len, run_hits);
                 }
@@ -507,10 +497,10 @@ __device__ __forceinline__ void rows_spread(const DnaRowsArgs &a, WarpSmem &sm, 
             const int32_t run_start = hasB ? j + 2 : j + 1;
             const int32_t V0 = sc.sg - run_start * u + incl;
             if (has_c && incl > AE_KNEG / 2 && run_start < jn && V0 > 0) {
-                const int32_t rl = min((int32_t)div_small((uint32_t)(V0 - 1), a.urec) + 1, jn - run_start);
+                const int32_t rl = min((int32_t)div_small((uint32_t)(V0 - 1), a.sc.urec) + 1, jn - run_start);
                 if (traw + (run_start + rl - 1) * g <= 0) {   // threshold 0 over the whole run
                     run_len = rl;
-                    if (V0 >= H) run_hits = min(rl, (int32_t)div_small((uint32_t)(V0 - H), a.urec) + 1);
+                    if (V0 >= H) run_hits = min(rl, (int32_t)div_small((uint32_t)(V0 - H), a.sc.urec) + 1);
                 } else {                                       // the query's last columns: exact form
                     run_of(run_start, jn, incl, sc, m, H, u, run_len, run_hits);
                 }
@@ -925,6 +915,7 @@ struct __align__(16) PackRegion {
 };
 
 struct PackWarp {
+    uint64_t base[3];            // before this level's leaf entries, injections and hits
     PackRegion reg[4];           // the frontier regions by child index
     int32_t carry[4];            // the open row's horizontal-gap key (0: none)
     uint64_t off[PK_N];          // the node's row
@@ -1001,10 +992,10 @@ __device__ __forceinline__ void pack_finish(const DnaRowsArgs &a, const PackEntr
     o.rs = e.hasB ? e.j + 2 : e.j + 1;
     o.V0 = base - (e.hasB ? 2 * u : u) + incl;
     if (has && o.V0 > 0 && o.rs < e.jn) {
-        const int32_t rl = min((int32_t)div_small((uint32_t)(o.V0 - 1), a.urec) + 1, e.jn - o.rs);
+        const int32_t rl = min((int32_t)div_small((uint32_t)(o.V0 - 1), a.sc.urec) + 1, e.jn - o.rs);
         if (e.traw + (o.rs + rl - 1 - e.j) * sc.gmax <= 0) {   // threshold 0 over the whole run
             o.run_len = rl;
-            if (o.V0 >= e.H) o.run_hits = min(rl, (int32_t)div_small((uint32_t)(o.V0 - e.H), a.urec) + 1);
+            if (o.V0 >= e.H) o.run_hits = min(rl, (int32_t)div_small((uint32_t)(o.V0 - e.H), a.sc.urec) + 1);
         } else {
             run_of(o.rs, e.jn, incl, sc, e.m, e.H, u, o.run_len, o.run_hits);
         }
@@ -1029,18 +1020,19 @@ __device__ __forceinline__ void pack_each(const DnaRowsArgs &a, const PackEntry 
 
 // A warp's output state besides its entry regions (all values warp-uniform)
 struct PackOut {
+    uint32_t region_ent, region_node;   // as in DnaRowsArgs
     uint64_t npos;          // next free node record of the warp's region
     uint32_t nrem;          // what is left of it
     bool efull, nfull;      // an arena's capacity was passed: nothing is written to it any more
     uint32_t ents, nodes;   // written to the frontier since the counts were last added up
 };
 
-// Slots of `n` for a warp on one of the level's cursors; ok = within `cap`
-__device__ __forceinline__ uint64_t pack_take(const DnaRowsArgs &a, unsigned long long *cursor, uint64_t n, uint64_t cap,
-                                              int lane, bool &ok) {
+// Slots of `n` for a warp on one of the level's cursors, behind `base`; ok = within `cap`
+__device__ __forceinline__ uint64_t pack_take(const DnaRowsArgs &a, unsigned long long *cursor, uint64_t base, uint64_t n,
+                                              uint64_t cap, int lane, bool &ok) {
     unsigned long long b = 0;
     if (lane == 0) b = atomicAdd(cursor, (unsigned long long)n);
-    b = __shfl_sync(FULL, b, 0);
+    b = base + __shfl_sync(FULL, b, 0);
     ok = b + n <= cap;
     if (!ok && lane == 0) atomicExch(&a.ctr->retry, 1ull);
     return b;
@@ -1052,10 +1044,10 @@ __device__ __forceinline__ void pack_new_region(const DnaRowsArgs &a, PackOut &o
                                                 uint32_t need) {
     const uint64_t old = g.pos - part;
     // an open row may still grow: twice the room, so that a long row moves a few times only
-    const uint32_t n = max(a.region_ent, part ? 2 * (part + need) : need);
+    const uint32_t n = max(o.region_ent, part ? 2 * (part + need) : need);
     const bool had = !o.efull;
     bool ok;
-    const uint64_t b = pack_take(a, &a.ctr->fr_ent, n, a.fr_ent_cap, lane, ok);
+    const uint64_t b = pack_take(a, &a.ctr->fr_ent, 0, n, a.fr_ent_cap, lane, ok);
     if (!ok) o.efull = true;
     __syncwarp();   // the part written so far is complete
     if (had && ok)
@@ -1079,9 +1071,9 @@ __device__ __forceinline__ PackPlace pack_node_room(const DnaRowsArgs &a, PackOu
     o.npos += p.room;
     o.nrem -= p.room;
     if (p.room < need) {
-        const uint32_t n = max(a.region_node, need - p.room);
+        const uint32_t n = max(o.region_node, need - p.room);
         bool ok;
-        o.npos = pack_take(a, &a.ctr->fr_node, n, a.fr_node_cap, lane, ok);
+        o.npos = pack_take(a, &a.ctr->fr_node, 0, n, a.fr_node_cap, lane, ok);
         o.nrem = n;
         if (!ok) o.nfull = true;
     }
@@ -1250,7 +1242,7 @@ __device__ __forceinline__ void pack_rows(const DnaRowsArgs &a, PackWarp &w, Pac
                 if (__any_sync(FULL, hc)) {
                     const uint32_t hi = warp_incl_sum(hc);
                     bool ok;
-                    uint64_t h = pack_take(a, &a.ctr->hits, __shfl_sync(FULL, hi, 31), a.hit_cap, lane, ok) + (hi - hc);
+                    uint64_t h = pack_take(a, &a.ctr->hits, w.base[2], __shfl_sync(FULL, hi, 31), a.hit_cap, lane, ok) + (hi - hc);
                     if (ok && hc)
                         pack_each(a, e, o, [&](int32_t col, int32_t M, uint32_t) {
                             if (M >= H)
@@ -1265,8 +1257,8 @@ __device__ __forceinline__ void pack_rows(const DnaRowsArgs &a, PackWarp &w, Pac
                     const uint32_t c = done && go ? cells : 0u, li = warp_incl_sum(c);
                     const uint32_t lt_ent = __shfl_sync(FULL, li, 31);
                     bool ok, nok;
-                    const uint64_t b = pack_take(a, &a.ctr->lf_ent, lt_ent, a.lf_ent_cap, lane, ok) + (li - c);
-                    const uint64_t y = pack_take(a, &a.ctr->lf_node, __popc(bl), a.lf_node_cap, lane, nok);
+                    const uint64_t b = pack_take(a, &a.ctr->lf_ent, w.base[0], lt_ent, a.lf_ent_cap, lane, ok) + (li - c);
+                    const uint64_t y = pack_take(a, &a.ctr->lf_node, w.base[1], __popc(bl), a.lf_node_cap, lane, nok);
                     out.ents -= lt_ent;
                     __syncwarp();   // the rows are complete
                     if (ok && !out.efull) {
@@ -1297,15 +1289,52 @@ __device__ __forceinline__ void pack_rows(const DnaRowsArgs &a, PackWarp &w, Pac
     }
 }
 
+// Nodes per task: enough for a task per warp, and not fewer than fill a chunk
+// (a chunk takes the same time however many of its lanes have an entry)
+__host__ __device__ __forceinline__ int pack_task_nodes(int64_t slots, int64_t nodes, int64_t entries, int64_t warps) {
+    int64_t n = (slots + warps - 1) / warps;
+    const int64_t chunk = 32 * nodes / (entries > 0 ? entries : 1);
+    if (n < chunk) n = chunk;
+    return (int)(n < 1 ? 1 : n > PK_N ? PK_N : n);
+}
+
 __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsArgs a) {
     __shared__ PackWarp smem[PK_W];
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     PackWarp &w = smem[threadIdx.x >> 5];
-    const int npt = a.nodes_per_task;
-    const uint64_t ntask = (uint64_t)((a.nnodes + npt - 1) / npt);
-    uint64_t trip = 0, ents = 0, nodes = 0;   // (child, parent entry) pairs of this lane; entries and nodes written
+    int64_t nnodes = a.nnodes;
+    int npt = a.nodes_per_task;
     PackOut out;
+    out.region_ent = a.region_ent;
+    out.region_node = a.region_node;
+    if (lane < 3) w.base[lane] = a.base[lane];
+    if (a.chain_pos > 0) {
+        uint64_t b[3] = {a.base[0], a.base[1], a.base[2]};
+        bool again = false;
+        for (int l = 0; l < a.chain_pos; ++l) {
+            const LevelCounters &c = a.chain[l];
+            b[0] += c.lf_ent;
+            b[1] += c.lf_node;
+            b[2] += c.hits;
+            again = again || c.retry;
+        }
+        const LevelCounters &c = a.chain[a.chain_pos - 1];
+        nnodes = again || !c.n_node ? 0 : (int64_t)c.fr_node;
+        if (nnodes == 0) return;
+        if (lane == 0) {
+            w.base[0] = b[0];
+            w.base[1] = b[1];
+            w.base[2] = b[2];
+        }
+        const int64_t warps = (int64_t)gridDim.x * PK_W;
+        npt = pack_task_nodes(nnodes, (int64_t)c.n_node, (int64_t)c.n_ent, warps);
+        out.region_ent = (uint32_t)max((int64_t)64, min((int64_t)2048, (int64_t)c.n_ent / (8 * warps)));
+        const int64_t rn = nnodes / (4 * warps);
+        out.region_node = rn >= 32 ? (uint32_t)min(rn, (int64_t)1024) : 0u;
+    }
+    const uint64_t ntask = (uint64_t)((nnodes + npt - 1) / npt);
+    uint64_t trip = 0, ents = 0, nodes = 0;   // (child, parent entry) pairs of this lane; entries and nodes written
     out.npos = 0;
     out.nrem = out.ents = out.nodes = 0;
     out.efull = out.nfull = false;
@@ -1313,11 +1342,9 @@ __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsAr
         w.reg[lane] = PackRegion{0, 0, 0};
         w.carry[lane] = 0;
     }
-    for (;;) {
-        unsigned long long task = 0;
-        if (lane == 0) task = atomicAdd(&a.ctr->task_c, 1ull);
-        task = __shfl_sync(FULL, task, 0);
-        if (task >= ntask) break;
+    // a warp's first task is its own number, the next ones come from the counter
+    const uint64_t nwarps = (uint64_t)gridDim.x * PK_W;
+    for (uint64_t task = (uint64_t)blockIdx.x * PK_W + (threadIdx.x >> 5); task < ntask;) {
         // ---- prologue: child ranges, PK_R nodes per lane, then their order
         Node nd[PK_R];
         unsigned km[PK_R];
@@ -1325,7 +1352,7 @@ __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsAr
         for (int r = 0; r < PK_R; ++r) {
             const int64_t v = (int64_t)task * npt + r * 32 + lane;
             nd[r] = Node{0, 0, 0, 0, 0};
-            if (r * 32 + lane < npt && v < a.nnodes) nd[r] = a.nodes[v];
+            if (r * 32 + lane < npt && v < nnodes) nd[r] = a.nodes[v];
         }
 #pragma unroll
         for (int r = 0; r < PK_R; ++r) {
@@ -1383,6 +1410,10 @@ __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsAr
         nodes += out.nodes;
         out.ents = out.nodes = 0;
         __syncwarp();
+        if (ntask <= nwarps) break;
+        unsigned long long next = 0;
+        if (lane == 0) next = atomicAdd(&a.ctr->task_c, 1ull);
+        task = nwarps + __shfl_sync(FULL, next, 0);
     }
     if (!out.nfull)   // the rest of the node region holds empty records
         for (uint32_t i = lane; i < out.nrem; i += 32) a.fnodes[out.npos + i] = Node{0, 0, 0, 0, 0};
@@ -1576,10 +1607,10 @@ __global__ void __launch_bounds__(WB_T) k_rows_dna_wide(DnaRowsArgs a) {
                     const int32_t run_start = hasB ? j + 2 : j + 1;
                     const int32_t V0 = sc.sg - run_start * u + incl;
                     if (ok && incl > AE_KNEG / 2 && run_start < jn && V0 > 0) {
-                        const int32_t rl = min((int32_t)div_small((uint32_t)(V0 - 1), a.urec) + 1, jn - run_start);
+                        const int32_t rl = min((int32_t)div_small((uint32_t)(V0 - 1), a.sc.urec) + 1, jn - run_start);
                         if (traw + (run_start + rl - 1) * g <= 0) {
                             run_len = rl;
-                            if (V0 >= H) run_hits = min(rl, (int32_t)div_small((uint32_t)(V0 - H), a.urec) + 1);
+                            if (V0 >= H) run_hits = min(rl, (int32_t)div_small((uint32_t)(V0 - H), a.sc.urec) + 1);
                         } else {
                             run_of(run_start, jn, incl, sc, m, H, u, run_len, run_hits);
                         }
@@ -1732,10 +1763,12 @@ int ae_rows_dna_blocks_per_sm() { return AE_DNA_MINB; }
 int ae_rows_dna_warps_per_block() { return DW; }
 int ae_rows_pack_blocks_per_sm() { return AE_PACK_MINB; }
 int ae_rows_pack_warps_per_block() { return PK_W; }
-int ae_rows_pack_nodes() { return PK_N; }
+int ae_rows_pack_task_nodes(int64_t slots, int64_t nodes, int64_t entries, int64_t warps) {
+    return pack_task_nodes(slots, nodes, entries, warps);
+}
 
 void ae_rows_dna(const DnaRowsArgs &a, int blocks, cudaStream_t st) {
-    if (a.nnodes <= 0) return;
+    if (a.nnodes <= 0 && a.chain_pos == 0) return;
     ++g_launches;
     if (a.sequential == 3) {   // rows packed over the lanes
         k_rows_pack<<<blocks, PK_W * 32, 0, st>>>(a);
