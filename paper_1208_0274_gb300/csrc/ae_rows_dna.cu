@@ -1173,7 +1173,8 @@ __device__ __forceinline__ void pack_rows(const DnaRowsArgs &a, PackWarp &w, Pac
             const uint32_t part = cont_in ? g.part : 0u;
             // ---- places: ranks over the warp, one row after the other
             uint32_t cnt, ci, tot;
-            if (__any_sync(FULL, incl != 0) || cin) {   // some horizontal gap is alive
+            const bool gaps = __any_sync(FULL, incl != 0) || cin;
+            if (gaps) {   // some horizontal gap is alive
                 int32_t excl;
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
@@ -1227,14 +1228,23 @@ __device__ __forceinline__ void pack_rows(const DnaRowsArgs &a, PackWarp &w, Pac
             const unsigned be = __ballot_sync(FULL, done && !go);
             if (be) {
                 const uint32_t nn = __popc(be);
-                const PackPlace np = pack_node_room(a, out, lane, nn);
-                if (done && !go && !out.nfull) {
-                    const uint32_t r = __popc(be & lt);
-                    pack_put_node(a, r < np.room ? np.at + r : out.npos + (r - np.room), w.lo[i][s], w.hi[i][s],
-                                  w.item[s], cells, epos + row0 - before);
+                if (out.nrem >= nn) {   // warp-uniform, nearly always
+                    if (done && !go && !out.nfull)
+                        pack_put_node(a, out.npos + __popc(be & lt), w.lo[i][s], w.hi[i][s], w.item[s], cells,
+                                      epos + row0 - before);
+                    out.npos += nn;
+                    out.nrem -= nn;
+                    out.nodes += nn;
+                } else {
+                    const PackPlace np = pack_node_room(a, out, lane, nn);
+                    if (done && !go && !out.nfull) {
+                        const uint32_t r = __popc(be & lt);
+                        pack_put_node(a, r < np.room ? np.at + r : out.npos + (r - np.room), w.lo[i][s], w.hi[i][s],
+                                      w.item[s], cells, epos + row0 - before);
+                    }
+                    out.npos += nn - np.room;
+                    out.nrem -= nn - np.room;
                 }
-                out.npos += nn - np.room;
-                out.nrem -= nn - np.room;
             }
             // ---- range hits of the rows that stay
             if (may_hit) {
@@ -1289,10 +1299,10 @@ __device__ __forceinline__ void pack_rows(const DnaRowsArgs &a, PackWarp &w, Pac
     }
 }
 
-// Nodes per task: enough for a task per warp, and not fewer than fill a chunk
-// (a chunk takes the same time however many of its lanes have an entry)
+// Nodes per task: an eighth of a warp's share, and not fewer than fill a chunk (a
+// chunk takes the same time however many of its lanes have an entry)
 __host__ __device__ __forceinline__ int pack_task_nodes(int64_t slots, int64_t nodes, int64_t entries, int64_t warps) {
-    int64_t n = (slots + warps - 1) / warps;
+    int64_t n = slots / (8 * warps);
     const int64_t chunk = 32 * nodes / (entries > 0 ? entries : 1);
     if (n < chunk) n = chunk;
     return (int)(n < 1 ? 1 : n > PK_N ? PK_N : n);
@@ -1346,40 +1356,37 @@ __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsAr
     const uint64_t nwarps = (uint64_t)gridDim.x * PK_W;
     for (uint64_t task = (uint64_t)blockIdx.x * PK_W + (threadIdx.x >> 5); task < ntask;) {
         // ---- prologue: child ranges, PK_R nodes per lane, then their order
-        Node nd[PK_R];
-        unsigned km[PK_R];
-#pragma unroll
-        for (int r = 0; r < PK_R; ++r) {
+        unsigned kms = 0;   // child masks, four bits a round
+#pragma unroll 1
+        for (int r = 0; r * 32 < npt; ++r) {
             const int64_t v = (int64_t)task * npt + r * 32 + lane;
-            nd[r] = Node{0, 0, 0, 0, 0};
-            if (r * 32 + lane < npt && v < nnodes) nd[r] = a.nodes[v];
-        }
-#pragma unroll
-        for (int r = 0; r < PK_R; ++r) {
+            Node nd = Node{0, 0, 0, 0, 0};
+            if (r * 32 + lane < npt && v < nnodes) nd = a.nodes[v];
             uint32_t clo[4], chi[4];
-            km[r] = nd[r].cnt ? kids4(a.ix, nd[r].lo, nd[r].hi, clo, chi) : 0u;
-            trip += (uint64_t)__popc(km[r]) * nd[r].cnt;
-            if (!km[r]) continue;
+            const unsigned km = nd.cnt ? kids4(a.ix, nd.lo, nd.hi, clo, chi) : 0u;
+            kms |= km << (4 * r);
+            trip += (uint64_t)__popc(km) * nd.cnt;
+            if (!km) continue;
             const int s = r * 32 + lane;
             // a child stays in the walk while it has several occurrences, or for
             // the first leaf_delay levels after it became a single one
-            const bool young = (int)((uint32_t)nd[r].item >> 24) + 1 <= a.leaf_delay;
-            uint32_t kid = (uint32_t)__popc(km[r]) << 12;
+            const bool young = (int)((uint32_t)nd.item >> 24) + 1 <= a.leaf_delay;
+            uint32_t kid = (uint32_t)__popc(km) << 12;
             int i = 0;
 #pragma unroll
             for (int c = 0; c < 4; ++c)
-                if ((km[r] >> c) & 1u) {
+                if ((km >> c) & 1u) {
                     kid |= (uint32_t)c << (2 * i);
                     if (young || chi[c] - clo[c] >= 2) kid |= 256u << i;
                     w.lo[i][s] = clo[c];
                     w.hi[i][s] = chi[c];
                     ++i;
                 }
-            const int32_t qid = nd[r].item & 0xFFFFFF;
+            const int32_t qid = nd.item & 0xFFFFFF;
             w.kid[s] = kid;
-            w.off[s] = nd[r].off;
-            w.len[s] = nd[r].cnt;
-            w.item[s] = (uint32_t)nd[r].item;
+            w.off[s] = nd.off;
+            w.len[s] = nd.cnt;
+            w.item[s] = (uint32_t)nd.item;
             w.m[s] = a.qv.m[qid];
             w.H[s] = a.qv.H[qid];
             w.qoff[s] = (uint32_t)a.qv.off[qid];
@@ -1389,7 +1396,7 @@ __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsAr
         for (int k = 4; k > 0; --k) {
 #pragma unroll
             for (int r = 0; r < PK_R; ++r) {
-                const bool mine = __popc(km[r]) == k;
+                const bool mine = __popc((kms >> (4 * r)) & 15u) == k;
                 const unsigned b = __ballot_sync(FULL, mine);
                 if (mine) w.ord[n + __popc(b & lt)] = (uint8_t)(r * 32 + lane);
                 n += __popc(b);

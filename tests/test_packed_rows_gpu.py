@@ -48,7 +48,9 @@ def test_packed_rows_equal_general_rows(case):
     for general in (1, 0):
         hits, counts = ae.ae_search(idx, qs, Scheme(*sch), H, options=ae.make_options(general_rows=general, **opts))
         st = ae.ae_last_stats()
-        got.append((hits, counts, [st[k] for k in ("entries", "triples", "nodes", "injections", "levels", "reroutes")]))
+        # the trie's entries (those of the sweep depend on the order of rows injected at one position)
+        got.append((hits, counts, [st["entries"] - st["entries_leaf"]] +
+                    [st[k] for k in ("triples", "nodes", "injections", "reroutes")]))
     idx.close()
     assert got[0][0].size > 0
     assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
