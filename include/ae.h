@@ -191,7 +191,7 @@ void ae_options_default(ae_options *opt);
  * for protein) with sampled ranks, the text-end array (entry h = end position
  * in T of the substrings whose reverse prefixes suffix h), and the forward
  * text (Section 2.3 and Section 5 (1)-(3)).  The suffix array is built on the
- * current CUDA device (ae_suffix_array_device, about 33 bytes of device memory
+ * current CUDA device (ae_suffix_array_device, about 45 bytes of device memory
  * per letter while it runs, beside the index's own 5.5), and the arrays are
  * filled from it there; the host keeps no copy.
  * Errors: AE_EINVAL (n < 1, unknown letter, bad alphabet), AE_EUNSUPPORTED
@@ -328,12 +328,14 @@ ae_status ae_suffix_array(const uint8_t *codes, int64_t n, int32_t sigma, int32_
  * receives the start positions of the suffixes of s followed by a sentinel
  * smaller than every code, in lexicographic order (d_sa[0] = n).
  * Method: prefix doubling (Manber & Myers 1993).  Each suffix's first key
- * packs its first 64/b letters (b bits per letter value and the sentinel),
- * and a stable LSD radix sort groups equal keys.  The group index becomes the
- * rank, and the next key (rank of i, rank of i + h) orders by twice as many
- * letters.  Rounds stop when every rank is distinct.
+ * packs its first letters (enough for about 100 n different keys), and a
+ * stable LSD radix sort groups equal keys.  A group's first place becomes the
+ * rank of its suffixes, and the suffixes that share a key are sorted again by
+ * (rank of i, rank of i + h), which orders by twice as many letters (the
+ * others stay, as in Larsson & Sadakane 2007).  Rounds stop when every rank is
+ * distinct.
  * d_codes and d_sa are device memory: codes in [0, sigma), 1 <= sigma <= 255,
- * 0 <= n < 2^31 - 2.  The call allocates and frees about 33 bytes of device
+ * 0 <= n < 2^31 - 2.  The call allocates and frees about 45 bytes of device
  * memory per letter, and returns once `stream` (NULL = the legacy default
  * stream) has finished its work.
  * Errors: AE_EINVAL (NULL pointer, sigma out of range, a code >= sigma),

@@ -160,8 +160,26 @@ void scan_rec(const In *const *inp, uint64_t *const *outp, int64_t N, uint64_t *
 }
 
 // ------------------------------------------------------------------ radix sort
+//
+// Stable LSD sort of (key, value) pairs, 8 bits a pass.  A tile's pairs are
+// ranked by digit in registers and put in digit order in shared memory, so that
+// they leave in runs (16 pairs of a digit on average, 128 bytes of keys) instead
+// of one scattered 8-byte store each.  10^7 pairs take 88 us in the scatter (240
+// MB, 2.7 TB/s; bound by the ranking's votes and shared-memory chain) and 27 in
+// the histogram, where one store per pair took 290 us a pass in all.  Up to
+// RS_SMALL pairs one block does all passes in shared memory in one launch (the
+// sorts of a small search were 5 passes of 3 launches, 24 us a pass).
+constexpr int RS_T = 256, RS_I = 16, RS_TILE = RS_T * RS_I;
+constexpr int RS_ST = 1024, RS_SI = 8, RS_SMALL = RS_ST * RS_SI;
 
-constexpr int RS_T = 256, RS_TILE = 2048, RS_PER_WARP = 256;
+template <int T, int I>
+struct RsSmem {
+    uint64_t key[T * I];
+    uint32_t val[T * I];
+    uint32_t wcnt[T / 32][256];   // per warp and digit: pairs, then the pairs of earlier warps
+    uint32_t first[256];          // the digit's first place in the tile
+    uint32_t wsum[8];
+};
 
 __global__ void __launch_bounds__(RS_T) k_rs_hist(const uint64_t *keys, int64_t N, int shift, uint32_t *hist,
                                                   int64_t ntiles) {
@@ -169,57 +187,137 @@ __global__ void __launch_bounds__(RS_T) k_rs_hist(const uint64_t *keys, int64_t 
     cnt[threadIdx.x] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    for (int i = threadIdx.x; i < RS_TILE; i += RS_T) {
-        int64_t idx = base + i;
+#pragma unroll
+    for (int i = 0; i < RS_I; ++i) {
+        const int64_t idx = base + i * RS_T + threadIdx.x;
         if (idx < N) atomicAdd(&cnt[(keys[idx] >> shift) & 255], 1u);
     }
     __syncthreads();
     hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
 }
 
-__global__ void __launch_bounds__(RS_T) k_rs_scatter(const uint64_t *kin, const uint32_t *vin, uint64_t *kout,
+// A tile's pairs (thread order: warp, round, lane; the first n are there) into
+// digit order in s.key / s.val; s.first holds each digit's first place
+template <int T, int I>
+__device__ __forceinline__ void rs_tile(RsSmem<T, I> &s, const uint64_t (&k)[I], const uint32_t (&v)[I], int n, int shift) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int d = lane; d < 256; d += 32) s.wcnt[wid][d] = 0;
+    __syncwarp();
+    uint32_t rank[I];   // among the warp's pairs of the same digit
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+        const bool valid = wid * 32 * I + i * 32 + lane < n;
+        const int d = (int)((k[i] >> shift) & 255);
+        // the lanes with the same digit, bit by bit (eight votes: the match instruction
+        // takes three times as long)
+        unsigned peers = __ballot_sync(FULL, valid);
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            const unsigned vote = __ballot_sync(FULL, (d >> x) & 1);
+            peers &= ((d >> x) & 1) ? vote : ~vote;
+        }
+        const uint32_t c = valid ? s.wcnt[wid][d] : 0u;
+        __syncwarp();
+        rank[i] = c + __popc(peers & lt);
+        if (valid && lane == __ffs(peers) - 1) s.wcnt[wid][d] = c + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    if (threadIdx.x < 256) {
+        uint32_t sum = 0;
+        for (int x = 0; x < T / 32; ++x) {
+            const uint32_t c = s.wcnt[x][threadIdx.x];
+            s.wcnt[x][threadIdx.x] = sum;
+            sum += c;
+        }
+        const uint32_t incl = warp_incl_sum(sum);
+        if (lane == 31) s.wsum[wid] = incl;
+        s.first[threadIdx.x] = incl - sum;
+    }
+    __syncthreads();
+    if (threadIdx.x < 256) {
+        uint32_t before = 0;
+        for (int x = 0; x < wid; ++x) before += s.wsum[x];
+        s.first[threadIdx.x] += before;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+        if (wid * 32 * I + i * 32 + lane >= n) continue;
+        const int d = (int)((k[i] >> shift) & 255);
+        const uint32_t x = s.first[d] + s.wcnt[wid][d] + rank[i];
+        s.key[x] = k[i];
+        s.val[x] = v[i];
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(RS_T, 3) k_rs_scatter(const uint64_t *kin, const uint32_t *vin, uint64_t *kout,
                                                      uint32_t *vout, int64_t N, int shift, const uint64_t *offs,
                                                      int64_t ntiles) {
-    __shared__ uint32_t wcnt[RS_T / 32][256];
+    extern __shared__ __align__(16) unsigned char rs_smem[];
+    RsSmem<RS_T, RS_I> &s = *reinterpret_cast<RsSmem<RS_T, RS_I> *>(rs_smem);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int d = lane; d < 256; d += 32) wcnt[wid][d] = 0;
-    __syncwarp();
-    const int64_t wbase = (int64_t)blockIdx.x * RS_TILE + (int64_t)wid * RS_PER_WARP;
-    const unsigned lt = (1u << lane) - 1u;
-    for (int r = 0; r < RS_PER_WARP / 32; ++r) {
-        int64_t idx = wbase + r * 32 + lane;
-        bool valid = idx < N;
-        int d = valid ? (int)((kin[idx] >> shift) & 255) : 256;
-        unsigned peers = __match_any_sync(FULL, d);
-        if (valid && lane == __ffs(peers) - 1) wcnt[wid][d] += __popc(peers);
-        __syncwarp();
+    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+    const int n = (int)min((int64_t)RS_TILE, N - base);
+    uint64_t k[RS_I];
+    uint32_t v[RS_I];
+#pragma unroll
+    for (int i = 0; i < RS_I; ++i) {
+        const int x = wid * 32 * RS_I + i * 32 + lane;
+        k[i] = x < n ? kin[base + x] : 0;
+        v[i] = x < n ? vin[base + x] : 0;
     }
+    // where the tile's pairs of each digit go
+    const uint64_t out0 = offs[(int64_t)threadIdx.x * ntiles + blockIdx.x];
+    rs_tile<RS_T, RS_I>(s, k, v, n, shift);
+    uint64_t *out = reinterpret_cast<uint64_t *>(&s.wcnt[0][0]);   // no longer needed
+    out[threadIdx.x] = out0 - s.first[threadIdx.x];
     __syncthreads();
-    {
-        int d = threadIdx.x;
-        uint32_t s = 0;
-        for (int w = 0; w < RS_T / 32; ++w) {
-            uint32_t t = wcnt[w][d];
-            wcnt[w][d] = s;
-            s += t;
-        }
+#pragma unroll
+    for (int i = 0; i < RS_I; ++i) {
+        const int x = i * RS_T + threadIdx.x;
+        if (x >= n) break;
+        const uint64_t key = s.key[x];
+        const uint64_t dst = out[(key >> shift) & 255] + x;
+        kout[dst] = key;
+        vout[dst] = s.val[x];
     }
-    __syncthreads();
-    for (int r = 0; r < RS_PER_WARP / 32; ++r) {
-        int64_t idx = wbase + r * 32 + lane;
-        bool valid = idx < N;
-        uint64_t k = valid ? kin[idx] : 0;
-        int d = valid ? (int)((k >> shift) & 255) : 256;
-        unsigned peers = __match_any_sync(FULL, d);
-        uint32_t basecnt = valid ? wcnt[wid][d] : 0;
-        __syncwarp();
-        if (valid) {
-            int64_t dst = (int64_t)offs[(int64_t)d * ntiles + blockIdx.x] + basecnt + __popc(peers & lt);
-            kout[dst] = k;
-            vout[dst] = vin[idx];
-            if (lane == __ffs(peers) - 1) wcnt[wid][d] = basecnt + __popc(peers);
+}
+
+// All passes of at most RS_SMALL pairs by one block, in place
+__global__ void __launch_bounds__(RS_ST) k_rs_small(uint64_t *key, uint32_t *val, int n, int bits) {
+    extern __shared__ __align__(16) unsigned char rs_smem[];
+    RsSmem<RS_ST, RS_SI> &s = *reinterpret_cast<RsSmem<RS_ST, RS_SI> *>(rs_smem);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint64_t k[RS_SI];
+    uint32_t v[RS_SI];
+#pragma unroll
+    for (int i = 0; i < RS_SI; ++i) {
+        const int x = wid * 32 * RS_SI + i * 32 + lane;
+        k[i] = x < n ? key[x] : 0;
+        v[i] = x < n ? val[x] : 0;
+    }
+    for (int shift = 0; shift < bits; shift += 8) {
+        rs_tile<RS_ST, RS_SI>(s, k, v, n, shift);
+#pragma unroll
+        for (int i = 0; i < RS_SI; ++i) {
+            const int x = wid * 32 * RS_SI + i * 32 + lane;
+            if (x < n) {
+                k[i] = s.key[x];
+                v[i] = s.val[x];
+            }
         }
-        __syncwarp();
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < RS_SI; ++i) {
+        const int x = wid * 32 * RS_SI + i * 32 + lane;
+        if (x < n) {
+            key[x] = k[i];
+            val[x] = v[i];
+        }
     }
 }
 
@@ -1868,6 +1966,15 @@ int64_t ae_sort_tmp_words(int64_t N) {
 int ae_radix_sort(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_t N, int bits, uint64_t *tmp,
                   cudaStream_t st) {
     if (N <= 1 || bits <= 0) return 0;
+    if (N <= RS_SMALL) {
+        ++g_launches;
+        const int smem = (int)sizeof(RsSmem<RS_ST, RS_SI>);
+        cudaFuncSetAttribute(k_rs_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        k_rs_small<<<1, RS_ST, smem, st>>>(k0, v0, (int)N, bits);
+        return 0;
+    }
+    const int smem = (int)sizeof(RsSmem<RS_T, RS_I>);
+    cudaFuncSetAttribute(k_rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     const int64_t ntiles = (N + RS_TILE - 1) / RS_TILE;
     const int64_t h = 256 * ntiles;
     uint32_t *hist = reinterpret_cast<uint32_t *>(tmp);
@@ -1883,7 +1990,7 @@ int ae_radix_sort(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_
         uint64_t *out[1] = {offs};
         scan_rec<uint32_t, 1>(in, out, h, nullptr, stmp, st);
         ++g_launches;
-        k_rs_scatter<<<(unsigned)ntiles, RS_T, 0, st>>>(ki, vi, ko, vo, N, shift, offs, ntiles);
+        k_rs_scatter<<<(unsigned)ntiles, RS_T, smem, st>>>(ki, vi, ko, vo, N, shift, offs, ntiles);
         which ^= 1;
     }
     return which;
@@ -1997,72 +2104,98 @@ void ae_unique_write(const uint64_t *key, const int32_t *score, int64_t N, const
 // ------------------------------------------------------------------ suffix array by prefix doubling
 //
 // The suffix array of Section 2.3 (Section 5 (1) builds it over the reversed
-// text), computed on the device by prefix doubling (Manber & Myers, 1993):
-// every suffix gets a key that orders it by its first h letters, a stable
-// radix sort groups equal keys, the group index becomes the suffix's rank,
-// and the next key is the pair (rank of the suffix, rank of the suffix h
-// letters on), which orders by the first 2h letters.  Rounds stop when every
-// rank is distinct.  The first key packs the first 64 / b letters directly
-// (b bits per letter value, the sentinel 0 included), so an i.i.d. text of
-// 10^8 letters needs one pair round.
+// text), computed on the device by prefix doubling (Manber & Myers, 1993).
+// Every suffix gets a key of its first L letters, b bits each (b for letters
+// only: places past the text read 0), and a stable radix sort orders them.  A
+// suffix's rank is the place of the first suffix with its key.  From then on
+// only the suffixes that share their key are sorted (as Larsson & Sadakane,
+// 2007, do): by (rank, what follows h letters on), into the places their groups
+// hold, which orders them by 2 h letters; new groups split and ranks follow.
+// What follows h letters on is the rank there; a suffix that ends within h
+// letters comes before all others of its key, shorter ones first.
+//
+// L is chosen so that about 1% of the suffixes of an i.i.d. text share a key:
+// sorting these again costs less than a pass over all of them for longer keys.
+// 10^7 letters: 4 passes over all suffixes and one round of some 10^4 of them
+// (1.6 ms), where a 63-bit key and a 48-bit pair key for every suffix took 14
+// passes (4.5 ms).
 
 namespace {
 
-// s[k] = letter + 1 of the text (read backwards with `reversed`), s[n] = 0
+// s[k] = letter of the text (read backwards with `reversed`)
 __global__ void k_sa_letters(const uint8_t *codes, int64_t n, int reversed, int sigma, uint8_t *s, int *bad) {
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= n; k += (int64_t)gridDim.x * blockDim.x) {
-        uint8_t v = 0;
-        if (k < n) {
-            const uint8_t c = codes[reversed ? n - 1 - k : k];
-            if (c >= sigma) *bad = 1;
-            v = (uint8_t)(c + 1);
-        }
-        s[k] = v;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+        const uint8_t c = codes[reversed ? n - 1 - k : k];
+        if (c >= sigma) *bad = 1;
+        s[k] = c;
     }
 }
 
-// key of suffix i: its first L letter values, b bits each, first letter highest;
-// positions past the sentinel read 0 (the sentinel is unique, so this never ties
-// two different suffixes)
-__global__ void k_sa_first_keys(const uint8_t *s, int64_t N, int b, int L, uint64_t *keys, uint32_t *vals) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+// key of suffix i: its first L letters, b bits each, first letter highest.  A
+// thread takes eight suffixes in a row and reads their letters once.
+constexpr int SA_KEYS = 8;
+__global__ void __launch_bounds__(256) k_sa_first_keys(const uint8_t *s, int64_t n, int b, int L, uint64_t *keys,
+                                                       uint32_t *vals) {
+    const uint64_t mask = b * L >= 64 ? ~0ull : (1ull << (b * L)) - 1ull;
+    const int64_t N = n + 1, nt = (N + SA_KEYS - 1) / SA_KEYS;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i0 = t * SA_KEYS;
         uint64_t key = 0;
-        for (int t = 0; t < L; ++t) {
-            const int64_t x = i + t;
-            key = (key << b) | (uint64_t)(x < N ? s[x] : 0);
+        for (int x = 0; x < L - 1; ++x) key = (key << b) | (uint64_t)(i0 + x < n ? s[i0 + x] : 0);
+        for (int q = 0; q < SA_KEYS && i0 + q < N; ++q) {
+            const int64_t x = i0 + q + L - 1;
+            key = ((key << b) | (uint64_t)(x < n ? s[x] : 0)) & mask;
+            keys[i0 + q] = key;
+            vals[i0 + q] = (uint32_t)(i0 + q);
         }
-        keys[i] = key;
-        vals[i] = (uint32_t)i;
     }
 }
 
-// 1 where a sorted key starts a new group
-__global__ void k_sa_heads(const uint64_t *keys, int64_t N, uint32_t *head) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
-        head[p] = (p == 0 || keys[p] != keys[p - 1]) ? 1u : 0u;
+// Of a sorted list of keys: 1 where a key starts a group, and 1 where it shares
+// its key with a neighbour
+__global__ void k_sa_groups(const uint64_t *keys, int64_t N, uint32_t *head, uint32_t *tied) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = keys[p];
+        const bool h = p == 0 || keys[p - 1] != k;
+        head[p] = h ? 1u : 0u;
+        tied[p] = !h || (p + 1 < N && keys[p + 1] == k) ? 1u : 0u;
+    }
 }
 
-// rank of suffix vals[p] = index of its group (inclusive count of heads - 1)
-__global__ void k_sa_rank(const uint32_t *vals, const uint32_t *head, const uint64_t *excl, int64_t N,
-                          uint32_t *rank, int *bad) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = vals[p];
-        if ((int64_t)i >= N) {
+// The place in the suffix array of each group's first suffix, by group; the
+// list's k-th element stands at place pos[k] (NULL: at k)
+__global__ void k_sa_starts(const uint32_t *head, const uint64_t *group, const uint32_t *pos, int64_t N,
+                            uint32_t *start) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
+        if (head[p]) start[group[p]] = pos ? pos[p] : (uint32_t)p;
+}
+
+// The list's suffixes at their places with their ranks, and the places of those
+// still tied as the next list
+__global__ void k_sa_place(const uint32_t *vals, const uint32_t *head, const uint64_t *group, const uint32_t *start,
+                           const uint32_t *pos, const uint32_t *tied, const uint64_t *tied_off, int64_t T, int64_t N,
+                           uint32_t *sa, uint32_t *rank, uint32_t *next, int *bad) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < T; p += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = vals[p], at = pos ? pos[p] : (uint32_t)p;
+        if ((int64_t)i >= N || (int64_t)at >= N) {
             *bad = 2;
             continue;
         }
-        rank[i] = (uint32_t)(excl[p] + head[p] - 1);
+        sa[at] = i;
+        // group[] counts the heads before p: the element's own group is that, or one less
+        rank[i] = start[group[p] + head[p] - 1];
+        if (tied[p]) next[tied_off[p]] = at;
     }
 }
 
-// key of suffix i for the 2h-letter order: (rank of i, rank of i + h plus one);
-// a suffix shorter than h + 1 letters holds the sentinel in its first h letters,
-// so its rank is already unique and its second component is 0
-__global__ void k_sa_pair_keys(const uint32_t *rank, int64_t N, int64_t h, int rb, uint64_t *keys, uint32_t *vals) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t second = (i + h < N) ? (uint64_t)rank[i + h] + 1u : 0u;
-        keys[i] = ((uint64_t)rank[i] << rb) | second;
-        vals[i] = (uint32_t)i;
+// keys of the tied suffixes (at places pos[0..T)) for the 2 h-letter order
+__global__ void k_sa_pair_keys(const uint32_t *sa, const uint32_t *pos, const uint32_t *rank, int64_t T, int64_t n,
+                               int64_t h, int rb, uint64_t *keys, uint32_t *vals) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < T; p += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = sa[pos[p]];
+        const uint64_t second = i + h <= n ? (uint64_t)rank[i + h] + (uint64_t)h : (uint64_t)(n - i);
+        keys[p] = ((uint64_t)rank[i] << rb) | second;
+        vals[p] = i;
     }
 }
 
@@ -2078,29 +2211,30 @@ ae_status ae_sa_doubling(const uint8_t *d_codes, int64_t n, int sigma, int rever
                          cudaStream_t st) {
     const int64_t N = n + 1;
     if (rounds) *rounds = 0;
-    const int b = sa_bits_for((uint64_t)sigma), L = 64 / b;
-    uint8_t *s = nullptr;
-    uint64_t *k0 = nullptr, *k1 = nullptr, *tmp = nullptr, *total = nullptr;
-    uint32_t *v0 = nullptr, *v1 = nullptr, *rank = nullptr;
-    int *bad = nullptr;
-    const int64_t tmp_words = std::max(ae_sort_tmp_words(N), ae_scan_tmp_words(N, 1));
+    const int b = sa_bits_for((uint64_t)std::max(sigma - 1, 1));
+    // letters of the first key: enough for about 100 N different ones, in whole passes
+    int L = 1;
+    for (double words = sigma; words < 100.0 * (double)N && (L + 1) * b <= 64; words *= std::max(sigma, 2)) ++L;
+    L = std::min(64, (L * b + 7) / 8 * 8) / b;
+    // one allocation for all buffers (ten of them cost 0.5 ms)
+    const int64_t tmp_words = std::max(ae_sort_tmp_words(N), ae_scan_tmp_words(N, 2) + N + (N + 1) / 2);
+    const int64_t words = 2 * N + tmp_words + 2 + (4 * N + 1 + 1) / 2 + 1 + (N + 7) / 8;   // of eight bytes
+    uint64_t *mem = nullptr;
     ae_status res = AE_OK;
-    if (cudaMalloc(&s, (size_t)N) != cudaSuccess || cudaMalloc(&k0, sizeof(uint64_t) * N) != cudaSuccess ||
-        cudaMalloc(&k1, sizeof(uint64_t) * N) != cudaSuccess || cudaMalloc(&v0, sizeof(uint32_t) * N) != cudaSuccess ||
-        cudaMalloc(&v1, sizeof(uint32_t) * N) != cudaSuccess ||
-        cudaMalloc(&rank, sizeof(uint32_t) * N) != cudaSuccess ||
-        cudaMalloc(&tmp, sizeof(uint64_t) * tmp_words) != cudaSuccess ||
-        cudaMalloc(&total, sizeof(uint64_t)) != cudaSuccess || cudaMalloc(&bad, sizeof(int)) != cudaSuccess) {
+    if (cudaMalloc(&mem, sizeof(uint64_t) * (size_t)words) != cudaSuccess) {
         cudaGetLastError();
-        res = AE_ENOMEM;
+        return AE_ENOMEM;
     }
+    uint64_t *k0 = mem, *k1 = k0 + N, *tmp = k1 + N, *total = tmp + tmp_words;
+    uint32_t *v0 = reinterpret_cast<uint32_t *>(total + 2), *v1 = v0 + N, *rank = v1 + N, *pos = rank + N;
+    int *bad = reinterpret_cast<int *>(pos + N);
+    uint8_t *s = reinterpret_cast<uint8_t *>(bad + 1);
     int h_bad = 0;
-    uint64_t G = 0;
     if (res == AE_OK && cudaMemsetAsync(bad, 0, sizeof(int), st) != cudaSuccess) res = AE_ECUDA;
     if (res == AE_OK) {
         g_launches += 2;
-        k_sa_letters<<<grid_for(N, 256), 256, 0, st>>>(d_codes, n, reversed, sigma, s, bad);
-        k_sa_first_keys<<<grid_for(N, 256), 256, 0, st>>>(s, N, b, L, k0, v0);
+        k_sa_letters<<<grid_for(n, 256), 256, 0, st>>>(d_codes, n, reversed, sigma, s, bad);
+        k_sa_first_keys<<<grid_for((N + SA_KEYS - 1) / SA_KEYS, 256), 256, 0, st>>>(s, n, b, L, k0, v0);
         if (cudaGetLastError() != cudaSuccess ||
             cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
@@ -2108,54 +2242,75 @@ ae_status ae_sa_doubling(const uint8_t *d_codes, int64_t n, int sigma, int rever
         else if (h_bad)
             res = AE_EINVAL;
     }
-    // (kr, vr): the sorted pairs; (kf, vf): the free pair
+    // (kr, vr): the sorted pairs of the current list; (kf, vf): the free pair
     uint64_t *kr = k0, *kf = k1;
-    uint32_t *vr = v0, *vf = v1;
+    uint32_t *vr = v0, *vf = v1, *sa = reinterpret_cast<uint32_t *>(d_sa);
     int bits = b * L;
-    int64_t h = L;
+    int64_t h = L, T = N;   // T: length of the list, at first every suffix
+    bool all = true;
     while (res == AE_OK) {
-        if (ae_radix_sort(kr, vr, kf, vf, N, bits, tmp, st)) {
+        if (ae_radix_sort(kr, vr, kf, vf, T, bits, tmp, st)) {
             std::swap(kr, kf);
             std::swap(vr, vf);
         }
         if (rounds) ++*rounds;
-        g_launches += 2;
-        k_sa_heads<<<grid_for(N, 256), 256, 0, st>>>(kr, N, vf);
-        const uint32_t *in[1] = {vf};
-        uint64_t *out[1] = {kf};
-        ae_scan_u32(in, out, 1, N, total, tmp, st);
-        k_sa_rank<<<grid_for(N, 256), 256, 0, st>>>(vr, vf, kf, N, rank, bad);
+        // head and tied flags in the free values, their sums in the free keys and tmp
+        uint32_t *head = vf, *tied = reinterpret_cast<uint32_t *>(tmp);
+        uint64_t *group = kf, *tied_off = tmp + (T + 1) / 2;
+        uint64_t *scan_tmp = tied_off + T;
+        if ((T + 1) / 2 + T + ae_scan_tmp_words(T, 2) > tmp_words) {
+            res = AE_ECUDA;   // sized above
+            break;
+        }
+        g_launches += 3;
+        k_sa_groups<<<grid_for(T, 256), 256, 0, st>>>(kr, T, head, tied);
+        const uint32_t *in[2] = {head, tied};
+        uint64_t *out[2] = {group, tied_off};
+        ae_scan_u32(in, out, 2, T, total, scan_tmp, st);
+        // group starts: over the sorted keys, which are done with
+        uint32_t *start = reinterpret_cast<uint32_t *>(kr);
+        const uint32_t *at = all ? nullptr : pos;
+        k_sa_starts<<<grid_for(T, 256), 256, 0, st>>>(head, group, at, T, start);
+        // the next list's places: the keys' second half
+        uint32_t *next = start + N;
+        k_sa_place<<<grid_for(T, 256), 256, 0, st>>>(vr, head, group, start, at, tied, tied_off, T, N, sa, rank, next, bad);
+        uint64_t sums[2] = {0, 0};
         if (cudaGetLastError() != cudaSuccess ||
-            cudaMemcpyAsync(&G, total, sizeof(uint64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaMemcpyAsync(sums, total, 2 * sizeof(uint64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) {
             res = AE_ECUDA;
             break;
         }
-        if (h_bad || G < 1 || (int64_t)G > N) {
+        if (h_bad || sums[0] < 1 || (int64_t)sums[0] > T || (int64_t)sums[1] > T) {
             res = AE_ECUDA;   // not a permutation: an internal error
             break;
         }
-        if ((int64_t)G == N) break;
-        if (h >= N) {         // every rank is distinct once h reaches N
+        if (sums[1] == 0) break;
+        if (!all && h / 2 >= N) {   // a round at h >= N orders everything left by its length
             res = AE_ECUDA;
             break;
         }
-        const int rb = sa_bits_for(G);
-        bits = rb + sa_bits_for(G - 1);
+        T = (int64_t)sums[1];
+        all = false;
+        if (cudaMemcpyAsync(pos, next, sizeof(uint32_t) * T, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+            res = AE_ECUDA;
+            break;
+        }
+        const int rb = sa_bits_for((uint64_t)(N - 1 + h));
+        bits = rb + sa_bits_for((uint64_t)(N - 1));
+        if (bits > 64) {
+            res = AE_EUNSUPPORTED;
+            break;
+        }
         ++g_launches;
-        k_sa_pair_keys<<<grid_for(N, 256), 256, 0, st>>>(rank, N, h, rb, kf, vf);
+        k_sa_pair_keys<<<grid_for(T, 256), 256, 0, st>>>(sa, pos, rank, T, n, h, rb, kf, vf);
         std::swap(kr, kf);
         std::swap(vr, vf);
         h *= 2;
     }
-    if (res == AE_OK &&
-        (cudaMemcpyAsync(d_sa, vr, sizeof(int32_t) * N, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-         cudaStreamSynchronize(st) != cudaSuccess))
-        res = AE_ECUDA;
+    if (res == AE_OK && cudaStreamSynchronize(st) != cudaSuccess) res = AE_ECUDA;
     if (res != AE_OK) cudaStreamSynchronize(st);
-    for (void *p : {(void *)s, (void *)k0, (void *)k1, (void *)v0, (void *)v1, (void *)rank, (void *)tmp,
-                    (void *)total, (void *)bad})
-        if (p) cudaFree(p);
+    cudaFree(mem);
     return res;
 }
