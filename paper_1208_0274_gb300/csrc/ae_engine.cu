@@ -851,14 +851,20 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 #define AE_LEAF_WIDE_POOL (1 << 22)
 #endif
 
-// Sweep tasks are cut at gaps of more than AE_LEAF_GAP text positions between
-// injections, as long as a query's injections lie at least half that far apart
-// on average over the text (denser ones leave too few gaps to cut at).  Cut at
-// multiples of 32 injections instead, each part of a homologous region walked on
-// to the region's end beside the others: 13 times the cells and hit records on
-// six homologous reads (sweep 100 ms against 17)
+// Sweep tasks are cut at gaps between injections of more than AE_LEAF_GAP text
+// positions, or one and a half times the average gap of the batch's queries
+// where that is less (a fifth of the gaps of randomly placed injections is
+// longer; along a homolog they lie every few positions).  Cut at multiples of 32
+// injections instead, each part of a homologous region walked on to the
+// region's end beside the others: 13 times the cells and hit records on six
+// homologous reads (sweep 100 ms against 17).  Injections closer than
+// AE_LEAF_DENSE positions on average (protein at low thresholds) leave no gaps
+// to cut at.
 #ifndef AE_LEAF_GAP
 #define AE_LEAF_GAP 64
+#endif
+#ifndef AE_LEAF_DENSE
+#define AE_LEAF_DENSE 4
 #endif
 
 // Levels of at most AE_WIDE_NODES nodes whose rows average AE_WIDE_ROW_AVG
@@ -1307,7 +1313,8 @@ void Search::leaf_phase(int64_t ninj) {
                                                                  : (int64_t)(ninj * w->hit_ratio) + 4096);
     // wide walks move to blocks (not inside the fixed arena of the no-allocation
     // entry point, nor when entries are counted by tier, which only the warp walk does)
-    const bool sparse = (double)ninj * (AE_LEAF_GAP / 2) <= (double)ix.n * batch_queries;
+    const double spacing = (double)ix.n * (double)batch_queries / (double)ninj;
+    const bool sparse = spacing >= AE_LEAF_DENSE;
     // the default chooses: where injections leave gaps the few wide walks set the
     // sweep's time, and a step on a block is faster from the first row past a warp's
     // lanes on (613 bp query: 0.76 ms from 32 entries, 0.79 from 64, 1.09 from 128);
@@ -1382,7 +1389,7 @@ void Search::leaf_phase(int64_t ninj) {
             la.wide_blocks = wide_blocks;
         }
         la.keys = keys;
-        la.gap = sparse ? AE_LEAF_GAP : 0;
+        la.gap = sparse ? (uint32_t)std::min<double>(AE_LEAF_GAP, 1.5 * spacing) : 0;
         prof.mark(K_LEAF);
         ++stats.leaf_sweeps;
         const auto t_sweep = std::chrono::steady_clock::now();

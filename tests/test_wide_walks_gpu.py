@@ -46,3 +46,31 @@ def test_block_walks_equal_warp_walks(lengths, div, H, scheme, opts):
         found += want.size
         idx.close()
     assert found > 0
+
+
+# Injections from a fortieth of the text's positions to most of them: tasks cut at
+# 64 positions, at one and a half average gaps, and not at all
+@pytest.mark.parametrize("m,queries", [(40, 1), (150, 1), (600, 1), (2_000, 1), (9_000, 1), (1_200, 5)])
+def test_task_cuts_by_spacing(m, queries):
+    import oracle
+    rng = np.random.default_rng(m)
+    T = iid_text(30_000, DNA, P, rng)
+    qs = []
+    for _ in range(queries):
+        q = iid_text(m, DNA, P, rng)
+        L = min(m - 10, 900)
+        s = int(rng.integers(0, T.size - L))
+        q[5:5 + L] = T[s:s + L]
+        qs.append(q)
+    idx = ae.ae_index_build(T, ae.AE_DNA)
+    sch = Scheme(1, -3, -5, -2)
+    got, counts = ae.ae_search(idx, qs, sch, 11)
+    idx.close()
+    at = 0
+    for q, c in zip(qs, counts):
+        i, j, s = oracle.sw_hits(T, q, sch, 11)
+        part = got[at:at + c]
+        at += int(c)
+        assert sorted(zip(part["text_end"].tolist(), part["query_end"].tolist(), part["score"].tolist())) == \
+            sorted(zip(np.asarray(i).tolist(), np.asarray(j).tolist(), np.asarray(s).tolist()))
+    assert at == got.size > 0
