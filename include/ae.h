@@ -174,8 +174,8 @@ typedef struct {
                                  entries continues on a whole thread block (each step spread over
                                  its threads) instead of one warp; 0: never.  The default, 128,
                                  lets the library choose: 32 where the injected rows leave gaps
-                                 along the text, 1,024 where they lie at most positions.  The
-                                 results are the same */
+                                 along the text, 1,024 (128 for the last walks) where they lie
+                                 at most positions.  The results are the same */
 } ae_options;
 
 /* Fill *opt with the defaults: qprefix_seed 1, leaf_segment 0, item_columns

@@ -867,6 +867,16 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 #define AE_LEAF_DENSE 4
 #endif
 
+// Row length at which a warp's walk moves to a block once the sweep's tasks are
+// all taken.  Dense injections make rows of hundreds of entries the rule, and
+// blocks walk those slower than the warps do together, so they take only the
+// widest (1,024) while there are tasks; then the warps run out of work and a
+// block shortens the walks that are left (protein batch: sweep 69 -> 58 ms; from 40
+// to 400 entries the same).
+#ifndef AE_LEAF_WIDE_TAIL
+#define AE_LEAF_WIDE_TAIL 128
+#endif
+
 // Levels of at most AE_WIDE_NODES nodes whose rows average AE_WIDE_ROW_AVG
 // entries or more give each node a whole block (k_rows_dna_wide)
 #ifndef AE_WIDE_NODES
@@ -1319,8 +1329,8 @@ void Search::leaf_phase(int64_t ninj) {
     // sweep's time, and a step on a block is faster from the first row past a warp's
     // lanes on (613 bp query: 0.76 ms from 32 entries, 0.79 from 64, 1.09 from 128);
     // where they are dense every task walks a wide row and warps are the better use of
-    // the chip (1 M residues, BLOSUM62: from 128 entries 153 ms, 512: 173, 1,024: 91,
-    // never: 103)
+    // the chip (1 M residues, BLOSUM62, sweep: from 128 entries 127 ms, 512: 104,
+    // 1,024: 69, never: 84), until the tasks run out (AE_LEAF_WIDE_TAIL)
     const int32_t wide = opt.leaf_wide_rows != 128 ? opt.leaf_wide_rows : sparse ? 32 : 1024;
     const int32_t esc_min = (g_arena || opt.tier_stats) ? 0 : wide;
     const int32_t esc_max = esc_min > 0 ? AE_LEAF_WIDE_SLOTS : 0;
@@ -1334,7 +1344,7 @@ void Search::leaf_phase(int64_t ninj) {
             ensure(w->esc, (size_t)esc_max * sizeof(EscWalk), st);
             ensure(w->esc_count, 24, st);
             ensure(w->esc_pool, (size_t)AE_LEAF_WIDE_POOL * 12, st);
-            ensure(w->wide_rows, (size_t)wide_blocks * 12 * (size_t)w->wide_cap * 4, st);
+            ensure(w->wide_rows, (size_t)wide_blocks * 6 * (size_t)w->wide_cap * 4, st);
             CU(cudaMemsetAsync(w->esc_count.p, 0, 24, st));
         }
         hits_reserve(hit_cap);
@@ -1378,6 +1388,7 @@ void Search::leaf_phase(int64_t ninj) {
         la.tiers = opt.tier_stats ? 1 : 0;
         la.stats = ptr<DevStats>(w->stats);
         la.esc_min = esc_max > 0 ? esc_min : 0;
+        la.esc_tail = std::min(la.esc_min, opt.leaf_wide_rows == 128 ? AE_LEAF_WIDE_TAIL : la.esc_min);
         la.esc_max = esc_max;
         if (esc_max > 0) {
             la.esc_count = ptr<unsigned long long>(w->esc_count);

@@ -489,14 +489,6 @@ __device__ __forceinline__ int64_t lower_bound_g(const int32_t *a, int64_t n, in
     }
     return lo;
 }
-__device__ __forceinline__ int64_t upper_bound_g(const int32_t *a, int64_t n, int32_t x) {
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        if (a[mid] <= x) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
 
 // Hit records of the sweep are staged per warp in shared memory and appended
 // to the global buffer LEAF_HS at a time, so that the walk along a homologous
@@ -595,38 +587,67 @@ __device__ __forceinline__ void make_slots(const ScoreView &sc, const int8_t *sm
     s.next_col = jn;
 }
 
-// Merge the rows injected at (qid, p) into the walked row Rn (nlen entries).  They are finished rows, and
-// the union of two finished rows taken by maximum per column is again
-// finished (each is closed under the horizontal-gap recurrence), so the
-// merge needs no second finish.  Cells where an injected row brings a
-// new or larger value report their hits here.
+// Merge the rows injected at (qid, p) into the walked row Rn (nlen entries), in
+// place.  They are finished rows, and the union of two finished rows taken by
+// maximum per column is again finished (each is closed under the horizontal-gap
+// recurrence), so the merge needs no second finish.  Cells where an injected row
+// brings a new or larger value report their hits here.
+//
+// Where most positions have an injection (protein at low thresholds) half of the
+// sweep's rows are merged, so the walked row is touched as little as possible: a
+// lane looks up one injected entry (the one search there is); columns both rows
+// have are raised where they stand; for new columns the entries behind the first
+// of them move up, 32 at a time from the row's end (each moves by the number of
+// new columns before it, so none is overwritten before it is read).
+// Against a merge through two copies of the row: protein, 5.1 M injections of 28
+// entries into rows of 130, sweep 89 -> 69 ms.
 // Used by the warp walk of k_leaf and, run by one warp, by the block walk of
 // k_leaf_wide.
 __device__ __forceinline__ void leaf_merge(const LeafArgs &a, int lane, int32_t qid, int32_t p, int32_t H,
-                                           uint64_t jmask, int64_t &k, int64_t kend, Buf &Rn, Buf &Cb, Buf &C2,
-                                           int64_t &nlen, int64_t cap, bool &overflow, HitStage &hstage,
-                                           unsigned long long &st_ent, unsigned long long &st_reused,
-                                           unsigned long long &st_t0) {
+                                           uint64_t jmask, int64_t &k, int64_t kend, const Buf &Rn, int64_t &nlen,
+                                           int64_t cap, bool &overflow, HitStage &hstage, unsigned long long &st_ent,
+                                           unsigned long long &st_reused, unsigned long long &st_t0) {
+    const unsigned lt = (1u << lane) - 1u;
+    const uint64_t kq = ((uint64_t)qid << (a.be + a.bj)) | ((uint64_t)(uint32_t)p << a.bj);
     while (k < kend) {
         const Inject I = a.inj[a.order[k]];
         if (I.qid != qid || I.e != p) break;
         ++k;
         const int32_t *ij = a.lj + I.off, *iM = a.lM + I.off, *iGa = a.lGa + I.off;
-        const int64_t icnt = I.cnt;
+        const int32_t icnt = (int32_t)I.cnt;
+        // the entry of this lane, its place in the walked row and the values there
+        int32_t n = (int32_t)nlen, y = 0, Mi = AE_NEG, Gi = AE_NEG, q = INT32_MAX, Mv = AE_NEG, Gv = AE_NEG;
+        bool same = false;
+        auto look = [&](int32_t idx) {
+            q = INT32_MAX;
+            same = false;
+            Mi = Gi = Mv = Gv = AE_NEG;
+            if (idx < icnt) {
+                y = ij[idx];
+                Mi = iM[idx];
+                Gi = iGa[idx];
+                int32_t lo = 0, hi = n;
+                while (lo < hi) {
+                    const int32_t mid = (lo + hi) >> 1;
+                    if (Rn.j[mid] < y) lo = mid + 1; else hi = mid;
+                }
+                q = lo;
+                same = q < n && Rn.j[q] == y;
+                if (same) {
+                    Mv = Rn.M[q];
+                    Gv = Rn.Ga[q];
+                }
+            }
+        };
         // an injected row whose every entry the walked row already has with
         // M and G_a at least as large changes nothing (its hits were reported
         // with the walked values): skip it.  Along a homologous region the row
         // walked from earlier starts usually dominates the later forks.
-        bool dominated = nlen > 0;
-        for (int64_t base = 0; dominated && base < icnt; base += 32) {
-            const int64_t idx = base + lane;
-            bool ok = true;
-            if (idx < icnt) {
-                const int32_t y = ij[idx];
-                const int64_t q = lower_bound_g(Rn.j, nlen, y);
-                ok = q < nlen && Rn.j[q] == y && Rn.M[q] >= iM[idx] && Rn.Ga[q] >= iGa[idx];
-            }
-            dominated = __all_sync(FULL, ok);
+        bool dominated = true;
+        int32_t at = 0;
+        for (; dominated && at < icnt; at += 32) {
+            look(at + lane);
+            dominated = __all_sync(FULL, at + lane >= icnt || (same && Mv >= Mi && Gv >= Gi));
         }
         if (dominated) {
             st_reused += (unsigned long long)icnt;   // the whole row rides on the walked one
@@ -636,81 +657,61 @@ __device__ __forceinline__ void leaf_merge(const LeafArgs &a, int lane, int32_t 
             overflow = true;
             break;
         }
-        for (int64_t base = 0; base < nlen; base += 32) {
-            const int64_t idx = base + lane;
-            if (idx < nlen) {
-                const int32_t x = Rn.j[idx];
-                const int64_t d = idx + lower_bound_g(ij, icnt, x);
-                C2.j[d] = x;
-                C2.M[d] = Rn.M[idx];
-                C2.Ga[d] = Rn.Ga[idx];
+        for (int32_t base = 0; base < icnt; base += 32) {
+            if (at != 32 || base) look(base + lane);   // (the first 32 may have been looked up just now)
+            const bool fresh = base + lane < icnt && !same;
+            const bool hit = Mi > Mv && Mi >= H;
+            if (same) {
+                if (Mi > Mv) Rn.M[q] = Mi;
+                if (Gi > Gv) Rn.Ga[q] = Gi;
             }
-        }
-        for (int64_t base = 0; base < icnt; base += 32) {
-            const int64_t idx = base + lane;
-            if (idx < icnt) {
-                const int32_t y = ij[idx];
-                const int64_t d = idx + upper_bound_g(Rn.j, nlen, y);
-                C2.j[d] = (int32_t)((uint32_t)y | 0x80000000u);   // tag: from the injected row
-                C2.M[d] = iM[idx];
-                C2.Ga[d] = iGa[idx];
-            }
-        }
-        __syncwarp();
-        // an equal column appears twice: the walked entry first, then the injected one
-        const int64_t len2 = nlen + icnt;
-        int64_t out = 0;
-        const uint64_t kq = ((uint64_t)qid << (a.be + a.bj)) | ((uint64_t)(uint32_t)p << a.bj);
-        for (int64_t base = 0; base < len2; base += 32) {
-            const int64_t idx = base + lane;
-            const bool valid = idx < len2;
-            int32_t j = 0, Mv = AE_NEG, Gv = AE_NEG;
-            bool keep = false, hit = false, fresh = false;
-            if (valid) {
-                const uint32_t raw = (uint32_t)C2.j[idx];
-                j = (int32_t)(raw & 0x7FFFFFFFu);
-                const bool from_inj = raw >> 31;
-                Mv = C2.M[idx];
-                Gv = C2.Ga[idx];
-                keep = !(idx > 0 && (int32_t)((uint32_t)C2.j[idx - 1] & 0x7FFFFFFFu) == j);
-                if (keep) {
-                    if (idx + 1 < len2 && (int32_t)((uint32_t)C2.j[idx + 1] & 0x7FFFFFFFu) == j) {
-                        const int32_t Mi = C2.M[idx + 1];
-                        hit = Mi > Mv && Mi >= H;
-                        Mv = max(Mv, Mi);
-                        Gv = max(Gv, C2.Ga[idx + 1]);
-                    } else {
-                        fresh = from_inj;
-                        hit = from_inj && Mv >= H;
-                    }
-                }
-            }
-            const uint32_t ci = warp_incl_sum(keep ? 1u : 0u);
-            const uint32_t tot = __shfl_sync(FULL, ci, 31);
-            const uint32_t hi = warp_incl_sum(hit ? 1u : 0u);
-            const uint32_t htot = __shfl_sync(FULL, hi, 31);
+            const unsigned bf = __ballot_sync(FULL, fresh), bh = __ballot_sync(FULL, hit);
             __syncwarp();
-            if (keep) {
-                const int64_t d = out + ci - 1;
-                Cb.j[d] = j;
-                Cb.M[d] = Mv;
-                Cb.Ga[d] = Gv;
+            if (bf) {
+                const int32_t first = __shfl_sync(FULL, q, __ffs(bf) - 1);
+                for (int32_t c = (n - 1) & ~31; n > 0 && c >= (first & ~31); c -= 32) {
+                    const int32_t x = c + lane;
+                    const bool moves = x >= first && x < n;
+                    int32_t vj = 0, vM = 0, vG = 0;
+                    if (moves) {
+                        vj = Rn.j[x];
+                        vM = Rn.M[x];
+                        vG = Rn.Ga[x];
+                    }
+                    int t = 0;   // injected entries with a place at or before x (places do not decrease)
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1)
+                        if (__shfl_sync(FULL, q, t + step - 1) <= x) t += step;
+                    if (__shfl_sync(FULL, q, t) <= x) ++t;
+                    const int32_t d = x + __popc(bf & (t < 32 ? (1u << t) - 1u : ~0u));
+                    __syncwarp();
+                    if (moves) {
+                        Rn.j[d] = vj;
+                        Rn.M[d] = vM;
+                        Rn.Ga[d] = vG;
+                    }
+                    __syncwarp();
+                }
+                if (fresh) {
+                    const int32_t d = q + __popc(bf & lt);
+                    Rn.j[d] = y;
+                    Rn.M[d] = Mi;
+                    Rn.Ga[d] = Gi;
+                }
+                n += __popc(bf);
+                if (a.tiers && fresh) ++st_t0;
             }
-            if (htot) {
+            if (bh) {
                 bool staged, hok;
-                const uint64_t hbase = stage_reserve(hstage, a, lane, htot, staged, hok);
-                if (hok && hit) hit_put(hstage, a, staged, hbase + hi - 1, kq | ((uint64_t)j & jmask), Mv);
+                const uint64_t hbase = stage_reserve(hstage, a, lane, __popc(bh), staged, hok);
+                if (hok && hit)
+                    hit_put(hstage, a, staged, hbase + __popc(bh & lt), kq | ((uint64_t)y & jmask), Mi);
             }
-            if (a.tiers && fresh) ++st_t0;
-            out += tot;
+            __syncwarp();
         }
-        __syncwarp();
-        st_ent += (unsigned long long)(out - nlen);
-        st_reused += (unsigned long long)(nlen + icnt - out);   // columns both rows had
-        Buf t = Rn;
-        Rn = Cb;
-        Cb = t;
-        nlen = out;
+        st_ent += (unsigned long long)(n - nlen);
+        st_reused += (unsigned long long)(icnt - (n - nlen));   // columns both rows had
+        nlen = n;
     }
 }
 
@@ -739,11 +740,6 @@ __device__ __forceinline__ int64_t task_start(const LeafArgs &a, int lane, int64
     return end == a.ninj ? a.ninj : k0;
 }
 
-#ifndef AE_LEAF_E
-#define AE_LEAF_E 2
-#endif
-constexpr int LEAF_E = AE_LEAF_E;   // row entries per lane in the wide sweep step
-
 // One warp per segment of `seg` consecutive injections (sorted by query and
 // text end).  The warp carries a row R along text positions p, p+1, ...:
 //   candidates of row p+1 = the vertical and diagonal slots generated from R
@@ -754,10 +750,15 @@ constexpr int LEAF_E = AE_LEAF_E;   // row entries per lane in the wide sweep st
 // sets leaf_overflow and the host reruns with a larger cap.
 // A walk whose row grows past esc_min entries is handed on, with the rest of
 // its segment, to a slot of k_leaf_wide (a block of threads per walk); when
-// the slots are taken the warp carries on itself.  The remaining warp walks
-// run fastest with registers to spare: 3 resident blocks per SM (measured).
+// the slots are taken the warp carries on itself.
+// A step is a chain of scans and dependent loads, so the resident warps set the
+// rate: 6 blocks per SM at one entry per lane (80 registers, a few spilled)
+// against 3 at two entries (162 registers, 38 % of the issue slots used; 526
+// warp instructions per 32 entries).  Sweeps of a protein batch, a 1 M-letter query
+// and a batch with cheap gaps: 51.7 / 22.9 / 11.3 ms against 58.5 / 28.8 / 16.1
+// (4 blocks 53.3 / 24.6 / 12.7; 8 blocks 53.2 / - / 11.3).
 #ifndef AE_LEAF_MINB
-#define AE_LEAF_MINB 3
+#define AE_LEAF_MINB 6
 #endif
 __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
     __shared__ int8_t smat[AE_MAX_SIGMA * AE_MAX_SIGMA];
@@ -772,14 +773,13 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
     const ScoreView &sc = a.sc;
     const int32_t u = -sc.ss, oe = sc.sg + sc.ss, g = sc.gmax;
     const int64_t cap = a.cap;
-    int32_t *wb = a.scratch + (int64_t)gw * 12 * cap;
+    int32_t *wb = a.scratch + (int64_t)gw * 6 * cap;
     Buf R = {wb, wb + cap, wb + 2 * cap};
     Buf Rn = {wb + 3 * cap, wb + 4 * cap, wb + 5 * cap};
-    Buf Cb = {wb + 6 * cap, wb + 7 * cap, wb + 8 * cap};
-    Buf C2 = {wb + 9 * cap, wb + 10 * cap, wb + 11 * cap};
     const uint64_t jmask = (1ull << a.bj) - 1ull;
     unsigned long long st_rows = 0, st_ent = 0, st_t0 = 0, st_t1 = 0, st_t2 = 0, st_reused = 0;
     bool overflow = false;
+    int32_t esc_at = a.esc_min;
 
     while (!overflow) {
         unsigned long long s = 0;
@@ -1045,77 +1045,49 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
                 }
                 const int c = (int)__shfl_sync(FULL, tw, (int)(p - tw_base));
                 // ---- slots from R with letter c and the horizontal finish, straight
-                // into Rn (the finished row at p) with its hits.  Each lane takes
-                // LEAF_E consecutive entries (a lane-local prefix, then one warp scan
-                // per quantity), so a wide row needs LEAF_E times fewer warp steps.
+                // into Rn (the finished row at p) with its hits
                 int32_t carry = AE_KNEG, prev_j = -2, prev_M = AE_NEG;
                 // the next chunk's entries are loaded while this chunk is computed
-                int32_t nj[LEAF_E], nM[LEAF_E], nG[LEAF_E];
-#pragma unroll
-                for (int e = 0; e < LEAF_E; ++e) {
-                    const int64_t x = (int64_t)lane * LEAF_E + e;
-                    const bool v = x < rlen;
-                    nj[e] = v ? R.j[x] : m;
-                    nM[e] = v ? R.M[x] : AE_NEG;
-                    nG[e] = v ? R.Ga[x] : AE_NEG;
-                }
-                for (int64_t base = 0; base < rlen; base += 32 * LEAF_E) {
-                    const int64_t i0 = base + (int64_t)lane * LEAF_E;
-                    int32_t jj[LEAF_E], MM[LEAF_E], GG[LEAF_E];
-#pragma unroll
-                    for (int e = 0; e < LEAF_E; ++e) {
-                        jj[e] = nj[e];
-                        MM[e] = nM[e];
-                        GG[e] = nG[e];
-                        const int64_t x = i0 + 32 * LEAF_E + e;
+                int32_t nj = lane < rlen ? R.j[lane] : m, nM = lane < rlen ? R.M[lane] : AE_NEG,
+                        nG = lane < rlen ? R.Ga[lane] : AE_NEG;
+                for (int64_t base = 0; base < rlen; base += 32) {
+                    const int64_t i0 = base + lane;
+                    const bool valid = i0 < rlen;
+                    const int32_t j = nj, M = nM, G = nG;
+                    {
+                        const int64_t x = i0 + 32;
                         const bool v = x < rlen;
-                        nj[e] = v ? R.j[x] : m;
-                        nM[e] = v ? R.M[x] : AE_NEG;
-                        nG[e] = v ? R.Ga[x] : AE_NEG;
+                        nj = v ? R.j[x] : m;
+                        nM = v ? R.M[x] : AE_NEG;
+                        nG = v ? R.Ga[x] : AE_NEG;
                     }
                     // the first entry of the next chunk (lane 0's next load), m past the row
-                    int32_t jnext = __shfl_down_sync(FULL, jj[0], 1);
-                    const int32_t jfirst_next = __shfl_sync(FULL, nj[0], 0);
-                    if (lane == 31) jnext = jfirst_next;
-                    int32_t pj0 = __shfl_up_sync(FULL, jj[LEAF_E - 1], 1), pM0 = __shfl_up_sync(FULL, MM[LEAF_E - 1], 1);
+                    int32_t jn = __shfl_down_sync(FULL, j, 1);
+                    const int32_t jfirst_next = __shfl_sync(FULL, nj, 0);
+                    if (lane == 31) jn = jfirst_next;
+                    if (i0 + 1 >= rlen) jn = m;
+                    int32_t pj = __shfl_up_sync(FULL, j, 1), pM = __shfl_up_sync(FULL, M, 1);
                     if (lane == 0) {
-                        pj0 = prev_j;
-                        pM0 = prev_M;
+                        pj = prev_j;
+                        pM = prev_M;
                     }
-                    Slots sl[LEAF_E];
-                    int32_t lk[LEAF_E];
-#pragma unroll
-                    for (int e = 0; e < LEAF_E; ++e) {
-                        const bool v = i0 + e < rlen;
-                        int32_t jn = (e + 1 < LEAF_E) ? jj[e + 1] : jnext;
-                        if (i0 + e + 1 >= rlen) jn = m;
-                        const int32_t pj = e ? jj[e - 1] : pj0, pM = e ? MM[e - 1] : pM0;
-                        make_slots(sc, smat, c, P, m, H, g, oe, v, jj[e], MM[e], GG[e], pj, pM, jn, sl[e]);
-                        const int32_t keyA = sl[e].MpA > AE_NEG ? sl[e].MpA + sl[e].colA * u : AE_KNEG;
-                        const int32_t keyB = sl[e].MpB > AE_NEG ? sl[e].MpB + (sl[e].colA + 1) * u : AE_KNEG;
-                        lk[e] = max(e ? lk[e - 1] : AE_KNEG, max(keyA, keyB));
-                    }
-                    int32_t lincl = warp_incl_max(lk[LEAF_E - 1]);
-                    int32_t lexcl = __shfl_up_sync(FULL, lincl, 1);
-                    if (lane == 0) lexcl = AE_KNEG;
-                    lincl = max(lincl, carry);
-                    lexcl = max(lexcl, carry);
-                    SlotOut o[LEAF_E];
-                    int32_t ik[LEAF_E];
-                    uint32_t cl = 0, hl = 0;
-#pragma unroll
-                    for (int e = 0; e < LEAF_E; ++e) {
-                        const int32_t ex = e ? max(lexcl, lk[e - 1]) : lexcl;
-                        ik[e] = max(lexcl, lk[e]);
-                        slot_finish(sl[e].colA, sl[e].MpA, sl[e].hasB, sl[e].MpB, sl[e].next_col, ex, ik[e], sc, m, H,
-                                    u, i0 + e < rlen, o[e]);
-                        cl += (uint32_t)o[e].aliveA + (uint32_t)o[e].aliveB + (uint32_t)o[e].run_len;
-                        hl += (uint32_t)(o[e].aliveA && o[e].MA >= H) + (uint32_t)(o[e].aliveB && o[e].MB >= H) +
-                              (uint32_t)o[e].run_hits;
-                    }
-                    carry = __shfl_sync(FULL, lincl, 31);
-                    prev_j = __shfl_sync(FULL, jj[LEAF_E - 1], 31);
-                    prev_M = __shfl_sync(FULL, MM[LEAF_E - 1], 31);
+                    Slots sl;
+                    make_slots(sc, smat, c, P, m, H, g, oe, valid, j, M, G, pj, pM, jn, sl);
+                    const int32_t keyA = sl.MpA > AE_NEG ? sl.MpA + sl.colA * u : AE_KNEG;
+                    const int32_t keyB = sl.MpB > AE_NEG ? sl.MpB + (sl.colA + 1) * u : AE_KNEG;
+                    int32_t incl = warp_incl_max(max(keyA, keyB));
+                    int32_t excl = __shfl_up_sync(FULL, incl, 1);
+                    if (lane == 0) excl = AE_KNEG;
+                    incl = max(incl, carry);
+                    excl = max(excl, carry);
+                    SlotOut o;
+                    slot_finish(sl.colA, sl.MpA, sl.hasB, sl.MpB, sl.next_col, excl, incl, sc, m, H, u, valid, o);
+                    const uint32_t nA = o.aliveA, nB = o.aliveB, nR = (uint32_t)o.run_len;
+                    const uint32_t hA = o.aliveA && o.MA >= H, hB = o.aliveB && o.MB >= H;
+                    const uint32_t cl = nA + nB + nR, hl = hA + hB + (uint32_t)o.run_hits;
+                    carry = __shfl_sync(FULL, incl, 31);
+                    prev_j = __shfl_sync(FULL, j, 31);
+                    prev_M = __shfl_sync(FULL, M, 31);
                     const uint32_t ci = warp_incl_sum(cl);
                     const uint32_t tot = __shfl_sync(FULL, ci, 31);
                     if (nlen + tot > cap) {
@@ -1128,64 +1100,47 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
                     uint64_t hbase = 0;
                     if (htot) hbase = stage_reserve(hstage, a, lane, htot, staged, hok);
                     const uint64_t kq = ((uint64_t)qid << (a.be + a.bj)) | ((uint64_t)(uint32_t)p << a.bj);
-                    int64_t eo = nlen + (int64_t)(ci - cl);
-                    uint64_t ho = hbase + hi - hl;
-                    int64_t run_d[LEAF_E];
-                    uint64_t run_h[LEAF_E];
-#pragma unroll
-                    for (int e = 0; e < LEAF_E; ++e) {
-                        const uint32_t nA = o[e].aliveA, nB = o[e].aliveB;
-                        const uint32_t hA = o[e].aliveA && o[e].MA >= H, hB = o[e].aliveB && o[e].MB >= H;
-                        const int32_t colA = sl[e].colA;
-                        if (o[e].aliveA) {
-                            Rn.j[eo] = colA;
-                            Rn.M[eo] = o[e].MA;
-                            Rn.Ga[eo] = sl[e].GaA;
-                            if (hA && hok) hit_put(hstage, a, staged, ho, kq | ((uint64_t)colA & jmask), o[e].MA);
-                            if (a.tiers) {
-                                const int tier = (sl[e].Dp > AE_NEG) + (sl[e].GaA > AE_NEG) +
-                                                 (o[e].GbA > thr_of(colA, m, H, g));
-                                st_t0 += tier <= 1;
-                                st_t1 += tier == 2;
-                                st_t2 += tier >= 3;
-                            }
+                    const int64_t eo = nlen + (int64_t)(ci - cl);
+                    const uint64_t ho = hbase + hi - hl;
+                    if (nA) {
+                        Rn.j[eo] = j;
+                        Rn.M[eo] = o.MA;
+                        Rn.Ga[eo] = sl.GaA;
+                        if (hA && hok) hit_put(hstage, a, staged, ho, kq | ((uint64_t)j & jmask), o.MA);
+                        if (a.tiers) {
+                            const int tier = (sl.Dp > AE_NEG) + (sl.GaA > AE_NEG) + (o.GbA > thr_of(j, m, H, g));
+                            st_t0 += tier <= 1;
+                            st_t1 += tier == 2;
+                            st_t2 += tier >= 3;
                         }
-                        if (o[e].aliveB) {
-                            Rn.j[eo + nA] = colA + 1;
-                            Rn.M[eo + nA] = o[e].MB;
-                            Rn.Ga[eo + nA] = AE_NEG;
-                            if (hB && hok)
-                                hit_put(hstage, a, staged, ho + hA, kq | ((uint64_t)(colA + 1) & jmask), o[e].MB);
-                            if (a.tiers) {
-                                if ((sl[e].Dk > AE_NEG) && (o[e].GbB > thr_of(colA + 1, m, H, g))) ++st_t1; else ++st_t0;
-                            }
-                        }
-                        if (a.tiers) st_t0 += (uint32_t)o[e].run_len;
-                        run_d[e] = eo + nA + nB;
-                        run_h[e] = ho + hA + hB;
-                        eo += nA + nB + (uint32_t)o[e].run_len;
-                        ho += hA + hB + (uint32_t)o[e].run_hits;
                     }
-#pragma unroll
-                    for (int e = 0; e < LEAF_E; ++e) {
-                        unsigned rmask = __ballot_sync(FULL, o[e].run_len > 0);
-                        while (rmask) {
-                            const int L = __ffs(rmask) - 1;
-                            rmask &= rmask - 1;
-                            const int32_t s0 = __shfl_sync(FULL, o[e].run_start, L);
-                            const int32_t rl = __shfl_sync(FULL, o[e].run_len, L);
-                            const int32_t rh = __shfl_sync(FULL, o[e].run_hits, L);
-                            const int32_t K = __shfl_sync(FULL, ik[e], L);
-                            const int64_t d0 = __shfl_sync(FULL, run_d[e], L);
-                            const uint64_t hd = __shfl_sync(FULL, run_h[e], L);
-                            for (int32_t t = lane; t < rl; t += 32) {
-                                const int32_t cc = s0 + t;
-                                const int32_t v = sc.sg - cc * u + K;
-                                Rn.j[d0 + t] = cc;
-                                Rn.M[d0 + t] = v;
-                                Rn.Ga[d0 + t] = AE_NEG;
-                                if (t < rh && hok) hit_put(hstage, a, staged, hd + t, kq | ((uint64_t)cc & jmask), v);
-                            }
+                    if (nB) {
+                        Rn.j[eo + nA] = j + 1;
+                        Rn.M[eo + nA] = o.MB;
+                        Rn.Ga[eo + nA] = AE_NEG;
+                        if (hB && hok) hit_put(hstage, a, staged, ho + hA, kq | ((uint64_t)(j + 1) & jmask), o.MB);
+                        if (a.tiers) {
+                            if ((sl.Dk > AE_NEG) && (o.GbB > thr_of(j + 1, m, H, g))) ++st_t1; else ++st_t0;
+                        }
+                    }
+                    if (a.tiers) st_t0 += nR;
+                    unsigned rmask = __ballot_sync(FULL, nR > 0);
+                    while (rmask) {
+                        const int L = __ffs(rmask) - 1;
+                        rmask &= rmask - 1;
+                        const int32_t s0 = __shfl_sync(FULL, o.run_start, L);
+                        const int32_t rl = __shfl_sync(FULL, o.run_len, L);
+                        const int32_t rh = __shfl_sync(FULL, o.run_hits, L);
+                        const int32_t K = __shfl_sync(FULL, incl, L);
+                        const int64_t d0 = __shfl_sync(FULL, eo + nA + nB, L);
+                        const uint64_t hd = __shfl_sync(FULL, ho + hA + hB, L);
+                        for (int32_t t = lane; t < rl; t += 32) {
+                            const int32_t cc = s0 + t;
+                            const int32_t v = sc.sg - cc * u + K;
+                            Rn.j[d0 + t] = cc;
+                            Rn.M[d0 + t] = v;
+                            Rn.Ga[d0 + t] = AE_NEG;
+                            if (t < rh && hok) hit_put(hstage, a, staged, hd + t, kq | ((uint64_t)cc & jmask), v);
                         }
                     }
                     nlen += tot;
@@ -1194,8 +1149,7 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
                 if (overflow) break;
                 st_ent += (unsigned long long)nlen;
             }
-            leaf_merge(a, lane, qid, p, H, jmask, k, kend, Rn, Cb, C2, nlen, cap, overflow, hstage, st_ent, st_reused,
-                       st_t0);
+            leaf_merge(a, lane, qid, p, H, jmask, k, kend, Rn, nlen, cap, overflow, hstage, st_ent, st_reused, st_t0);
             if (overflow) break;
             if (k < kend) {
                 const Inject In = a.inj[a.order[k]];
@@ -1211,7 +1165,12 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
             ++st_rows;
             ++seg_steps;
             seg_width = max(seg_width, (unsigned long long)nlen);
-            if (a.esc_min > 0 && rlen > a.esc_min) {
+            // once every task is taken, warps fall idle while the last wide walks go on, and
+            // a block each is the better use of the chip from narrower rows on
+            if (rlen > a.esc_tail && esc_at != a.esc_tail && (seg_steps & 7) == 0 &&
+                *(volatile unsigned long long *)a.next_seg >= (unsigned long long)a.nseg)
+                esc_at = a.esc_tail;
+            if (esc_at > 0 && rlen > esc_at) {
                 // a wide row goes on on a whole block (k_leaf_wide), with the rest of
                 // this task's injections; the warp takes its next task
                 unsigned long long slot = 0, at = 0;
@@ -1338,7 +1297,7 @@ struct __align__(16) WideSmem {
     int32_t mq[32], mM[32], mG[32];      // a merge: place in the row (new entries: ~place), values
     unsigned long long walk, hbase;
     int64_t nlen;
-    int32_t swapped, overflow;
+    int32_t overflow;
     int8_t mat[AE_MAX_SIGMA * AE_MAX_SIGMA];
 };
 
@@ -1394,8 +1353,8 @@ __global__ void __launch_bounds__(WIDE_T, 1) k_leaf_wide(LeafArgs a) {
     const ScoreView &sc = a.sc;
     const int32_t u = -sc.ss, oe = sc.sg + sc.ss, g = sc.gmax;
     const uint64_t jmask = (1ull << a.bj) - 1ull;
-    int32_t *eb = a.wide_rows + (int64_t)blockIdx.x * 12 * a.wide_cap;
-    // buffers 0 and 1: the rows in shared memory; 2 to 5: in global memory
+    int32_t *eb = a.wide_rows + (int64_t)blockIdx.x * 6 * a.wide_cap;
+    // buffers 0 and 1: the rows in shared memory; 2 and 3: in global memory
     auto buf = [&](int x) {
         if (x < 2) return Buf{s.j[x], s.M[x], s.G[x]};
         int32_t *b = eb + (int64_t)(x - 2) * 3 * a.wide_cap;
@@ -1789,16 +1748,13 @@ __global__ void __launch_bounds__(WIDE_T, 1) k_leaf_wide(LeafArgs a) {
                         __syncthreads();
                     }
                     if (wid == 0) {
-                        Buf A = buf(nxt), Cb = buf(4), C2 = buf(5);
-                        int32_t *const was = A.j;
                         bool ovf = nxt < 2;   // longer than the buffers: reported
                         int64_t kk = k, nl = nlen;
                         if (!ovf)
-                            leaf_merge(a, lane, qid, p, H, jmask, kk, k + 1, A, Cb, C2, nl, (int64_t)a.wide_cap, ovf, mstage,
+                            leaf_merge(a, lane, qid, p, H, jmask, kk, k + 1, buf(nxt), nl, (int64_t)a.wide_cap, ovf, mstage,
                                        st_ent, st_reused, st_t0);
                         if (lane == 0) {
                             s.nlen = nl;
-                            s.swapped = A.j != was;
                             if (ovf) s.overflow = 1;
                         }
                     }
@@ -1808,7 +1764,6 @@ __global__ void __launch_bounds__(WIDE_T, 1) k_leaf_wide(LeafArgs a) {
                         break;
                     }
                     nlen = s.nlen;
-                    if (s.swapped) wide_copy(buf(nxt), buf(4), nlen);
                     __syncthreads();
                 }
                 __syncthreads();   // the ring's flags are read before the next group's are written
@@ -2048,7 +2003,7 @@ void ae_inject_keys(const Inject *inj, int64_t ninj, uint64_t *keys, uint32_t *v
 
 int ae_leaf_wide_blocks_per_sm() { return 1; }
 
-int64_t ae_leaf_scratch_words(int32_t cap, int32_t nwarps) { return (int64_t)12 * cap * nwarps; }
+int64_t ae_leaf_scratch_words(int32_t cap, int32_t nwarps) { return (int64_t)6 * cap * nwarps; }
 
 void ae_leaf_sweep(const LeafArgs &a, int blocks, int threads, cudaStream_t st) {
     if (a.nseg <= 0) return;

@@ -74,3 +74,27 @@ def test_task_cuts_by_spacing(m, queries):
         assert sorted(zip(part["text_end"].tolist(), part["query_end"].tolist(), part["score"].tolist())) == \
             sorted(zip(np.asarray(i).tolist(), np.asarray(j).tolist(), np.asarray(s).tolist()))
     assert at == got.size > 0
+
+
+# Rows injected at most positions and merged into the walked row: rows of more than
+# 32 entries, buffers grown from the smallest capacity, warps alone and blocks
+@pytest.mark.parametrize("m,opts", [
+    (150, dict(leaf_wide_rows=0, leaf_capacity=64)),
+    (1_500, dict(leaf_wide_rows=0)),
+    (1_500, dict(leaf_wide_rows=20, leaf_capacity=64)),
+    (4_000, dict(leaf_delay=0)),
+    (4_000, dict(leaf_wide_rows=40, leaf_segment=7)),
+])
+def test_merged_rows(m, opts):
+    import oracle
+    rng = np.random.default_rng(m)
+    T, q = iid_text(3_000, DNA, P, rng), iid_text(m, DNA, P, rng)
+    q[20:120] = T[-100:]
+    sch = Scheme(2, -3, -2, -1)
+    i, j, s = oracle.sw_hits(T, q, sch, 16)
+    idx = ae.ae_index_build(T, ae.AE_DNA)
+    got, counts = ae.ae_search(idx, [q], sch, 16, options=ae.make_options(**opts))
+    st = ae.ae_last_stats()
+    idx.close()
+    assert st["injections"] > 0 and st["reused"] > 0
+    assert np.array_equal(got["text_end"], i) and np.array_equal(got["query_end"], j) and np.array_equal(got["score"], s)
