@@ -35,7 +35,7 @@ constexpr int NORM_XMU = 0, NORM_XISD = NIN, NORM_YMU = 2 * NIN, NORM_YSD = 2 * 
 // B(k, n) = B[k*sbk + n*sbn] (fp32 in memory, rounded to bf16 for the
 // product, fp32 accumulate).  Epilogue per element: + bias[n]; Z = that value
 // (pre-activation); zeroed where mask <= 0; relu; stored to C (ld ldc).  One
-// warp owns a 16 x 32 tile (four m16n8k16 products per k step of 16).
+// warp owns a 16 x 16 tile (two m16n8k16 products per k step of 16).
 //
 // Split K: the weight gradients are products with a small output (at most
 // 128 x 128) and K = the batch rows, which a few warps would walk alone.  With
@@ -45,10 +45,10 @@ constexpr int NORM_XMU = 0, NORM_XISD = NIN, NORM_YMU = 2 * NIN, NORM_YSD = 2 * 
 // scheduling.
 //
 // A training step of 64 rows is a chain of small products, each bound by the
-// latency of its loads and its launch.  The next k step's operands are loaded
-// while this one's products run, and products that wait for the same input share
-// a launch (two GemmArgs): a step takes 9 launches instead of 17 (32 steps with
-// features, forward and gradients 5.95 -> 2.93 ms with the split of k_features).
+// latency of its loads and its launch.  So a warp loads GEMM_KU k steps' operands
+// together, its tile is small (more warps), and products that wait for the same
+// input share a launch (two GemmArgs), 9 launches a step instead of 17: 82 us a
+// step with one k step in flight and 16 x 32 tiles, 59 us so.
 
 struct GemmArgs {
     const float *A;
@@ -69,7 +69,8 @@ struct GemmPair {
     GemmArgs a[2];
 };
 
-constexpr int GEMM_NT = 4;      // n8 sub-tiles per warp
+constexpr int GEMM_NT = 2;      // n8 sub-tiles per warp
+constexpr int GEMM_KU = 4;      // k steps whose operands are loaded together
 constexpr int GEMM_WARPS = 4;
 constexpr int GEMM_KSPLIT_MAX = 64;
 constexpr int GEMM_TARGET_BLOCKS = 2 * 152;
@@ -92,7 +93,7 @@ __global__ void __launch_bounds__(GEMM_WARPS * 32) k_gemm(GemmPair pr) {
     const int g = lane >> 2, t = lane & 3;
     const int nb0 = pr.a[0].blocks * pr.a[0].nsplit;
     const bool second = (int)blockIdx.x >= nb0;
-    const GemmArgs &a = pr.a[second];
+    const GemmArgs a = second ? pr.a[1] : pr.a[0];
     const int block = (int)blockIdx.x - (second ? nb0 : 0), chunk = block / a.blocks;
     const int64_t tiles_n = (a.N + 8 * GEMM_NT - 1) / (8 * GEMM_NT);
     const int64_t tiles_m = (a.M + 15) / 16;
@@ -100,39 +101,55 @@ __global__ void __launch_bounds__(GEMM_WARPS * 32) k_gemm(GemmPair pr) {
     if (tile >= tiles_m * tiles_n) return;
     const int m0 = (int)(tile / tiles_n) * 16, n0 = (int)(tile % tiles_n) * 8 * GEMM_NT;
     const int kbeg = chunk * a.kchunk, kend = min(a.K, kbeg + a.kchunk);
-    auto ldA = [&](int m, int k) -> float {
-        return (m < a.M && k < kend) ? a.A[(int64_t)m * a.sam + (int64_t)k * a.sak] : 0.f;
-    };
-    auto ldB = [&](int k, int n) -> float {
-        return (k < kend && n < a.N) ? a.B[(int64_t)k * a.sbk + (int64_t)n * a.sbn] : 0.f;
-    };
     float acc[GEMM_NT][4];
 #pragma unroll
     for (int j = 0; j < GEMM_NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
     // A fragment (16 x 16, row major): rows g and g+8, columns 2t, 2t+1 and 2t+8, 2t+9;
-    // B fragment (16 x 8, column major): rows 2t, 2t+1 and 2t+8, 2t+9 of column g
-    float fa[8], fb[GEMM_NT][4];
-    auto load = [&](int k0) {
+    // B fragment (16 x 8, column major): rows 2t, 2t+1 and 2t+8, 2t+9 of column g.
+    // An element outside the operands reads the first of its row or column instead and
+    // counts as 0, so that the loads need no branches and all go out together.
+    const float *pa[2], *pb[GEMM_NT];
+    bool va[2], vb[GEMM_NT];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) fa[i] = ldA(m0 + g + ((i >> 1) & 1) * 8, k0 + 2 * t + (i & 1) + (i >> 2) * 8);
+    for (int i = 0; i < 2; ++i) {
+        va[i] = m0 + g + 8 * i < a.M;
+        pa[i] = a.A + (va[i] ? (int64_t)(m0 + g + 8 * i) * a.sam : 0);
+    }
 #pragma unroll
-        for (int j = 0; j < GEMM_NT; ++j)
+    for (int j = 0; j < GEMM_NT; ++j) {
+        vb[j] = n0 + 8 * j + g < a.N;
+        pb[j] = a.B + (vb[j] ? (int64_t)(n0 + 8 * j + g) * a.sbn : 0);
+    }
+    for (int k0 = kbeg; k0 < kend; k0 += 16 * GEMM_KU) {
+        float fa[GEMM_KU][2][4], fb[GEMM_KU][GEMM_NT][4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) fb[j][i] = ldB(k0 + 2 * t + (i & 1) + (i >> 1) * 8, n0 + 8 * j + g);
-    };
-    load(kbeg);
-    for (int k0 = kbeg; k0 < kend; k0 += 16) {
-        uint32_t ra[4], rb[GEMM_NT][2];
+        for (int s = 0; s < GEMM_KU; ++s) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) ra[i] = pack_bf16x2(fa[2 * i], fa[2 * i + 1]);
+            for (int i = 0; i < 4; ++i) {
+                const int k = k0 + 16 * s + 2 * t + (i & 1) + (i >> 1) * 8;
+                const bool vk = k < kend;
+                const int64_t ka = vk ? (int64_t)k * a.sak : 0, kb = vk ? (int64_t)k * a.sbk : 0;
 #pragma unroll
-        for (int j = 0; j < GEMM_NT; ++j) {
-            rb[j][0] = pack_bf16x2(fb[j][0], fb[j][1]);
-            rb[j][1] = pack_bf16x2(fb[j][2], fb[j][3]);
+                for (int x = 0; x < 2; ++x) {
+                    const float v = pa[x][ka];
+                    fa[s][x][i] = va[x] && vk ? v : 0.f;
+                }
+#pragma unroll
+                for (int j = 0; j < GEMM_NT; ++j) {
+                    const float v = pb[j][kb];
+                    fb[s][j][i] = vb[j] && vk ? v : 0.f;
+                }
+            }
         }
-        load(k0 + 16);   // zeros past the end
 #pragma unroll
-        for (int j = 0; j < GEMM_NT; ++j) mma_bf16_16816(acc[j], ra, rb[j][0], rb[j][1]);
+        for (int s = 0; s < GEMM_KU; ++s) {
+            const uint32_t ra[4] = {pack_bf16x2(fa[s][0][0], fa[s][0][1]), pack_bf16x2(fa[s][1][0], fa[s][1][1]),
+                                    pack_bf16x2(fa[s][0][2], fa[s][0][3]), pack_bf16x2(fa[s][1][2], fa[s][1][3])};
+#pragma unroll
+            for (int j = 0; j < GEMM_NT; ++j)
+                mma_bf16_16816(acc[j], ra, pack_bf16x2(fb[s][j][0], fb[s][j][1]),
+                               pack_bf16x2(fb[s][j][2], fb[s][j][3]));
+        }
     }
 #pragma unroll
     for (int j = 0; j < GEMM_NT; ++j) {
@@ -178,8 +195,9 @@ __global__ void k_gemm_reduce(GemmArgs a) {
 }
 
 void plan(GemmArgs &a) {
-    const int64_t tiles = ((a.M + 15) / 16) * ((a.N + 8 * GEMM_NT - 1) / (8 * GEMM_NT));
-    const int64_t blocks = (tiles + GEMM_WARPS - 1) / GEMM_WARPS;
+    const int64_t tiles_m = (a.M + 15) / 16;
+    // blocks of 16 x 128, the unit that the number of chunks is chosen by
+    const int64_t blocks = (tiles_m * ((a.N + 31) / 32) + 3) / 4;
     const int ksteps = (a.K + 15) / 16;
     // chunks of at least 4 k steps, enough of them to fill the GPU
     int nsplit = 1;
@@ -188,7 +206,7 @@ void plan(GemmArgs &a) {
     const int steps_per = (ksteps + nsplit - 1) / nsplit;
     a.kchunk = 16 * std::max(steps_per, 1);
     a.nsplit = std::max(1, (a.K + a.kchunk - 1) / a.kchunk);
-    a.blocks = (int)blocks;
+    a.blocks = (int)((tiles_m * ((a.N + 8 * GEMM_NT - 1) / (8 * GEMM_NT)) + GEMM_WARPS - 1) / GEMM_WARPS);
 }
 
 // one product, or two that do not depend on each other
