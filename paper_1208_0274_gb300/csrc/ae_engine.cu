@@ -891,7 +891,8 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 constexpr int AE_CHAIN_MAX = 8;
 
 // Average parent-row length up to which a level's rows are packed over the
-// lanes; longer rows are spread one entry per lane.  Per level of the 100 Mbp
+// lanes; longer rows are spread one entry per lane.  Per level (before the
+// packed kernel's last tuning, which took another tenth) of the 100 Mbp
 // text with queries of 10 kbp to 1 Mbp (packed against the walk it replaces):
 // rows of 158 entries 2.4 ms against 6.3, 57: 3.3 / 6.2, 59 (2.0 M nodes):
 // 8.3 / 10.7, 30: 10.6 / 11.8, 13: 20.2 / 15.8, 7.2: 26.2 / 38.8, 5.0: 41.8 /

@@ -16,11 +16,15 @@
 //             stage_cap entries per lane, DnaRowsArgs) are copied, longer rows
 //             and the other layouts are computed a second time.
 //
-// Rows are computed in one of three layouts chosen per level: short parent
-// rows walked one lane per (node, child) in column order (the horizontal gap
-// as a running key), long rows spread one parent entry per lane with the
-// horizontal gap as a segmented max-plus scan, and levels of few nodes with
-// long rows one node per block of WB_T threads (k_rows_dna_wide).  The general
+// Rows are computed in one of four layouts chosen per level: short parent rows
+// packed densely over the lanes, all of a task's entries in chunks of 32, one
+// child index after the other, each child row computed once (k_rows_pack, which
+// takes nearly all levels); long rows spread one parent entry per lane with the
+// horizontal gap as a segmented max-plus scan; levels of few nodes with long
+// rows one node per block of WB_T threads (k_rows_dna_wide); and, inside the
+// fixed arena of the no-allocation entry point and with row_layout 1, short rows
+// walked one lane per (node, child) in column order with the horizontal gap as a
+// running key.  The general
 // kernel (ae_trie.cu) handles protein, the int32 route, root rows and cost-tier
 // counting; all produce the same nodes and arenas.
 #include <cuda_runtime.h>
@@ -898,6 +902,14 @@ __global__ void __launch_bounds__(DW * 32, AE_DNA_MINB) k_rows_dna(DnaRowsArgs a
 // region to the leaf arena when complete; they and the range hits are few and
 // reserved exactly.  A reservation past an arena's capacity raises `retry` and
 // is not written; the cursors keep counting.
+//
+// Bound by instruction issue: 74 % of the slots (ALU pipe 66 %, L1 50 %, DRAM a
+// tenth of its peak), some 366 warp instructions per chunk and child, where the
+// walk takes 33-37 per output triple with 16 lanes active.  Whole searches, the
+// walk against this: 96 queries of 100 bp to 20 kbp 121 -> 67 ms, eight of 10 kbp to
+// 1 Mbp 383 -> 266 ms, cheap gaps 125 -> 90 ms.  Two prologue rounds (64 nodes a
+// task) leave L1 room that four take for shared memory (283 against 297 ms on
+// the second); resident blocks 5 / 6 / 7 / 8 / 9: 319 / 294 / 283 / 286 / 302 ms.
 constexpr int PK_W = 4;           // warps per block
 #ifndef AE_PACK_ROUNDS
 #define AE_PACK_ROUNDS 2
