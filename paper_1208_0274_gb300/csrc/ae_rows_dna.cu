@@ -904,8 +904,8 @@ __global__ void __launch_bounds__(DW * 32, AE_DNA_MINB) k_rows_dna(DnaRowsArgs a
 // is not written; the cursors keep counting.
 //
 // Bound by instruction issue: 74 % of the slots (ALU pipe 66 %, L1 50 %, DRAM a
-// tenth of its peak), some 366 warp instructions per chunk and child, where the
-// walk takes 33-37 per output triple with 16 lanes active.  Whole searches, the
+// fifth of its peak), 18-32 warp instructions per (child, parent entry) with 25
+// lanes active, where the walk takes 27-37 with 16-19.  Whole searches, the
 // walk against this: 96 queries of 100 bp to 20 kbp 121 -> 67 ms, eight of 10 kbp to
 // 1 Mbp 383 -> 266 ms, cheap gaps 125 -> 90 ms.  Two prologue rounds (64 nodes a
 // task) leave L1 room that four take for shared memory (283 against 297 ms on
