@@ -1167,9 +1167,11 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
             seg_width = max(seg_width, (unsigned long long)nlen);
             // once every task is taken, warps fall idle while the last wide walks go on, and
             // a block each is the better use of the chip from narrower rows on
-            if (rlen > a.esc_tail && esc_at != a.esc_tail && (seg_steps & 7) == 0 &&
-                *(volatile unsigned long long *)a.next_seg >= (unsigned long long)a.nseg)
-                esc_at = a.esc_tail;
+            if (rlen > a.esc_tail && esc_at != a.esc_tail && (seg_steps & 7) == 0) {
+                unsigned long long taken = 0;   // read once for the whole warp: the branches below are its
+                if (lane == 0) taken = *(volatile unsigned long long *)a.next_seg;
+                if (__shfl_sync(FULL, taken, 0) >= (unsigned long long)a.nseg) esc_at = a.esc_tail;
+            }
             if (esc_at > 0 && rlen > esc_at) {
                 // a wide row goes on on a whole block (k_leaf_wide), with the rest of
                 // this task's injections; the warp takes its next task
