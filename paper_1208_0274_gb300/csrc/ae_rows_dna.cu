@@ -1330,9 +1330,8 @@ __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsAr
     PackOut out;
     out.region_ent = a.region_ent;
     out.region_node = a.region_node;
-    if (lane < 3) w.base[lane] = a.base[lane];
+    uint64_t b[3] = {a.base[0], a.base[1], a.base[2]};   // before this level's leaf entries, injections and hits
     if (a.chain_pos > 0) {
-        uint64_t b[3] = {a.base[0], a.base[1], a.base[2]};
         bool again = false;
         for (int l = 0; l < a.chain_pos; ++l) {
             const LevelCounters &c = a.chain[l];
@@ -1344,11 +1343,6 @@ __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsAr
         const LevelCounters &c = a.chain[a.chain_pos - 1];
         nnodes = again || !c.n_node ? 0 : (int64_t)c.fr_node;
         if (nnodes == 0) return;
-        if (lane == 0) {
-            w.base[0] = b[0];
-            w.base[1] = b[1];
-            w.base[2] = b[2];
-        }
         const int64_t warps = (int64_t)gridDim.x * PK_W;
         npt = pack_task_nodes(nnodes, (int64_t)c.n_node, (int64_t)c.n_ent, warps);
         out.region_ent = (uint32_t)max((int64_t)64, min((int64_t)2048, (int64_t)c.n_ent / (8 * warps)));
@@ -1360,6 +1354,11 @@ __global__ void __launch_bounds__(PK_W * 32, AE_PACK_MINB) k_rows_pack(DnaRowsAr
     out.npos = 0;
     out.nrem = out.ents = out.nodes = 0;
     out.efull = out.nfull = false;
+    if (lane == 0) {   // one lane, once: stores of several lanes to a word would not be ordered
+        w.base[0] = b[0];
+        w.base[1] = b[1];
+        w.base[2] = b[2];
+    }
     if (lane < 4) {
         w.reg[lane] = PackRegion{0, 0, 0};
         w.carry[lane] = 0;
