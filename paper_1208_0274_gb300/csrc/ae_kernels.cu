@@ -782,11 +782,14 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
     int32_t esc_at = a.esc_min;
 
     while (!overflow) {
+        // one lane reads the counter and the overflow flag, which other warps write meanwhile:
+        // the whole warp goes on or stops together
         unsigned long long s = 0;
-        if (lane == 0) s = atomicAdd(a.next_seg, 1ull);
+        if (lane == 0)
+            s = *(volatile unsigned long long *)&a.stats->leaf_overflow ? (unsigned long long)a.nseg
+                                                                        : atomicAdd(a.next_seg, 1ull);
         s = __shfl_sync(FULL, s, 0);
         if (s >= (unsigned long long)a.nseg) break;
-        if (*(volatile unsigned long long *)&a.stats->leaf_overflow) break;
         int64_t k = task_start(a, lane, (int64_t)s);
         const int64_t kend = task_start(a, lane, (int64_t)s + 1);
         if (k >= kend) continue;
