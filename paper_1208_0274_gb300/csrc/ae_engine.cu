@@ -173,7 +173,7 @@ struct Workspace {
     // point hits of the whole search
     DevBuf hkey, hscore, hcount, hk1, hv1;
     // leaf sweep scratch; walks handed on to blocks (state, count, row buffers)
-    DevBuf scratch, next_seg, esc, esc_count, esc_pool, wide_rows;
+    DevBuf scratch, next_seg, esc, esc_count, esc_pool, wide_rows, cuts, qrange;
     // walk layout of the DNA row kernel: per warp and lane, the count phase's child rows
     DevBuf stage;
     // output
@@ -207,7 +207,7 @@ struct Workspace {
                 &aM[1], &aGa[0], &aGa[1], &nodes[0], &nodes[1], &cnt[0], &cnt[1], &cnt[2], &cnt[3],
                 &cnt[4], &off[0], &off[1], &off[2], &off[3], &off[4], &totals, &scan_tmp, &lj, &lM,
                 &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hkey, &hscore, &hcount, &hk1,
-                &hv1, &scratch, &next_seg, &esc, &esc_count, &esc_pool, &wide_rows, &stage, &uniq, &uflags, &uoff, &qcount, &stats, &stats_keep, &segs, &ctr, &chain, &seg_cnt, &seg_hit,
+                &hv1, &scratch, &next_seg, &esc, &esc_count, &esc_pool, &wide_rows, &cuts, &qrange, &stage, &uniq, &uflags, &uoff, &qcount, &stats, &stats_keep, &segs, &ctr, &chain, &seg_cnt, &seg_hit,
                 &task_first, &task_tot, &task_off, &task_tmp, &task_sum, &res, &res_key};
     }
 
@@ -230,7 +230,7 @@ struct Workspace {
     void trim_batch() {
         DevBuf *drop[] = {&aj[0], &aj[1], &aM[0], &aM[1], &aGa[0], &aGa[1], &nodes[0], &nodes[1], &cnt[0], &cnt[1],
                           &cnt[2], &cnt[3], &cnt[4], &off[0], &off[1], &off[2], &off[3], &off[4], &scan_tmp, &lj,
-                          &lM, &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hk1, &hv1, &scratch, &esc_pool, &wide_rows,
+                          &lM, &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hk1, &hv1, &scratch, &esc_pool, &wide_rows, &cuts,
                           &uniq,
                           &uflags, &uoff, &segs, &seg_cnt, &seg_hit, &task_first, &task_tot, &task_off, &task_tmp,
                           &res, &res_key};
@@ -478,7 +478,7 @@ struct Search {
     int be, bj, bq;
     int d0;
     int64_t nhits = 0;        // point hits accumulated in w->hkey/hscore
-    int64_t batch_queries = 1; // work items of the current batch
+    bool one_query = true;    // the current batch holds columns of one query only
     double batch_hint = -1;   // expected sweep hit records of the current batch (< 0: no hints)
     ae_stats stats;
     // the frontier's nodes and entries (its arenas may also hold unused ends of regions)
@@ -526,7 +526,7 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
     }
     const int sigma = ix.sigma;
     const int64_t batch_hits0 = nhits;
-    batch_queries = (int64_t)items.size();
+    one_query = items.front().qid == items.back().qid;
     const int nitems = (int)items.size();
     ensure(w->items, sizeof(WorkItem) * items.size(), st);
     CU(cudaMemcpyAsync(w->items.p, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, st));
@@ -849,22 +849,6 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 #endif
 #ifndef AE_LEAF_WIDE_POOL
 #define AE_LEAF_WIDE_POOL (1 << 22)
-#endif
-
-// Sweep tasks are cut at gaps between injections of more than AE_LEAF_GAP text
-// positions, or one and a half times the average gap of the batch's queries
-// where that is less (a fifth of the gaps of randomly placed injections is
-// longer; along a homolog they lie every few positions).  Cut at multiples of 32
-// injections instead, each part of a homologous region walked on to the
-// region's end beside the others: 13 times the cells and hit records on six
-// homologous reads (sweep 100 ms against 17).  Injections closer than
-// AE_LEAF_DENSE positions on average (protein at low thresholds) leave no gaps
-// to cut at.
-#ifndef AE_LEAF_GAP
-#define AE_LEAF_GAP 64
-#endif
-#ifndef AE_LEAF_DENSE
-#define AE_LEAF_DENSE 4
 #endif
 
 // Row length at which a warp's walk moves to a block once the sweep's tasks are
@@ -1324,15 +1308,14 @@ void Search::leaf_phase(int64_t ninj) {
                                                                  : (int64_t)(ninj * w->hit_ratio) + 4096);
     // wide walks move to blocks (not inside the fixed arena of the no-allocation
     // entry point, nor when entries are counted by tier, which only the warp walk does)
-    const double spacing = (double)ix.n * (double)batch_queries / (double)ninj;
-    const bool sparse = spacing >= AE_LEAF_DENSE;
     // the default chooses: where injections leave gaps the few wide walks set the
     // sweep's time, and a step on a block is faster from the first row past a warp's
     // lanes on (613 bp query: 0.76 ms from 32 entries, 0.79 from 64, 1.09 from 128);
     // where they are dense every task walks a wide row and warps are the better use of
     // the chip (1 M residues, BLOSUM62, sweep: from 128 entries 127 ms, 512: 104,
     // 1,024: 69, never: 84), until the tasks run out (AE_LEAF_WIDE_TAIL)
-    const int32_t wide = opt.leaf_wide_rows != 128 ? opt.leaf_wide_rows : sparse ? 32 : 1024;
+    const bool choose = opt.leaf_wide_rows == 128;
+    const int32_t wide = choose ? 32 : opt.leaf_wide_rows;
     const int32_t esc_min = (g_arena || opt.tier_stats) ? 0 : wide;
     const int32_t esc_max = esc_min > 0 ? AE_LEAF_WIDE_SLOTS : 0;
     // the counters before the sweep: one that is run again counts once
@@ -1389,7 +1372,8 @@ void Search::leaf_phase(int64_t ninj) {
         la.tiers = opt.tier_stats ? 1 : 0;
         la.stats = ptr<DevStats>(w->stats);
         la.esc_min = esc_max > 0 ? esc_min : 0;
-        la.esc_tail = std::min(la.esc_min, opt.leaf_wide_rows == 128 ? AE_LEAF_WIDE_TAIL : la.esc_min);
+        la.esc_dense = choose && la.esc_min > 0 ? 1024 : la.esc_min;
+        la.esc_tail = std::min(la.esc_dense, choose ? AE_LEAF_WIDE_TAIL : la.esc_min);
         la.esc_max = esc_max;
         if (esc_max > 0) {
             la.esc_count = ptr<unsigned long long>(w->esc_count);
@@ -1400,8 +1384,11 @@ void Search::leaf_phase(int64_t ninj) {
             la.wide_cap = w->wide_cap;
             la.wide_blocks = wide_blocks;
         }
-        la.keys = keys;
-        la.gap = sparse ? (uint32_t)std::min<double>(AE_LEAF_GAP, 1.5 * spacing) : 0;
+        ensure(w->cuts, (size_t)la.nseg * 4, st);
+        if (!one_query) ensure(w->qrange, sizeof(uint2) * (size_t)nq, st);
+        la.qrange = one_query ? nullptr : ptr<uint2>(w->qrange);
+        if (attempt == 0) ae_leaf_cuts(la, keys, ptr<uint2>(w->qrange), ptr<uint32_t>(w->cuts), st);
+        la.cuts = ptr<uint32_t>(w->cuts);
         prof.mark(K_LEAF);
         ++stats.leaf_sweeps;
         const auto t_sweep = std::chrono::steady_clock::now();

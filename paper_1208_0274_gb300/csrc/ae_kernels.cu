@@ -477,6 +477,87 @@ __global__ void k_inject_keys(const Inject *inj, int64_t ninj, uint64_t *keys, u
     }
 }
 
+// Of the sorted keys: the range of each query's injections
+__global__ void k_query_ranges(const uint64_t *keys, int64_t ninj, uint2 *range) {
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ninj; t += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t q = (uint32_t)(keys[t] >> 32);
+        if (t == 0 || (uint32_t)(keys[t - 1] >> 32) != q) range[q].x = (uint32_t)t;
+        if (t + 1 == ninj || (uint32_t)(keys[t + 1] >> 32) != q) range[q].y = (uint32_t)(t + 1);
+    }
+}
+
+// Whether the injections of query q lie so close that they leave no gaps
+__device__ __forceinline__ bool leaf_dense(const LeafArgs &a, int32_t q) {
+    const uint64_t c = a.qrange ? a.qrange[q].y - a.qrange[q].x : (uint64_t)a.ninj;
+    return (uint64_t)a.ix.n < AE_LEAF_DENSE * c;
+}
+
+// Where tasks of the sweep may start: for each multiple of seg, the first place
+// before the next multiple at which the injections are cut (an offset, or
+// LEAF_NO_CUT).  Rows injected close to each other, as along a homologous region,
+// belong to one walk: cut apart, each part's walk would run on to the region's
+// end beside the others, over the same cells.  So they are cut
+// - where the query changes,
+// - at gaps of more than AE_LEAF_GAP text positions, or one and a half times the
+//   query's average gap where that is less (a fifth of the gaps of randomly placed
+//   injections is longer; along a homolog they lie every few positions),
+// - at multiples of a span of two to four query lengths, if there was no gap for
+//   a span before.  A row lives about as long as its query, so a longer task only
+//   walks one row after the other that could be walked side by side, as in a
+//   tandem repeat that the query holds one copy of (3,000 copies of 171 letters,
+//   613 bp query: sweep 17.3 ms without, 10.6 with this cut),
+// - at every multiple of seg if the query's injections are dense.
+// Cut at multiples of 32 injections instead, six homologous reads wrote 13 times
+// the hit records (sweep 100 ms against 17).  One warp per multiple.
+constexpr uint32_t LEAF_NO_CUT = 0xFFFFFFFFu;
+__global__ void __launch_bounds__(256) k_leaf_cuts(LeafArgs a, const uint64_t *keys, uint32_t *cuts) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t s = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); s < a.nseg;
+         s += (int64_t)gridDim.x * (blockDim.x >> 5)) {
+        const int64_t k0 = s * a.seg, k1 = min(k0 + a.seg, a.ninj);
+        uint32_t at = LEAF_NO_CUT;
+        for (int64_t k = k0; k < k1 && at == LEAF_NO_CUT; k += 32) {
+            const int64_t x = k + lane;
+            bool cut = false, past = false;
+            uint64_t y = 0;
+            uint32_t gap = 0;
+            int span = 0;   // log2
+            if (x < k1) {
+                y = keys[x];
+                const uint64_t z = x ? keys[x - 1] : ~0ull;
+                const int32_t q = (int32_t)(y >> 32);
+                const uint64_t c = a.qrange ? a.qrange[q].y - a.qrange[q].x : (uint64_t)a.ninj;
+                gap = (uint32_t)min((uint64_t)AE_LEAF_GAP, 3 * (uint64_t)a.ix.n / (2 * c));
+                span = min(max(33 - __clz(a.qv.m[q]), AE_LEAF_SPAN_MIN), AE_LEAF_SPAN_MAX);
+                cut = (y >> 32) != (z >> 32) || (uint32_t)y - (uint32_t)z > gap || (x == k0 && leaf_dense(a, q));
+                past = !cut && ((uint32_t)y >> span) != ((uint32_t)z >> span);
+            }
+            const unsigned bc = __ballot_sync(FULL, cut), bp = __ballot_sync(FULL, past);
+            for (unsigned b = bc | bp; b && at == LEAF_NO_CUT; b &= b - 1) {   // in order
+                const int l = __ffs(b) - 1;
+                bool here = (bc >> l) & 1u;
+                if (!here) {
+                    // past a multiple of the span: a cut if no gap lies within a span before it
+                    const uint64_t yl = __shfl_sync(FULL, y, l);
+                    const uint32_t gl = __shfl_sync(FULL, gap, l), len = 1u << __shfl_sync(FULL, span, l);
+                    unsigned ended = 0, broken = 0;
+                    for (int64_t w = k + l - 1; !(ended | broken); w -= 32) {
+                        const int64_t t = w - lane;
+                        const uint64_t v = t >= 0 ? keys[t] : ~0ull, u = t > 0 ? keys[t - 1] : ~0ull;
+                        const bool far = t >= 0 && (v >> 32) == (yl >> 32) && (uint32_t)yl - (uint32_t)v >= len;
+                        ended = __ballot_sync(FULL, far);
+                        broken = __ballot_sync(FULL, !far && ((u >> 32) != (v >> 32) || (uint32_t)v - (uint32_t)u > gl ||
+                                                              t <= 0));
+                    }
+                    here = ended && (!broken || __ffs(ended) < __ffs(broken));
+                }
+                if (here) at = (uint32_t)(k - k0) + l;
+            }
+        }
+        if (lane == 0) cuts[s] = at;
+    }
+}
+
 struct Buf {
     int32_t *j, *M, *Ga;
 };
@@ -715,29 +796,19 @@ __device__ __forceinline__ void leaf_merge(const LeafArgs &a, int lane, int32_t 
     }
 }
 
-// First injection of task s.  Rows injected close to each other, as along a
-// homologous region, belong to one walk: cut apart, each part's walk would run
-// on to the region's end beside the others, over the same cells.  So a task
-// starts where the injections leave a gap.  A stretch of TASK_REACH injections
-// without one is cut at the multiple of seg.  The result depends on s alone and
-// does not decrease.
-constexpr int64_t TASK_REACH = 65536;
+// First injection of task s: the first cut at or behind the multiple of seg.  It
+// depends on s alone and does not decrease.
 __device__ __forceinline__ int64_t task_start(const LeafArgs &a, int lane, int64_t s) {
-    const int64_t k0 = s * a.seg;
-    if (k0 >= a.ninj) return a.ninj;
-    if (s == 0 || a.gap == 0) return k0;
-    const int64_t end = min(k0 + TASK_REACH, a.ninj);
-    for (int64_t k = k0; k < end; k += 32) {
-        const int64_t x = k + lane;
-        bool cut = false;
-        if (x < end) {
-            const uint64_t y = a.keys[x], z = a.keys[x - 1];
-            cut = (y >> 32) != (z >> 32) || (uint32_t)y - (uint32_t)z > a.gap;
+    if (!a.cuts || s == 0) return min(s * a.seg, a.ninj);
+    for (int64_t t = s; t < a.nseg; t += 32) {
+        const uint32_t c = t + lane < a.nseg ? a.cuts[t + lane] : LEAF_NO_CUT;
+        const unsigned b = __ballot_sync(FULL, c != LEAF_NO_CUT);
+        if (b) {
+            const int l = __ffs(b) - 1;
+            return (t + l) * a.seg + __shfl_sync(FULL, c, l);
         }
-        const unsigned b = __ballot_sync(FULL, cut);
-        if (b) return k + __ffs(b) - 1;
     }
-    return end == a.ninj ? a.ninj : k0;
+    return a.ninj;
 }
 
 // One warp per segment of `seg` consecutive injections (sorted by query and
@@ -779,7 +850,7 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
     const uint64_t jmask = (1ull << a.bj) - 1ull;
     unsigned long long st_rows = 0, st_ent = 0, st_t0 = 0, st_t1 = 0, st_t2 = 0, st_reused = 0;
     bool overflow = false;
-    int32_t esc_at = a.esc_min;
+    bool tail = false;   // every task is taken
 
     while (!overflow) {
         // one lane reads the counter and the overflow flag, which other warps write meanwhile:
@@ -812,6 +883,10 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
             nk_qid = In.qid;
             nk_e = In.e;
         }
+        // row length at which the walk moves to a block
+        int32_t esc_at = a.esc_min;
+        if (a.esc_min != a.esc_dense && leaf_dense(a, nk_qid)) esc_at = a.esc_dense;
+        if (tail) esc_at = min(esc_at, a.esc_tail);
         while (true) {
             if (rlen == 0 && k < kend) {
                 // ---- jump to a lone injected row: it is already a finished row
@@ -1170,10 +1245,11 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
             seg_width = max(seg_width, (unsigned long long)nlen);
             // once every task is taken, warps fall idle while the last wide walks go on, and
             // a block each is the better use of the chip from narrower rows on
-            if (rlen > a.esc_tail && esc_at != a.esc_tail && (seg_steps & 7) == 0) {
+            if (rlen > a.esc_tail && esc_at > a.esc_tail && (seg_steps & 7) == 0) {
                 unsigned long long taken = 0;   // read once for the whole warp: the branches below are its
                 if (lane == 0) taken = *(volatile unsigned long long *)a.next_seg;
-                if (__shfl_sync(FULL, taken, 0) >= (unsigned long long)a.nseg) esc_at = a.esc_tail;
+                tail = __shfl_sync(FULL, taken, 0) >= (unsigned long long)a.nseg;
+                if (tail) esc_at = a.esc_tail;
             }
             if (esc_at > 0 && rlen > esc_at) {
                 // a wide row goes on on a whole block (k_leaf_wide), with the rest of
@@ -2009,6 +2085,16 @@ void ae_inject_keys(const Inject *inj, int64_t ninj, uint64_t *keys, uint32_t *v
 int ae_leaf_wide_blocks_per_sm() { return 1; }
 
 int64_t ae_leaf_scratch_words(int32_t cap, int32_t nwarps) { return (int64_t)6 * cap * nwarps; }
+
+void ae_leaf_cuts(const LeafArgs &a, const uint64_t *keys, uint2 *qrange, uint32_t *cuts, cudaStream_t st) {
+    if (a.nseg <= 0) return;
+    if (a.qrange) {
+        ++g_launches;
+        k_query_ranges<<<grid_for(a.ninj, 256), 256, 0, st>>>(keys, a.ninj, qrange);
+    }
+    ++g_launches;
+    k_leaf_cuts<<<grid_for(a.nseg, 8), 256, 0, st>>>(a, keys, cuts);
+}
 
 void ae_leaf_sweep(const LeafArgs &a, int blocks, int threads, cudaStream_t st) {
     if (a.nseg <= 0) return;

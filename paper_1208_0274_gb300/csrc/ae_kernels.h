@@ -228,6 +228,21 @@ int ae_rows_pack_blocks_per_sm();
 int ae_rows_pack_warps_per_block();
 // nodes per task of a level with `nodes` nodes in `slots` records and `entries` row entries
 int ae_rows_pack_task_nodes(int64_t slots, int64_t nodes, int64_t entries, int64_t warps);
+// Sweep: the widest gap between injections that a task may hold (text positions),
+// injections closer than AE_LEAF_DENSE positions on average leave no gaps (protein
+// at low thresholds), log2 of the shortest and longest span of a task
+#ifndef AE_LEAF_GAP
+#define AE_LEAF_GAP 64
+#endif
+#ifndef AE_LEAF_DENSE
+#define AE_LEAF_DENSE 4
+#endif
+#ifndef AE_LEAF_SPAN_MIN
+#define AE_LEAF_SPAN_MIN 10
+#endif
+#ifndef AE_LEAF_SPAN_MAX
+#define AE_LEAF_SPAN_MAX 16
+#endif
 struct LeafArgs {
     IndexView ix;
     ScoreView sc;
@@ -250,24 +265,24 @@ struct LeafArgs {
     int32_t tiers;                // 1: count entries by cost tier
     DevStats *stats;
     // walks whose row grows past esc_min entries (0: never) continue on a whole
-    // block (k_leaf_wide) with the rest of their task's injections (past esc_tail
-    // once all tasks are taken): esc[slot] is
+    // block (k_leaf_wide) with the rest of their task's injections (past esc_dense where
+    // the query's injections are dense, past esc_tail once all tasks are taken): esc[slot] is
     // the walk's state, its row lies in the pool at esc[slot].row.  esc_count counts
     // the slots taken, the pool's entries taken and the walks the blocks have
     // taken; the first two may pass esc_max and esc_pool_cap: a walk that finds no
     // room stays on its warp.  Each of the wide_blocks blocks has 6 * wide_cap
     // words of row buffers at wide_rows.
-    int32_t esc_min, esc_tail, esc_max;
+    int32_t esc_min, esc_dense, esc_tail, esc_max;
     int64_t esc_pool_cap;
     unsigned long long *esc_count;
     struct EscWalk *esc;
     int32_t *esc_pool;
     int32_t *wide_rows;
     int32_t wide_cap, wide_blocks;
-    // sorted (query, text end) of the injections; a task starts at the first one past
-    // a multiple of seg that is more than `gap` positions from the one before it
-    const uint64_t *keys;
-    uint32_t gap;
+    // where tasks may start, by multiple of seg (ae_leaf_cuts; NULL: at every multiple),
+    // and each query's range of the sorted injections (NULL: all are one query's)
+    const uint32_t *cuts;
+    const uint2 *qrange;
 };
 // A sweep walk handed from a warp to a block: its query, text position, the
 // row at that position (rlen entries from `row` on in the pool) and its task's
@@ -277,6 +292,9 @@ struct EscWalk {
     int64_t rlen, k, kend, row;
 };
 int ae_leaf_wide_blocks_per_sm();
+// Cuts between the sorted injections (`keys`: query, text end); a's ninj, seg, nseg,
+// qrange (NULL, or `qrange`, which is filled first) and views are set.
+void ae_leaf_cuts(const LeafArgs &a, const uint64_t *keys, uint2 *qrange, uint32_t *cuts, cudaStream_t st);
 void ae_inject_keys(const Inject *inj, int64_t ninj, uint64_t *keys, uint32_t *vals, cudaStream_t st);
 void ae_leaf_sweep(const LeafArgs &a, int blocks, int threads, cudaStream_t st);
 int64_t ae_leaf_scratch_words(int32_t cap, int32_t nwarps);
