@@ -1370,6 +1370,7 @@ void Search::leaf_phase(int64_t ninj) {
         la.be = be;
         la.bj = bj;
         la.tiers = opt.tier_stats ? 1 : 0;
+        la.few = esc_max == 0 ? 1 : 0;
         la.stats = ptr<DevStats>(w->stats);
         la.esc_min = esc_max > 0 ? esc_min : 0;
         la.esc_dense = choose && la.esc_min > 0 ? 1024 : la.esc_min;

@@ -684,6 +684,7 @@ __device__ __forceinline__ void make_slots(const ScoreView &sc, const int8_t *sm
 // entries into rows of 130, sweep 89 -> 69 ms.
 // Used by the warp walk of k_leaf and, run by one warp, by the block walk of
 // k_leaf_wide.
+template <bool RUN>
 __device__ __forceinline__ void leaf_merge(const LeafArgs &a, int lane, int32_t qid, int32_t p, int32_t H,
                                            uint64_t jmask, int64_t &k, int64_t kend, const Buf &Rn, int64_t &nlen,
                                            int64_t cap, bool &overflow, HitStage &hstage, unsigned long long &st_ent,
@@ -708,6 +709,10 @@ __device__ __forceinline__ void leaf_merge(const LeafArgs &a, int lane, int32_t 
                 Mi = iM[idx];
                 Gi = iGa[idx];
                 int32_t lo = 0, hi = n;
+                if (RUN && n > 0) {   // columns are consecutive along a homolog: look there first (2 % of such a walk)
+                    const int32_t x = y - Rn.j[0];
+                    if (x >= 0 && x < n && Rn.j[x] == y) lo = hi = x;
+                }
                 while (lo < hi) {
                     const int32_t mid = (lo + hi) >> 1;
                     if (Rn.j[mid] < y) lo = mid + 1; else hi = mid;
@@ -823,15 +828,21 @@ __device__ __forceinline__ int64_t task_start(const LeafArgs &a, int lane, int64
 // its segment, to a slot of k_leaf_wide (a block of threads per walk); when
 // the slots are taken the warp carries on itself.
 // A step is a chain of scans and dependent loads, so the resident warps set the
-// rate: 6 blocks per SM at one entry per lane (80 registers, a few spilled)
+// rate: 6 blocks per SM at one entry per lane (E = 1; 80 registers, some spilled)
 // against 3 at two entries (162 registers, 38 % of the issue slots used; 526
 // warp instructions per 32 entries).  Sweeps of a protein batch, a 1 M-letter query
 // and a batch with cheap gaps: 51.7 / 22.9 / 11.3 ms against 58.5 / 28.8 / 16.1
-// (4 blocks 53.3 / 24.6 / 12.7; 8 blocks 53.2 / - / 11.3).
+// (4 blocks 53.3 / 24.6 / 12.7; 8 blocks 53.2 / - / 11.3).  Where no walk moves to
+// a block (tier counting, leaf_wide_rows 0, the fixed arena of the no-allocation
+// entry point with its two blocks per SM) the longest walk sets the time, and two
+// entries per lane without spills are faster (E = 2, 164 registers): a 400-letter
+// homolog in the arena 1.81 ms against 2.36, 100 reads of 1,000 letters with tier
+// counting 11.1 / 15.3, six of 4,000-12,000 letters 1,030 / 1,650.
 #ifndef AE_LEAF_MINB
 #define AE_LEAF_MINB 6
 #endif
-__global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
+template <int E>
+__global__ void __launch_bounds__(128, E == 1 ? AE_LEAF_MINB : 2) k_leaf(LeafArgs a) {
     __shared__ int8_t smat[AE_MAX_SIGMA * AE_MAX_SIGMA];
     __shared__ uint64_t s_hkey[LEAF_WARPS][LEAF_HS];
     __shared__ int32_t s_hscore[LEAF_WARPS][LEAF_HS];
@@ -1126,46 +1137,72 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
                 // into Rn (the finished row at p) with its hits
                 int32_t carry = AE_KNEG, prev_j = -2, prev_M = AE_NEG;
                 // the next chunk's entries are loaded while this chunk is computed
-                int32_t nj = lane < rlen ? R.j[lane] : m, nM = lane < rlen ? R.M[lane] : AE_NEG,
-                        nG = lane < rlen ? R.Ga[lane] : AE_NEG;
-                for (int64_t base = 0; base < rlen; base += 32) {
-                    const int64_t i0 = base + lane;
-                    const bool valid = i0 < rlen;
-                    const int32_t j = nj, M = nM, G = nG;
-                    {
-                        const int64_t x = i0 + 32;
+                int32_t nj[E], nM[E], nG[E];
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int64_t x = (int64_t)lane * E + e;
+                    const bool v = x < rlen;
+                    nj[e] = v ? R.j[x] : m;
+                    nM[e] = v ? R.M[x] : AE_NEG;
+                    nG[e] = v ? R.Ga[x] : AE_NEG;
+                }
+                for (int64_t base = 0; base < rlen; base += 32 * E) {
+                    const int64_t i0 = base + (int64_t)lane * E;
+                    int32_t jj[E], MM[E], GG[E];
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        jj[e] = nj[e];
+                        MM[e] = nM[e];
+                        GG[e] = nG[e];
+                        const int64_t x = i0 + 32 * E + e;
                         const bool v = x < rlen;
-                        nj = v ? R.j[x] : m;
-                        nM = v ? R.M[x] : AE_NEG;
-                        nG = v ? R.Ga[x] : AE_NEG;
+                        nj[e] = v ? R.j[x] : m;
+                        nM[e] = v ? R.M[x] : AE_NEG;
+                        nG[e] = v ? R.Ga[x] : AE_NEG;
                     }
                     // the first entry of the next chunk (lane 0's next load), m past the row
-                    int32_t jn = __shfl_down_sync(FULL, j, 1);
-                    const int32_t jfirst_next = __shfl_sync(FULL, nj, 0);
-                    if (lane == 31) jn = jfirst_next;
-                    if (i0 + 1 >= rlen) jn = m;
-                    int32_t pj = __shfl_up_sync(FULL, j, 1), pM = __shfl_up_sync(FULL, M, 1);
+                    int32_t jnext = __shfl_down_sync(FULL, jj[0], 1);
+                    const int32_t jfirst_next = __shfl_sync(FULL, nj[0], 0);
+                    if (lane == 31) jnext = jfirst_next;
+                    int32_t pj0 = __shfl_up_sync(FULL, jj[E - 1], 1), pM0 = __shfl_up_sync(FULL, MM[E - 1], 1);
                     if (lane == 0) {
-                        pj = prev_j;
-                        pM = prev_M;
+                        pj0 = prev_j;
+                        pM0 = prev_M;
                     }
-                    Slots sl;
-                    make_slots(sc, smat, c, P, m, H, g, oe, valid, j, M, G, pj, pM, jn, sl);
-                    const int32_t keyA = sl.MpA > AE_NEG ? sl.MpA + sl.colA * u : AE_KNEG;
-                    const int32_t keyB = sl.MpB > AE_NEG ? sl.MpB + (sl.colA + 1) * u : AE_KNEG;
-                    int32_t incl = warp_incl_max(max(keyA, keyB));
+                    Slots sl[E];
+                    int32_t lk[E];   // the lane's keys up to and with entry e
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const bool v = i0 + e < rlen;
+                        int32_t jn = e + 1 < E ? jj[e + 1 < E ? e + 1 : 0] : jnext;
+                        if (i0 + e + 1 >= rlen) jn = m;
+                        const int32_t pj = e ? jj[e ? e - 1 : 0] : pj0, pM = e ? MM[e ? e - 1 : 0] : pM0;
+                        make_slots(sc, smat, c, P, m, H, g, oe, v, jj[e], MM[e], GG[e], pj, pM, jn, sl[e]);
+                        const int32_t keyA = sl[e].MpA > AE_NEG ? sl[e].MpA + sl[e].colA * u : AE_KNEG;
+                        const int32_t keyB = sl[e].MpB > AE_NEG ? sl[e].MpB + (sl[e].colA + 1) * u : AE_KNEG;
+                        lk[e] = max(e ? lk[e ? e - 1 : 0] : AE_KNEG, max(keyA, keyB));
+                    }
+                    int32_t incl = warp_incl_max(lk[E - 1]);
                     int32_t excl = __shfl_up_sync(FULL, incl, 1);
                     if (lane == 0) excl = AE_KNEG;
                     incl = max(incl, carry);
                     excl = max(excl, carry);
-                    SlotOut o;
-                    slot_finish(sl.colA, sl.MpA, sl.hasB, sl.MpB, sl.next_col, excl, incl, sc, m, H, u, valid, o);
-                    const uint32_t nA = o.aliveA, nB = o.aliveB, nR = (uint32_t)o.run_len;
-                    const uint32_t hA = o.aliveA && o.MA >= H, hB = o.aliveB && o.MB >= H;
-                    const uint32_t cl = nA + nB + nR, hl = hA + hB + (uint32_t)o.run_hits;
+                    SlotOut o[E];
+                    int32_t ik[E];
+                    uint32_t cl = 0, hl = 0;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const int32_t ex = e ? max(excl, lk[e ? e - 1 : 0]) : excl;
+                        ik[e] = max(excl, lk[e]);
+                        slot_finish(sl[e].colA, sl[e].MpA, sl[e].hasB, sl[e].MpB, sl[e].next_col, ex, ik[e], sc, m, H,
+                                    u, i0 + e < rlen, o[e]);
+                        cl += (uint32_t)o[e].aliveA + (uint32_t)o[e].aliveB + (uint32_t)o[e].run_len;
+                        hl += (uint32_t)(o[e].aliveA && o[e].MA >= H) + (uint32_t)(o[e].aliveB && o[e].MB >= H) +
+                              (uint32_t)o[e].run_hits;
+                    }
                     carry = __shfl_sync(FULL, incl, 31);
-                    prev_j = __shfl_sync(FULL, j, 31);
-                    prev_M = __shfl_sync(FULL, M, 31);
+                    prev_j = __shfl_sync(FULL, jj[E - 1], 31);
+                    prev_M = __shfl_sync(FULL, MM[E - 1], 31);
                     const uint32_t ci = warp_incl_sum(cl);
                     const uint32_t tot = __shfl_sync(FULL, ci, 31);
                     if (nlen + tot > cap) {
@@ -1178,48 +1215,56 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
                     uint64_t hbase = 0;
                     if (htot) hbase = stage_reserve(hstage, a, lane, htot, staged, hok);
                     const uint64_t kq = ((uint64_t)qid << (a.be + a.bj)) | ((uint64_t)(uint32_t)p << a.bj);
-                    const int64_t eo = nlen + (int64_t)(ci - cl);
-                    const uint64_t ho = hbase + hi - hl;
-                    if (nA) {
-                        Rn.j[eo] = j;
-                        Rn.M[eo] = o.MA;
-                        Rn.Ga[eo] = sl.GaA;
-                        if (hA && hok) hit_put(hstage, a, staged, ho, kq | ((uint64_t)j & jmask), o.MA);
-                        if (a.tiers) {
-                            const int tier = (sl.Dp > AE_NEG) + (sl.GaA > AE_NEG) + (o.GbA > thr_of(j, m, H, g));
-                            st_t0 += tier <= 1;
-                            st_t1 += tier == 2;
-                            st_t2 += tier >= 3;
+                    int64_t eo = nlen + (int64_t)(ci - cl);
+                    uint64_t ho = hbase + hi - hl;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const uint32_t nA = o[e].aliveA, nB = o[e].aliveB, nR = (uint32_t)o[e].run_len;
+                        const uint32_t hA = o[e].aliveA && o[e].MA >= H, hB = o[e].aliveB && o[e].MB >= H;
+                        const int32_t j = jj[e];
+                        if (nA) {
+                            Rn.j[eo] = j;
+                            Rn.M[eo] = o[e].MA;
+                            Rn.Ga[eo] = sl[e].GaA;
+                            if (hA && hok) hit_put(hstage, a, staged, ho, kq | ((uint64_t)j & jmask), o[e].MA);
+                            if (a.tiers) {
+                                const int tier = (sl[e].Dp > AE_NEG) + (sl[e].GaA > AE_NEG) + (o[e].GbA > thr_of(j, m, H, g));
+                                st_t0 += tier <= 1;
+                                st_t1 += tier == 2;
+                                st_t2 += tier >= 3;
+                            }
                         }
-                    }
-                    if (nB) {
-                        Rn.j[eo + nA] = j + 1;
-                        Rn.M[eo + nA] = o.MB;
-                        Rn.Ga[eo + nA] = AE_NEG;
-                        if (hB && hok) hit_put(hstage, a, staged, ho + hA, kq | ((uint64_t)(j + 1) & jmask), o.MB);
-                        if (a.tiers) {
-                            if ((sl.Dk > AE_NEG) && (o.GbB > thr_of(j + 1, m, H, g))) ++st_t1; else ++st_t0;
+                        if (nB) {
+                            Rn.j[eo + nA] = j + 1;
+                            Rn.M[eo + nA] = o[e].MB;
+                            Rn.Ga[eo + nA] = AE_NEG;
+                            if (hB && hok) hit_put(hstage, a, staged, ho + hA, kq | ((uint64_t)(j + 1) & jmask), o[e].MB);
+                            if (a.tiers) {
+                                if ((sl[e].Dk > AE_NEG) && (o[e].GbB > thr_of(j + 1, m, H, g))) ++st_t1; else ++st_t0;
+                            }
                         }
-                    }
-                    if (a.tiers) st_t0 += nR;
-                    unsigned rmask = __ballot_sync(FULL, nR > 0);
-                    while (rmask) {
-                        const int L = __ffs(rmask) - 1;
-                        rmask &= rmask - 1;
-                        const int32_t s0 = __shfl_sync(FULL, o.run_start, L);
-                        const int32_t rl = __shfl_sync(FULL, o.run_len, L);
-                        const int32_t rh = __shfl_sync(FULL, o.run_hits, L);
-                        const int32_t K = __shfl_sync(FULL, incl, L);
-                        const int64_t d0 = __shfl_sync(FULL, eo + nA + nB, L);
-                        const uint64_t hd = __shfl_sync(FULL, ho + hA + hB, L);
-                        for (int32_t t = lane; t < rl; t += 32) {
-                            const int32_t cc = s0 + t;
-                            const int32_t v = sc.sg - cc * u + K;
-                            Rn.j[d0 + t] = cc;
-                            Rn.M[d0 + t] = v;
-                            Rn.Ga[d0 + t] = AE_NEG;
-                            if (t < rh && hok) hit_put(hstage, a, staged, hd + t, kq | ((uint64_t)cc & jmask), v);
+                        if (a.tiers) st_t0 += nR;
+                        unsigned rmask = __ballot_sync(FULL, nR > 0);
+                        while (rmask) {
+                            const int L = __ffs(rmask) - 1;
+                            rmask &= rmask - 1;
+                            const int32_t s0 = __shfl_sync(FULL, o[e].run_start, L);
+                            const int32_t rl = __shfl_sync(FULL, o[e].run_len, L);
+                            const int32_t rh = __shfl_sync(FULL, o[e].run_hits, L);
+                            const int32_t K = __shfl_sync(FULL, ik[e], L);
+                            const int64_t d0 = __shfl_sync(FULL, eo + nA + nB, L);
+                            const uint64_t hd = __shfl_sync(FULL, ho + hA + hB, L);
+                            for (int32_t t = lane; t < rl; t += 32) {
+                                const int32_t cc = s0 + t;
+                                const int32_t v = sc.sg - cc * u + K;
+                                Rn.j[d0 + t] = cc;
+                                Rn.M[d0 + t] = v;
+                                Rn.Ga[d0 + t] = AE_NEG;
+                                if (t < rh && hok) hit_put(hstage, a, staged, hd + t, kq | ((uint64_t)cc & jmask), v);
+                            }
                         }
+                        eo += nA + nB + nR;
+                        ho += hA + hB + (uint32_t)o[e].run_hits;
                     }
                     nlen += tot;
                 }
@@ -1227,7 +1272,7 @@ __global__ void __launch_bounds__(128, AE_LEAF_MINB) k_leaf(LeafArgs a) {
                 if (overflow) break;
                 st_ent += (unsigned long long)nlen;
             }
-            leaf_merge(a, lane, qid, p, H, jmask, k, kend, Rn, nlen, cap, overflow, hstage, st_ent, st_reused, st_t0);
+            leaf_merge<E == 2>(a, lane, qid, p, H, jmask, k, kend, Rn, nlen, cap, overflow, hstage, st_ent, st_reused, st_t0);
             if (overflow) break;
             if (k < kend) {
                 const Inject In = a.inj[a.order[k]];
@@ -1832,7 +1877,7 @@ __global__ void __launch_bounds__(WIDE_T, 1) k_leaf_wide(LeafArgs a) {
                         bool ovf = nxt < 2;   // longer than the buffers: reported
                         int64_t kk = k, nl = nlen;
                         if (!ovf)
-                            leaf_merge(a, lane, qid, p, H, jmask, kk, k + 1, buf(nxt), nl, (int64_t)a.wide_cap, ovf, mstage,
+                            leaf_merge<true>(a, lane, qid, p, H, jmask, kk, k + 1, buf(nxt), nl, (int64_t)a.wide_cap, ovf, mstage,
                                        st_ent, st_reused, st_t0);
                         if (lane == 0) {
                             s.nlen = nl;
@@ -2099,7 +2144,8 @@ void ae_leaf_cuts(const LeafArgs &a, const uint64_t *keys, uint2 *qrange, uint32
 void ae_leaf_sweep(const LeafArgs &a, int blocks, int threads, cudaStream_t st) {
     if (a.nseg <= 0) return;
     ++g_launches;
-    k_leaf<<<blocks, threads, 0, st>>>(a);
+    if (a.few) k_leaf<2><<<blocks, threads, 0, st>>>(a);
+    else k_leaf<1><<<blocks, threads, 0, st>>>(a);
     if (a.esc_min > 0 && a.esc_max > 0) {   // the walks handed on to blocks
         ++g_launches;
         cudaFuncSetAttribute(k_leaf_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WideSmem));

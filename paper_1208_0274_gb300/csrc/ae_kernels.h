@@ -263,6 +263,7 @@ struct LeafArgs {
     uint64_t hit_cap;
     int32_t be, bj;               // key packing widths
     int32_t tiers;                // 1: count entries by cost tier
+    int32_t few;                  // 1: few warps run, each as fast as it can (two row entries per lane)
     DevStats *stats;
     // walks whose row grows past esc_min entries (0: never) continue on a whole
     // block (k_leaf_wide) with the rest of their task's injections (past esc_dense where
