@@ -170,6 +170,13 @@ void scan_rec(const In *const *inp, uint64_t *const *outp, int64_t N, uint64_t *
 // RS_SMALL pairs one block does all passes in shared memory in one launch (the
 // sorts of a small search were 5 passes of 3 launches, 24 us a pass).
 constexpr int RS_T = 256, RS_I = 16, RS_TILE = RS_T * RS_I;
+// Up to AE_RS_SPLIT pairs tiles of half the size are taken: a pass lasts as long
+// as the few tiles an SM has one after the other.  Merges of 8,193 / 100 k / 1 M /
+// 1.5 M records: 0.289 / 0.400 / 0.756 / 0.845 ms with half tiles, 0.313 / 0.431 /
+// 0.788 / 0.825 with full ones.
+#ifndef AE_RS_SPLIT
+#define AE_RS_SPLIT (1 << 20)
+#endif
 constexpr int RS_ST = 1024, RS_SI = 8, RS_SMALL = RS_ST * RS_SI;
 
 template <int T, int I>
@@ -181,14 +188,15 @@ struct RsSmem {
     uint32_t wsum[8];
 };
 
+template <int I>
 __global__ void __launch_bounds__(RS_T) k_rs_hist(const uint64_t *keys, int64_t N, int shift, uint32_t *hist,
                                                   int64_t ntiles) {
     __shared__ uint32_t cnt[256];
     cnt[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+    const int64_t base = (int64_t)blockIdx.x * (RS_T * I);
 #pragma unroll
-    for (int i = 0; i < RS_I; ++i) {
+    for (int i = 0; i < I; ++i) {
         const int64_t idx = base + i * RS_T + threadIdx.x;
         if (idx < N) atomicAdd(&cnt[(keys[idx] >> shift) & 255], 1u);
     }
@@ -253,30 +261,31 @@ __device__ __forceinline__ void rs_tile(RsSmem<T, I> &s, const uint64_t (&k)[I],
     __syncthreads();
 }
 
+template <int I>
 __global__ void __launch_bounds__(RS_T, 3) k_rs_scatter(const uint64_t *kin, const uint32_t *vin, uint64_t *kout,
                                                      uint32_t *vout, int64_t N, int shift, const uint64_t *offs,
                                                      int64_t ntiles) {
     extern __shared__ __align__(16) unsigned char rs_smem[];
-    RsSmem<RS_T, RS_I> &s = *reinterpret_cast<RsSmem<RS_T, RS_I> *>(rs_smem);
+    RsSmem<RS_T, I> &s = *reinterpret_cast<RsSmem<RS_T, I> *>(rs_smem);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    const int n = (int)min((int64_t)RS_TILE, N - base);
-    uint64_t k[RS_I];
-    uint32_t v[RS_I];
+    const int64_t base = (int64_t)blockIdx.x * (RS_T * I);
+    const int n = (int)min((int64_t)(RS_T * I), N - base);
+    uint64_t k[I];
+    uint32_t v[I];
 #pragma unroll
-    for (int i = 0; i < RS_I; ++i) {
-        const int x = wid * 32 * RS_I + i * 32 + lane;
+    for (int i = 0; i < I; ++i) {
+        const int x = wid * 32 * I + i * 32 + lane;
         k[i] = x < n ? kin[base + x] : 0;
         v[i] = x < n ? vin[base + x] : 0;
     }
     // where the tile's pairs of each digit go
     const uint64_t out0 = offs[(int64_t)threadIdx.x * ntiles + blockIdx.x];
-    rs_tile<RS_T, RS_I>(s, k, v, n, shift);
+    rs_tile<RS_T, I>(s, k, v, n, shift);
     uint64_t *out = reinterpret_cast<uint64_t *>(&s.wcnt[0][0]);   // no longer needed
     out[threadIdx.x] = out0 - s.first[threadIdx.x];
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < RS_I; ++i) {
+    for (int i = 0; i < I; ++i) {
         const int x = i * RS_T + threadIdx.x;
         if (x >= n) break;
         const uint64_t key = s.key[x];
@@ -2038,10 +2047,37 @@ void ae_scan_u32(const uint32_t *const *in, uint64_t *const *out, int W, int64_t
 }
 
 int64_t ae_sort_tmp_words(int64_t N) {
-    int64_t ntiles = (N + RS_TILE - 1) / RS_TILE;
+    // enough for any number of pairs up to N (short lists take smaller tiles)
+    const int64_t half = std::min<int64_t>(N, AE_RS_SPLIT);
+    const int64_t ntiles = std::max((N + RS_TILE - 1) / RS_TILE, (half + RS_TILE / 2 - 1) / (RS_TILE / 2));
     int64_t h = 256 * ntiles;
     // hist (u32, packed two per word) + offsets (u64) + scan tmp
     return (h + 1) / 2 + h + ae_scan_tmp_words(h, 1) + 8;
+}
+
+template <int I>
+int rs_passes(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_t N, int bits, uint64_t *tmp, cudaStream_t st) {
+    const int smem = (int)sizeof(RsSmem<RS_T, I>);
+    cudaFuncSetAttribute(k_rs_scatter<I>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int64_t ntiles = (N + RS_T * I - 1) / (RS_T * I);
+    const int64_t h = 256 * ntiles;
+    uint32_t *hist = reinterpret_cast<uint32_t *>(tmp);
+    uint64_t *offs = tmp + (h + 1) / 2;
+    uint64_t *stmp = offs + h;
+    int which = 0;
+    for (int shift = 0; shift < bits; shift += 8) {
+        uint64_t *ki = which ? k1 : k0, *ko = which ? k0 : k1;
+        uint32_t *vi = which ? v1 : v0, *vo = which ? v0 : v1;
+        ++g_launches;
+        k_rs_hist<I><<<(unsigned)ntiles, RS_T, 0, st>>>(ki, N, shift, hist, ntiles);
+        const uint32_t *in[1] = {hist};
+        uint64_t *out[1] = {offs};
+        scan_rec<uint32_t, 1>(in, out, h, nullptr, stmp, st);
+        ++g_launches;
+        k_rs_scatter<I><<<(unsigned)ntiles, RS_T, smem, st>>>(ki, vi, ko, vo, N, shift, offs, ntiles);
+        which ^= 1;
+    }
+    return which;
 }
 
 int ae_radix_sort(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_t N, int bits, uint64_t *tmp,
@@ -2054,27 +2090,8 @@ int ae_radix_sort(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_
         k_rs_small<<<1, RS_ST, smem, st>>>(k0, v0, (int)N, bits);
         return 0;
     }
-    const int smem = (int)sizeof(RsSmem<RS_T, RS_I>);
-    cudaFuncSetAttribute(k_rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    const int64_t ntiles = (N + RS_TILE - 1) / RS_TILE;
-    const int64_t h = 256 * ntiles;
-    uint32_t *hist = reinterpret_cast<uint32_t *>(tmp);
-    uint64_t *offs = tmp + (h + 1) / 2;
-    uint64_t *stmp = offs + h;
-    int which = 0;
-    for (int shift = 0; shift < bits; shift += 8) {
-        uint64_t *ki = which ? k1 : k0, *ko = which ? k0 : k1;
-        uint32_t *vi = which ? v1 : v0, *vo = which ? v0 : v1;
-        ++g_launches;
-        k_rs_hist<<<(unsigned)ntiles, RS_T, 0, st>>>(ki, N, shift, hist, ntiles);
-        const uint32_t *in[1] = {hist};
-        uint64_t *out[1] = {offs};
-        scan_rec<uint32_t, 1>(in, out, h, nullptr, stmp, st);
-        ++g_launches;
-        k_rs_scatter<<<(unsigned)ntiles, RS_T, smem, st>>>(ki, vi, ko, vo, N, shift, offs, ntiles);
-        which ^= 1;
-    }
-    return which;
+    return N <= AE_RS_SPLIT ? rs_passes<RS_I / 2>(k0, v0, k1, v1, N, bits, tmp, st)
+                            : rs_passes<RS_I>(k0, v0, k1, v1, N, bits, tmp, st);
 }
 
 void ae_encode_queries(const uint8_t *ascii, uint8_t *codes, int64_t total, int alphabet, int *bad,
