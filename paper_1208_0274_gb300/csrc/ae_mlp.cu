@@ -35,7 +35,8 @@ constexpr int NORM_XMU = 0, NORM_XISD = NIN, NORM_YMU = 2 * NIN, NORM_YSD = 2 * 
 // B(k, n) = B[k*sbk + n*sbn] (fp32 in memory, rounded to bf16 for the
 // product, fp32 accumulate).  Epilogue per element: + bias[n]; Z = that value
 // (pre-activation); zeroed where mask <= 0; relu; stored to C (ld ldc).  One
-// warp owns a 16 x 16 tile (two m16n8k16 products per k step of 16).
+// warp owns a 16 x 16 tile (two m16n8k16 products per k step of 16), or 16 x 32 where
+// there are many rows.
 //
 // Split K: the weight gradients are products with a small output (at most
 // 128 x 128) and K = the batch rows, which a few warps would walk alone.  With
@@ -45,10 +46,11 @@ constexpr int NORM_XMU = 0, NORM_XISD = NIN, NORM_YMU = 2 * NIN, NORM_YSD = 2 * 
 // scheduling.
 //
 // A training step of 64 rows is a chain of small products, each bound by the
-// latency of its loads and its launch.  So a warp loads GEMM_KU k steps' operands
+// latency of its loads and its launch.  So a warp loads four k steps' operands
 // together, its tile is small (more warps), and products that wait for the same
-// input share a launch (two GemmArgs), 9 launches a step instead of 17: 82 us a
-// step with one k step in flight and 16 x 32 tiles, 59 us so.
+// input share a launch (two GemmArgs), 10 launches a step instead of 15 (13 at 128
+// rows, whose weight gradients split their sums): 82 us a step with one k step in
+// flight and 16 x 32 tiles, 59 us so.
 
 struct GemmArgs {
     const float *A;
@@ -69,8 +71,13 @@ struct GemmPair {
     GemmArgs a[2];
 };
 
-constexpr int GEMM_NT = 2;      // n8 sub-tiles per warp
-constexpr int GEMM_KU = 4;      // k steps whose operands are loaded together
+// NT: n8 sub-tiles per warp, KU: k steps whose operands are loaded together.  From
+// GEMM_WIDE tiles of 16 x 16 on (8,192 rows by 128 columns) there are warps enough to
+// hide the loads and the operands' traffic counts: a warp then takes 16 x 32, one k step
+// at a time.  Forward of 16,384 / 262,144 rows: 0.081 / 0.75 ms, with the small tile
+// 0.102 / 0.955 (16 x 32 with two k steps 0.097 / 0.78; 16 x 64 with one 0.084 / 0.72
+// but gradients of 262,144 rows 4.65 ms against 4.44).
+constexpr int64_t GEMM_WIDE = 4096;
 constexpr int GEMM_WARPS = 4;
 constexpr int GEMM_KSPLIT_MAX = 64;
 constexpr int GEMM_TARGET_BLOCKS = 2 * 152;
@@ -88,6 +95,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+template <int GEMM_NT, int GEMM_KU>
 __global__ void __launch_bounds__(GEMM_WARPS * 32) k_gemm(GemmPair pr) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
@@ -194,7 +202,7 @@ __global__ void k_gemm_reduce(GemmArgs a) {
     }
 }
 
-void plan(GemmArgs &a) {
+void plan(GemmArgs &a, int nt) {
     const int64_t tiles_m = (a.M + 15) / 16;
     // blocks of 16 x 128, the unit that the number of chunks is chosen by
     const int64_t blocks = (tiles_m * ((a.N + 31) / 32) + 3) / 4;
@@ -206,7 +214,7 @@ void plan(GemmArgs &a) {
     const int steps_per = (ksteps + nsplit - 1) / nsplit;
     a.kchunk = 16 * std::max(steps_per, 1);
     a.nsplit = std::max(1, (a.K + a.kchunk - 1) / a.kchunk);
-    a.blocks = (int)((tiles_m * ((a.N + 8 * GEMM_NT - 1) / (8 * GEMM_NT)) + GEMM_WARPS - 1) / GEMM_WARPS);
+    a.blocks = (int)((tiles_m * ((a.N + 8 * nt - 1) / (8 * nt)) + GEMM_WARPS - 1) / GEMM_WARPS);
 }
 
 // one product, or two that do not depend on each other
@@ -214,10 +222,16 @@ void gemm(GemmArgs a, cudaStream_t st, const GemmArgs *b = nullptr) {
     GemmPair pr{};
     pr.a[0] = a;
     if (b) pr.a[1] = *b;
-    plan(pr.a[0]);
-    if (b) plan(pr.a[1]);
+    int64_t tiles = 0;   // of 16 x 16
+    for (const GemmArgs &x : pr.a) tiles += (int64_t)((x.M + 15) / 16) * ((x.N + 15) / 16);
+    const bool wide = tiles >= GEMM_WIDE;
+    const int nt = wide ? 4 : 2;
+    plan(pr.a[0], nt);
+    if (b) plan(pr.a[1], nt);
+    const int blocks = pr.a[0].blocks * pr.a[0].nsplit + pr.a[1].blocks * pr.a[1].nsplit;
     ++g_launches;
-    k_gemm<<<pr.a[0].blocks * pr.a[0].nsplit + pr.a[1].blocks * pr.a[1].nsplit, GEMM_WARPS * 32, 0, st>>>(pr);
+    if (wide) k_gemm<4, 1><<<blocks, GEMM_WARPS * 32, 0, st>>>(pr);
+    else k_gemm<2, 4><<<blocks, GEMM_WARPS * 32, 0, st>>>(pr);
     for (const GemmArgs &x : pr.a)
         if (x.nsplit > 1) {
             ++g_launches;
