@@ -191,8 +191,8 @@ void ae_options_default(ae_options *opt);
  * for protein) with sampled ranks, the text-end array (entry h = end position
  * in T of the substrings whose reverse prefixes suffix h), and the forward
  * text (Section 2.3 and Section 5 (1)-(3)).  The suffix array is built on the
- * current CUDA device (ae_suffix_array_device, about 45 bytes of device memory
- * per letter while it runs, beside the index's own 5.5), and the arrays are
+ * current CUDA device (ae_suffix_array_device, about 33 bytes of device memory
+ * per letter while it runs, beside 5 of the index's own), and the arrays are
  * filled from it there; the host keeps no copy.
  * Errors: AE_EINVAL (n < 1, unknown letter, bad alphabet), AE_EUNSUPPORTED
  * (n >= 2^31 - 1), AE_ENOMEM, AE_ECUDA. */
@@ -335,7 +335,7 @@ ae_status ae_suffix_array(const uint8_t *codes, int64_t n, int32_t sigma, int32_
  * others stay, as in Larsson & Sadakane 2007).  Rounds stop when every rank is
  * distinct.
  * d_codes and d_sa are device memory: codes in [0, sigma), 1 <= sigma <= 255,
- * 0 <= n < 2^31 - 2.  The call allocates and frees about 45 bytes of device
+ * 0 <= n < 2^31 - 2.  The call allocates and frees about 33 bytes of device
  * memory per letter, and returns once `stream` (NULL = the legacy default
  * stream) has finished its work.
  * Errors: AE_EINVAL (NULL pointer, sigma out of range, a code >= sigma),

@@ -24,7 +24,7 @@ using namespace aedev;
 
 struct BuildArgs {
     const uint8_t *s;        // codes of the text, or of the joined collection (0: separator, letters + 1)
-    const int32_t *sa;       // J + 1 entries, suffix array of s reversed and the sentinel
+    const int32_t *sa;       // J + 1 entries, suffix array of s reversed and the sentinel (may be tend itself)
     int64_t J;               // letters and separators
     const int64_t *starts;   // collections: first positions of the sequences in the text
     int32_t nseq;            // 0: one text

@@ -331,14 +331,14 @@ const uint32_t *dom_table(const ae_index *cidx, int d0, cudaStream_t st) {
     return t;
 }
 
-// Device memory of the index's arrays, sized by idx->host
-ae_status alloc_index(ae_index *idx) {
+// Device memory of the index's arrays `which` (bit k: array k in file order), sized by
+// idx->host; those that are there already stay
+ae_status alloc_index(ae_index *idx, unsigned which = 31u) {
     const HostIndex &h = idx->host;
     void **const d[5] = {&idx->d_occ, &idx->d_tend, &idx->d_text, &idx->d_sep, &idx->d_ends};
     if (cudaGetDevice(&idx->device) != cudaSuccess) return AE_ECUDA;
-    idx->device_bytes = 0;
     for (int k = 0; k < 5; ++k) {
-        if (!h.bytes(k)) continue;
+        if (!h.bytes(k) || !((which >> k) & 1u) || *d[k]) continue;
         if (cudaMalloc(d[k], h.bytes(k)) != cudaSuccess) {
             cudaGetLastError();
             return AE_ENOMEM;
@@ -1707,7 +1707,9 @@ ae_status build_index(ae_index *idx, const uint8_t *text, int64_t n, int32_t alp
     };
     ae_status res = AE_OK;
     try {
-        res = alloc_index(idx);
+        // text ends, letters and sequence ends first, the others when the suffix array's
+        // working memory is free again
+        res = alloc_index(idx, 2u | 4u | 16u);
         if (res != AE_OK) throw ae_error{res};
         // letters (the ASCII text goes through the text-end array's memory)
         uint8_t *ascii = (uint8_t *)idx->d_tend, *codes = (uint8_t *)idx->d_text;
@@ -1730,17 +1732,19 @@ ae_status build_index(ae_index *idx, const uint8_t *text, int64_t n, int32_t alp
             d_starts = (int64_t *)alloc(sizeof(int64_t) * (size_t)nseq);
             CU(cudaMemsetAsync(joined, 0, (size_t)J, st));
             CU(cudaMemsetAsync(idx->d_ends, 0, h.bytes(4), st));
-            CU(cudaMemsetAsync(idx->d_sep, 0, h.bytes(3), st));
             CU(cudaMemcpyAsync(d_starts, starts, sizeof(int64_t) * (size_t)nseq, cudaMemcpyHostToDevice, st));
             ae_join_sequences(codes, n, d_starts, nseq, joined, (uint32_t *)idx->d_ends, st);
             s = joined;
         }
-        int32_t *sa = (int32_t *)alloc(sizeof(int32_t) * (size_t)N);
+        int32_t *sa = (int32_t *)idx->d_tend;   // each entry is replaced by its text end
         res = ae_sa_doubling(s, J, sigma + (nseq > 0 ? 1 : 0), 1, sa, nullptr, st);
+        if (res != AE_OK) throw ae_error{res};
+        res = alloc_index(idx);
         if (res != AE_OK) throw ae_error{res};
         uint32_t *cnt = (uint32_t *)alloc(sizeof(uint32_t) * (size_t)(sigma + 1) * (size_t)h.nblocks);
         uint64_t *tmp = (uint64_t *)alloc(8 * (size_t)ae_fill_tmp_words(h.nblocks));
         CU(cudaMemsetAsync(idx->d_occ, 0, h.bytes(0), st));
+        if (nseq > 0) CU(cudaMemsetAsync(idx->d_sep, 0, h.bytes(3), st));
         ae_fill_index(sigma, s, sa, J, d_starts, nseq, (uint32_t *)idx->d_occ, (uint32_t *)idx->d_sep,
                       (int32_t *)idx->d_tend, h.nblocks, cnt, tmp, ds->totals, &ds->dollar, &ds->bad_sa, st);
         CU(cudaGetLastError());

@@ -2218,7 +2218,7 @@ void ae_unique_write(const uint64_t *key, const int32_t *score, int64_t N, const
 // only: places past the text read 0), and a stable radix sort orders them.  A
 // suffix's rank is the place of the first suffix with its key.  From then on
 // only the suffixes that share their key are sorted (as Larsson & Sadakane,
-// 2007, do): by (rank, what follows h letters on), into the places their groups
+// 2007, do): by (group, what follows h letters on), into the places their groups
 // hold, which orders them by 2 h letters; new groups split and ranks follow.
 // What follows h letters on is the rank there; a suffix that ends within h
 // letters comes before all others of its key, shorter ones first.
@@ -2226,8 +2226,11 @@ void ae_unique_write(const uint64_t *key, const int32_t *score, int64_t N, const
 // L is chosen so that about 1% of the suffixes of an i.i.d. text share a key:
 // sorting these again costs less than a pass over all of them for longer keys.
 // 10^7 letters: 4 passes over all suffixes and one round of some 10^4 of them
-// (1.6 ms), where a 63-bit key and a 48-bit pair key for every suffix took 14
-// passes (4.5 ms).
+// (1.44 ms), where a 63-bit key and a 48-bit pair key for every suffix took 14
+// passes (4.5 ms).  Only groups of several suffixes are numbered, so a text of few
+// such groups sorts short pairs: 5 * 10^6 equal letters 8.7 ms, 12.8 with ranks as
+// group numbers.  The flags and sums of a round lie over the sorted keys and the
+// free pair, so that no other array of the text's length is needed.
 
 namespace {
 
@@ -2260,50 +2263,66 @@ __global__ void __launch_bounds__(256) k_sa_first_keys(const uint8_t *s, int64_t
     }
 }
 
-// Of a sorted list of keys: 1 where a key starts a group, and 1 where it shares
-// its key with a neighbour
-__global__ void k_sa_groups(const uint64_t *keys, int64_t N, uint32_t *head, uint32_t *tied) {
+// Of a sorted list of keys: whether a key is the first of several equal ones, and
+// (upper half) whether it shares its value with a neighbour.  One scan adds up both.
+__global__ void k_sa_groups(const uint64_t *keys, int64_t N, uint64_t *flags) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t k = keys[p];
-        const bool h = p == 0 || keys[p - 1] != k;
-        head[p] = h ? 1u : 0u;
-        tied[p] = !h || (p + 1 < N && keys[p + 1] == k) ? 1u : 0u;
+        const bool before = p > 0 && keys[p - 1] == k, after = p + 1 < N && keys[p + 1] == k;
+        flags[p] = (uint64_t)(!before && after) | (uint64_t)(before || after) << 32;
     }
 }
 
-// The place in the suffix array of each group's first suffix, by group; the
+// The place in the suffix array of the first suffix of each group of several; the
 // list's k-th element stands at place pos[k] (NULL: at k)
-__global__ void k_sa_starts(const uint32_t *head, const uint64_t *group, const uint32_t *pos, int64_t N,
+__global__ void k_sa_starts(const uint64_t *flags, const uint64_t *sums, const uint32_t *pos, int64_t N,
                             uint32_t *start) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
-        if (head[p]) start[group[p]] = pos ? pos[p] : (uint32_t)p;
+        if ((uint32_t)flags[p]) start[(uint32_t)sums[p]] = pos ? pos[p] : (uint32_t)p;
 }
 
-// The list's suffixes at their places with their ranks, and the places of those
-// still tied as the next list
-__global__ void k_sa_place(const uint32_t *vals, const uint32_t *head, const uint64_t *group, const uint32_t *start,
-                           const uint32_t *pos, const uint32_t *tied, const uint64_t *tied_off, int64_t T, int64_t N,
-                           uint32_t *sa, uint32_t *rank, uint32_t *next, int *bad) {
+// The list's suffixes at their places with their ranks.  The flags of an element
+// that still shares its key become its group's number with its place in the
+// upper half, vals[p] becomes 1 there and 0 elsewhere.
+__global__ void k_sa_place(uint32_t *vals, uint64_t *flags, const uint64_t *sums, const uint32_t *start,
+                           const uint32_t *pos, int64_t T, int64_t N, uint32_t *sa, uint32_t *rank, int *bad) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < T; p += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t i = vals[p], at = pos ? pos[p] : (uint32_t)p;
+        const uint64_t f = flags[p];
+        const bool tied = f >> 32;
+        vals[p] = tied;
+        // the sum counts the groups that start before p: the element's own is that, or one less
+        const uint32_t g = (uint32_t)sums[p] + (uint32_t)f - 1;
+        if (tied) flags[p] = (uint64_t)g | ((uint64_t)at << 32);
         if ((int64_t)i >= N || (int64_t)at >= N) {
             *bad = 2;
             continue;
         }
         sa[at] = i;
-        // group[] counts the heads before p: the element's own group is that, or one less
-        rank[i] = start[group[p] + head[p] - 1];
-        if (tied[p]) next[tied_off[p]] = at;
+        rank[i] = tied ? start[g] : at;
     }
 }
 
-// keys of the tied suffixes (at places pos[0..T)) for the 2 h-letter order
-__global__ void k_sa_pair_keys(const uint32_t *sa, const uint32_t *pos, const uint32_t *rank, int64_t T, int64_t n,
-                               int64_t h, int rb, uint64_t *keys, uint32_t *vals) {
+// The next list: places and groups of the elements that are still tied
+__global__ void k_sa_next(const uint32_t *tied, const uint64_t *sums, const uint64_t *group, int64_t T, uint32_t *pos,
+                          uint32_t *ord) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < T; p += (int64_t)gridDim.x * blockDim.x)
+        if (tied[p]) {
+            const uint64_t o = sums[p] >> 32, g = group[p];
+            pos[o] = (uint32_t)(g >> 32);
+            ord[o] = (uint32_t)g;
+        }
+}
+
+// keys of the tied suffixes (at places pos[0..T), in groups ord[0..T)) for the
+// 2 h-letter order.  Groups are numbered along the list, in the order of their
+// ranks: a text of few groups (one letter, a period) has short keys.
+__global__ void k_sa_pair_keys(const uint32_t *sa, const uint32_t *pos, const uint32_t *ord, const uint32_t *rank, int64_t T,
+                               int64_t n, int64_t h, int rb, uint64_t *keys, uint32_t *vals) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < T; p += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t i = sa[pos[p]];
         const uint64_t second = i + h <= n ? (uint64_t)rank[i + h] + (uint64_t)h : (uint64_t)(n - i);
-        keys[p] = ((uint64_t)rank[i] << rb) | second;
+        keys[p] = ((uint64_t)ord[p] << rb) | second;
         vals[p] = i;
     }
 }
@@ -2325,21 +2344,22 @@ ae_status ae_sa_doubling(const uint8_t *d_codes, int64_t n, int sigma, int rever
     int L = 1;
     for (double words = sigma; words < 100.0 * (double)N && (L + 1) * b <= 64; words *= std::max(sigma, 2)) ++L;
     L = std::min(64, (L * b + 7) / 8 * 8) / b;
-    // one allocation for all buffers (ten of them cost 0.5 ms)
-    const int64_t tmp_words = std::max(ae_sort_tmp_words(N), ae_scan_tmp_words(N, 2) + N + (N + 1) / 2);
-    const int64_t words = 2 * N + tmp_words + 2 + (4 * N + 1 + 1) / 2 + 1 + (N + 7) / 8;   // of eight bytes
+    // one allocation for all buffers (ten of them cost 0.5 ms): 32 bytes a letter and the sort's
+    const int64_t tmp_words = std::max(ae_sort_tmp_words(N), ae_scan_tmp_words(N, 1));
+    const int64_t words = 2 * N + tmp_words + 2 + 2 * N;   // of eight bytes
     uint64_t *mem = nullptr;
     ae_status res = AE_OK;
     if (cudaMalloc(&mem, sizeof(uint64_t) * (size_t)words) != cudaSuccess) {
         cudaGetLastError();
         return AE_ENOMEM;
     }
+    // total: groups of several and (upper half) tied suffixes, then an error flag
     uint64_t *k0 = mem, *k1 = k0 + N, *tmp = k1 + N, *total = tmp + tmp_words;
     uint32_t *v0 = reinterpret_cast<uint32_t *>(total + 2), *v1 = v0 + N, *rank = v1 + N, *pos = rank + N;
-    int *bad = reinterpret_cast<int *>(pos + N);
-    uint8_t *s = reinterpret_cast<uint8_t *>(bad + 1);
+    int *bad = reinterpret_cast<int *>(total + 1);
+    uint8_t *s = reinterpret_cast<uint8_t *>(k1);   // until the first sort
     int h_bad = 0;
-    if (res == AE_OK && cudaMemsetAsync(bad, 0, sizeof(int), st) != cudaSuccess) res = AE_ECUDA;
+    if (cudaMemsetAsync(total, 0, 2 * sizeof(uint64_t), st) != cudaSuccess) res = AE_ECUDA;
     if (res == AE_OK) {
         g_launches += 2;
         k_sa_letters<<<grid_for(n, 256), 256, 0, st>>>(d_codes, n, reversed, sigma, s, bad);
@@ -2363,59 +2383,46 @@ ae_status ae_sa_doubling(const uint8_t *d_codes, int64_t n, int sigma, int rever
             std::swap(vr, vf);
         }
         if (rounds) ++*rounds;
-        // head and tied flags in the free values, their sums in the free keys and tmp
-        uint32_t *head = vf, *tied = reinterpret_cast<uint32_t *>(tmp);
-        uint64_t *group = kf, *tied_off = tmp + (T + 1) / 2;
-        uint64_t *scan_tmp = tied_off + T;
-        if ((T + 1) / 2 + T + ae_scan_tmp_words(T, 2) > tmp_words) {
-            res = AE_ECUDA;   // sized above
-            break;
-        }
-        g_launches += 3;
-        k_sa_groups<<<grid_for(T, 256), 256, 0, st>>>(kr, T, head, tied);
-        const uint32_t *in[2] = {head, tied};
-        uint64_t *out[2] = {group, tied_off};
-        ae_scan_u32(in, out, 2, T, total, scan_tmp, st);
-        // group starts: over the sorted keys, which are done with
-        uint32_t *start = reinterpret_cast<uint32_t *>(kr);
+        // flags in the free keys, their sums over the sorted ones, which are done with; group
+        // starts, and then the next list's groups, in the free values
+        uint64_t *flags = kf, *sum = kr;
         const uint32_t *at = all ? nullptr : pos;
-        k_sa_starts<<<grid_for(T, 256), 256, 0, st>>>(head, group, at, T, start);
-        // the next list's places: the keys' second half
-        uint32_t *next = start + N;
-        k_sa_place<<<grid_for(T, 256), 256, 0, st>>>(vr, head, group, start, at, tied, tied_off, T, N, sa, rank, next, bad);
-        uint64_t sums[2] = {0, 0};
+        g_launches += 4;
+        k_sa_groups<<<grid_for(T, 256), 256, 0, st>>>(kr, T, flags);
+        const uint64_t *in[1] = {flags};
+        uint64_t *out[1] = {sum};
+        scan_rec<uint64_t, 1>(in, out, T, total, tmp, st);
+        k_sa_starts<<<grid_for(T, 256), 256, 0, st>>>(flags, sum, at, T, vf);
+        k_sa_place<<<grid_for(T, 256), 256, 0, st>>>(vr, flags, sum, vf, at, T, N, sa, rank, bad);
+        k_sa_next<<<grid_for(T, 256), 256, 0, st>>>(vr, sum, flags, T, pos, vf);
+        uint64_t back[2] = {0, 0};
         if (cudaGetLastError() != cudaSuccess ||
-            cudaMemcpyAsync(sums, total, 2 * sizeof(uint64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaMemcpyAsync(back, total, 2 * sizeof(uint64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) {
             res = AE_ECUDA;
             break;
         }
-        if (h_bad || sums[0] < 1 || (int64_t)sums[0] > T || (int64_t)sums[1] > T) {
+        const int64_t groups = (int64_t)(uint32_t)back[0], tied = (int64_t)(back[0] >> 32);
+        if (back[1] || tied > T || 2 * groups > tied || (tied > 0 && groups < 1)) {
             res = AE_ECUDA;   // not a permutation: an internal error
             break;
         }
-        if (sums[1] == 0) break;
+        if (tied == 0) break;
         if (!all && h / 2 >= N) {   // a round at h >= N orders everything left by its length
             res = AE_ECUDA;
             break;
         }
-        T = (int64_t)sums[1];
+        T = tied;
         all = false;
-        if (cudaMemcpyAsync(pos, next, sizeof(uint32_t) * T, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
-            res = AE_ECUDA;
-            break;
-        }
         const int rb = sa_bits_for((uint64_t)(N - 1 + h));
-        bits = rb + sa_bits_for((uint64_t)(N - 1));
+        bits = rb + sa_bits_for((uint64_t)(groups - 1));
         if (bits > 64) {
             res = AE_EUNSUPPORTED;
             break;
         }
         ++g_launches;
-        k_sa_pair_keys<<<grid_for(T, 256), 256, 0, st>>>(sa, pos, rank, T, n, h, rb, kf, vf);
+        k_sa_pair_keys<<<grid_for(T, 256), 256, 0, st>>>(sa, pos, vf, rank, T, n, h, rb, kf, vr);
         std::swap(kr, kf);
-        std::swap(vr, vf);
         h *= 2;
     }
     if (res == AE_OK && cudaStreamSynchronize(st) != cudaSuccess) res = AE_ECUDA;
