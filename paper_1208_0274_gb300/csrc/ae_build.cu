@@ -40,7 +40,7 @@ struct BuildArgs {
 __device__ __forceinline__ int32_t seq_of(const int64_t *starts, int32_t n, int64_t x, bool joined) {
     int32_t lo = 0, hi = n;
     while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
+        const int32_t mid = lo + ((hi - lo) >> 1);   // lo + hi may pass 2^31
         if (starts[mid] + (joined ? mid : 0) <= x) lo = mid; else hi = mid;
     }
     return lo;
@@ -54,7 +54,7 @@ __global__ void k_join(const uint8_t *codes, int64_t n, const int64_t *starts, i
 }
 
 __global__ void k_seq_ends(const int64_t *starts, int32_t nseq, int64_t n, uint32_t *ends) {
-    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < nseq; k += gridDim.x * blockDim.x) {
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nseq; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t e = k + 1 < nseq ? starts[k + 1] : n;
         if (e > starts[k]) atomicOr(&ends[(e - 1) >> 5], 1u << ((e - 1) & 31));
     }
