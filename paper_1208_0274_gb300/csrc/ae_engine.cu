@@ -1321,7 +1321,10 @@ void Search::leaf_phase(int64_t ninj) {
     // the counters before the sweep: one that is run again counts once
     ensure(w->stats_keep, sizeof(DevStats), st);
     CU(cudaMemcpyAsync(w->stats_keep.p, w->stats.p, sizeof(DevStats), cudaMemcpyDeviceToDevice, st));
-    for (int attempt = 0; attempt < 12; ++attempt) {
+    // Row buffers grow fourfold a time from at least 64 to at most 2^28 entries, those of
+    // the warps and those of the blocks each by itself (11 + 11 times), and the hit buffer
+    // once or twice.
+    for (int attempt = 0; attempt < 26; ++attempt) {
         if (attempt) CU(cudaMemcpyAsync(w->stats.p, w->stats_keep.p, sizeof(DevStats), cudaMemcpyDeviceToDevice, st));
         ensure(w->scratch, (size_t)ae_leaf_scratch_words(w->leaf_cap, nwarps) * 4, st);
         if (esc_max > 0) {
