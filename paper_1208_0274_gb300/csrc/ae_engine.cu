@@ -479,6 +479,7 @@ struct Search {
     int d0;
     int64_t nhits = 0;        // point hits accumulated in w->hkey/hscore
     bool one_query = true;    // the current batch holds columns of one query only
+    bool no_pack = false;     // the current batch's memory does not hold the packed layout's regions
     double batch_hint = -1;   // expected sweep hit records of the current batch (< 0: no hints)
     ae_stats stats;
     // the frontier's nodes and entries (its arenas may also hold unused ends of regions)
@@ -527,6 +528,7 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
     const int sigma = ix.sigma;
     const int64_t batch_hits0 = nhits;
     one_query = items.front().qid == items.back().qid;
+    no_pack = false;
     const int nitems = (int)items.size();
     ensure(w->items, sizeof(WorkItem) * items.size(), st);
     CU(cudaMemcpyAsync(w->items.p, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, st));
@@ -932,7 +934,7 @@ void Search::dna_args(DnaRowsArgs &da, int cur, int64_t lf_ent_base, int64_t lf_
 // While levels grow, only as many are launched as the arenas
 // will most likely hold.
 int Search::chain_levels(int depth, int64_t max_depth) const {
-    if (opt.row_layout != 0 || g_arena || opt.workspace_limit > 0) return 1;
+    if (opt.row_layout != 0 || g_arena || opt.workspace_limit > 0 || no_pack) return 1;
     if (live_ent > AE_PACK_ROW_AVG * live_nodes) return 1;
     const bool growing = !dna_ratio_ok || dna_ratio[0] > 0.9;
     int64_t k = live_ent <= (1 << 16) ? 8 : live_ent <= (growing ? 1 << 20 : 1 << 22) ? (growing ? 3 : 8) : 1;
@@ -1041,7 +1043,7 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
     const int nxt = cur ^ 1;
     // nodes per task: 32 (one per lane) unless the level is too small to give
     // every resident warp a few tasks
-    const bool packed = opt.row_layout == 0 && !g_arena && live_ent <= AE_PACK_ROW_AVG * live_nodes;
+    const bool packed = opt.row_layout == 0 && !g_arena && !no_pack && live_ent <= AE_PACK_ROW_AVG * live_nodes;
     const int64_t warps = packed ? (int64_t)num_sms * ae_rows_pack_blocks_per_sm() * ae_rows_pack_warps_per_block()
                                  : (int64_t)num_sms * ae_rows_dna_blocks_per_sm() * ae_rows_dna_warps_per_block();
     const int npt = packed ? ae_rows_pack_task_nodes(F, live_nodes, live_ent, warps)
@@ -1075,7 +1077,8 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
         const int64_t rn = want[2] / (8 * warps);
         if (rn >= 32) region_node = (uint32_t)std::min<int64_t>(rn, 1024);
     }
-    const int64_t slack_ent = 4 * warps * (int64_t)region_ent, slack_node = warps * (int64_t)region_node;
+    const int64_t takers = std::min<int64_t>(warps, (F + npt - 1) / npt);   // warps with a task: the others take no region
+    const int64_t slack_ent = 4 * takers * (int64_t)region_ent, slack_node = takers * (int64_t)region_node;
     // grow ahead only outside the fixed arena, and only as far as memory allows:
     // a capacity that falls short costs one more run of the level
     auto grow = [&](int64_t fe, int64_t le, int64_t fn, int64_t ln, int64_t h, bool exact) {
@@ -1170,7 +1173,17 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
         // how the packed layout's regions fall differs a little from run to run
         if (again > (packed ? 4 : 1)) throw ae_error{AE_ECUDA};
         ++dna_retries;
-        grow((int64_t)hc.fr_ent + again * slack_ent, lf_ent, (int64_t)hc.fr_node + again * slack_node, lf_node, hits, true);
+        try {
+            grow((int64_t)hc.fr_ent + again * slack_ent, lf_ent, (int64_t)hc.fr_node + again * slack_node, lf_node, hits,
+                 true);
+        } catch (const ae_error &e) {
+            // no room for the unused ends of the packed layout's regions: this level and the
+            // batch's next ones in the other layouts, which write their rows without gaps
+            if (e.st != AE_ENOMEM || !packed) throw;
+            no_pack = true;
+            dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base, d_items);
+            return;
+        }
         run();
         if ((int64_t)(packed ? hc.n_ent : hc.fr_ent) != n_ent || (int64_t)(packed ? hc.n_node : hc.fr_node) != n_node ||
             (int64_t)hc.lf_ent - lf_ent_base != lf_ent || (int64_t)hc.lf_node - lf_node_base != lf_node ||
@@ -1318,6 +1331,8 @@ void Search::leaf_phase(int64_t ninj) {
     const int32_t wide = choose ? 32 : opt.leaf_wide_rows;
     const int32_t esc_min = (g_arena || opt.tier_stats) ? 0 : wide;
     const int32_t esc_max = esc_min > 0 ? AE_LEAF_WIDE_SLOTS : 0;
+    // (a search with small row buffers has little room for its workspace)
+    const int64_t pool = std::min<int64_t>(AE_LEAF_WIDE_POOL, 1024 * (int64_t)opt.leaf_capacity);
     // the counters before the sweep: one that is run again counts once
     ensure(w->stats_keep, sizeof(DevStats), st);
     CU(cudaMemcpyAsync(w->stats_keep.p, w->stats.p, sizeof(DevStats), cudaMemcpyDeviceToDevice, st));
@@ -1330,7 +1345,7 @@ void Search::leaf_phase(int64_t ninj) {
         if (esc_max > 0) {
             ensure(w->esc, (size_t)esc_max * sizeof(EscWalk), st);
             ensure(w->esc_count, 24, st);
-            ensure(w->esc_pool, (size_t)AE_LEAF_WIDE_POOL * 12, st);
+            ensure(w->esc_pool, (size_t)pool * 12, st);
             ensure(w->wide_rows, (size_t)wide_blocks * 6 * (size_t)w->wide_cap * 4, st);
             CU(cudaMemsetAsync(w->esc_count.p, 0, 24, st));
         }
@@ -1383,7 +1398,7 @@ void Search::leaf_phase(int64_t ninj) {
             la.esc_count = ptr<unsigned long long>(w->esc_count);
             la.esc = ptr<EscWalk>(w->esc);
             la.esc_pool = ptr<int32_t>(w->esc_pool);
-            la.esc_pool_cap = AE_LEAF_WIDE_POOL;
+            la.esc_pool_cap = pool;
             la.wide_rows = ptr<int32_t>(w->wide_rows);
             la.wide_cap = w->wide_cap;
             la.wide_blocks = wide_blocks;
