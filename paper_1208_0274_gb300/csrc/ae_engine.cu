@@ -1910,7 +1910,7 @@ ae_status ae_index_save(const ae_index *idx, const char *path) {
         std::thread th;
         try {
             th = std::thread(fetch);
-        } catch (const std::system_error &) {
+        } catch (...) {   // no thread to be had: copied by this one first
             int dev = 0;
             cudaGetDevice(&dev);
             fetch();
