@@ -146,6 +146,8 @@ typedef struct {
                                  rerun of the sweep, never a result */
     int32_t tier_stats;       /* 1: count trie entries by cost tier into ae_stats.entries_tier
                                  (a few instructions per entry); 0: leave them 0 */
+    int32_t leaf_wide_auto;   /* 1 (default): while leaf_wide_rows has its default, 128, the library
+                                 chooses; 0: leaf_wide_rows is taken as given, 128 too */
     int64_t workspace_limit;  /* > 0: cap on the device bytes of the stream's workspace; a batch
                                  that would grow it further is searched as two halves (as after
                                  a failed device allocation; ae_stats.batch_splits); a single
@@ -172,15 +174,16 @@ typedef struct {
     int32_t fork_part;
     int32_t leaf_wide_rows;   /* a walk of the text-position sweep whose row grows past this many
                                  entries continues on a whole thread block (each step spread over
-                                 its threads) instead of one warp; 0: never.  The default, 128,
-                                 lets the library choose: 32 where the injected rows leave gaps
-                                 along the text, 1,024 (128 for the last walks) where they lie
-                                 at most positions.  The results are the same */
+                                 its threads) instead of one warp; 0: never.  With the
+                                 default, 128, and leaf_wide_auto 1 the library chooses: 32 where
+                                 a query's injected rows leave gaps along the text, 1,024 (128 for
+                                 the last walks) where they lie at most positions.  The results
+                                 are the same */
 } ae_options;
 
 /* Fill *opt with the defaults: qprefix_seed 1, leaf_segment 0, item_columns
  * 2^24, batch_columns 2^20, leaf_capacity 4096, profile 0, leaf_delay 8,
- * int16_limit 32000, hint_hits NULL, tier_stats 0, workspace_limit 0,
+ * int16_limit 32000, hint_hits NULL, tier_stats 0, leaf_wide_auto 1, workspace_limit 0,
  * general_rows 0, qprefix_domination 1, row_layout 0, fork_parts 1,
  * fork_part 0, leaf_wide_rows 128. */
 void ae_options_default(ae_options *opt);

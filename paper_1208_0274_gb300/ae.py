@@ -45,6 +45,7 @@ class ae_options(ctypes.Structure):
                 ("leaf_capacity", ctypes.c_int32), ("profile", ctypes.c_int32),
                 ("leaf_delay", ctypes.c_int32), ("int16_limit", ctypes.c_int32),
                 ("hint_hits", ctypes.c_void_p), ("tier_stats", ctypes.c_int32),
+                ("leaf_wide_auto", ctypes.c_int32),
                 ("workspace_limit", ctypes.c_int64), ("general_rows", ctypes.c_int32),
                 ("qprefix_domination", ctypes.c_int32), ("row_layout", ctypes.c_int32),
                 ("fork_parts", ctypes.c_int32), ("fork_part", ctypes.c_int32),
@@ -164,9 +165,12 @@ def ae_options_default():
 
 
 def make_options(hint_hits=None, **kw):
-    """ae_options with the given fields set.  hint_hits: per-query expected
-    sweep hit records (kept alive on the returned object)."""
+    """ae_options with the given fields set (a leaf_wide_rows that is given is
+    taken as it is).  hint_hits: per-query expected sweep hit records (kept alive
+    on the returned object)."""
     o = ae_options_default()
+    if kw.get("leaf_wide_rows") is not None:
+        kw.setdefault("leaf_wide_auto", 0)
     for k, v in kw.items():
         if v is not None:
             setattr(o, k, int(v))

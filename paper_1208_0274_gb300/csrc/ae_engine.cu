@@ -853,6 +853,9 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 #define AE_LEAF_WIDE_POOL (1 << 22)
 #endif
 
+// ae_options.leaf_wide_rows by default
+constexpr int32_t AE_LEAF_WIDE_DEFAULT = 128;
+
 // Row length at which a warp's walk moves to a block once the sweep's tasks are
 // all taken.  Dense injections make rows of hundreds of entries the rule, and
 // blocks walk those slower than the warps do together, so they take only the
@@ -1327,7 +1330,7 @@ void Search::leaf_phase(int64_t ninj) {
     // where they are dense every task walks a wide row and warps are the better use of
     // the chip (1 M residues, BLOSUM62, sweep: from 128 entries 127 ms, 512: 104,
     // 1,024: 69, never: 84), until the tasks run out (AE_LEAF_WIDE_TAIL)
-    const bool choose = opt.leaf_wide_rows == 128;
+    const bool choose = opt.leaf_wide_auto != 0 && opt.leaf_wide_rows == AE_LEAF_WIDE_DEFAULT;
     const int32_t wide = choose ? 32 : opt.leaf_wide_rows;
     const int32_t esc_min = (g_arena || opt.tier_stats) ? 0 : wide;
     const int32_t esc_max = esc_min > 0 ? AE_LEAF_WIDE_SLOTS : 0;
@@ -1828,7 +1831,8 @@ void ae_options_default(ae_options *opt) {
     opt->qprefix_domination = 1;
     opt->row_layout = 0;
     opt->fork_parts = 1;
-    opt->leaf_wide_rows = 128;
+    opt->leaf_wide_rows = AE_LEAF_WIDE_DEFAULT;
+    opt->leaf_wide_auto = 1;
     opt->fork_part = 0;
 }
 
