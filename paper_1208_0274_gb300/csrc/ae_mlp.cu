@@ -800,12 +800,14 @@ ae_status ae_mlp_train(ae_mlp *mlp, const float *d_x, const float *d_t, int32_t 
         if (mlp->perm_cap < n) {
             if (mlp->perm) cudaFree(mlp->perm);
             mlp->perm = nullptr;
+            mlp->perm_cap = 0;
             MC(cudaMalloc(&mlp->perm, sizeof(int32_t) * n));
             mlp->perm_cap = n;
         }
         if (mlp->loss_cap < steps) {
             if (mlp->loss) cudaFree(mlp->loss);
             mlp->loss = nullptr;
+            mlp->loss_cap = 0;
             MC(cudaMalloc(&mlp->loss, sizeof(float) * std::max(steps, 1024)));
             mlp->loss_cap = std::max(steps, 1024);
         }
@@ -841,6 +843,8 @@ ae_status ae_mlp_train(ae_mlp *mlp, const float *d_x, const float *d_t, int32_t 
     } catch (const mlp_error &e) {
         cudaGetLastError();
         return e.st;
+    } catch (const std::bad_alloc &) {
+        return AE_ENOMEM;
     }
     return AE_OK;
 }
