@@ -175,10 +175,10 @@ typedef struct {
     int32_t leaf_wide_rows;   /* a walk of the text-position sweep whose row grows past this many
                                  entries continues on a whole thread block (each step spread over
                                  its threads) instead of one warp; 0: never.  With the
-                                 default, 128, and leaf_wide_auto 1 the library chooses: 32 where
-                                 a query's injected rows leave gaps along the text, 1,024 (128 for
-                                 the last walks) where they lie at most positions.  The results
-                                 are the same */
+                                 default, 128, and leaf_wide_auto 1 the library chooses: 256
+                                 while the sweep has tasks and 32 for the last walks (1,024 and
+                                 128 for a query whose injected rows lie at most positions).
+                                 The results are the same */
 } ae_options;
 
 /* Fill *opt with the defaults: qprefix_seed 1, leaf_segment 0, item_columns

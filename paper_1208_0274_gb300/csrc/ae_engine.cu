@@ -856,12 +856,24 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 // ae_options.leaf_wide_rows by default
 constexpr int32_t AE_LEAF_WIDE_DEFAULT = 128;
 
-// Row length at which a warp's walk moves to a block once the sweep's tasks are
-// all taken.  Dense injections make rows of hundreds of entries the rule, and
-// blocks walk those slower than the warps do together, so they take only the
-// widest (1,024) while there are tasks; then the warps run out of work and a
-// block shortens the walks that are left (protein batch: sweep 69 -> 58 ms; from 40
-// to 400 entries the same).
+// Row lengths at which a warp's walk moves to a block by default: while the sweep
+// has tasks (AE_LEAF_WIDE_SPARSE, _DENSE where the query's injections are dense), and
+// once they are all taken (32, AE_LEAF_WIDE_TAIL), which with fewer tasks than warps
+// they are at once.  With tasks left, warps are the better use of the chip and
+// blocks take only the widest walks: 4,000 / 20,000 reads of 150 letters, rows to 74
+// entries, sweep 7.6 / 45.7 ms with blocks from 32 entries on, 4.3 / 20.7 so; 16
+// queries at cheap gaps, rows to 406 entries, 1,020 against 481 (from 96 entries 509,
+// from 128 to 512 the same); dense protein, rows of hundreds of entries, from 128
+// entries 127, 512: 104, 1,024: 69, never: 84.  Without tasks the longest walk sets the
+// time, and a step on a block is faster from the first row past a warp's lanes on
+// (613 bp query 0.76 ms from 32 entries, 0.79 from 64, 1.09 from 128), for dense
+// injections from about 128 (69 -> 58 ms; from 40 to 400 entries the same).
+#ifndef AE_LEAF_WIDE_DENSE
+#define AE_LEAF_WIDE_DENSE 1024
+#endif
+#ifndef AE_LEAF_WIDE_SPARSE
+#define AE_LEAF_WIDE_SPARSE 256
+#endif
 #ifndef AE_LEAF_WIDE_TAIL
 #define AE_LEAF_WIDE_TAIL 128
 #endif
@@ -1324,15 +1336,8 @@ void Search::leaf_phase(int64_t ninj) {
                                                                  : (int64_t)(ninj * w->hit_ratio) + 4096);
     // wide walks move to blocks (not inside the fixed arena of the no-allocation
     // entry point, nor when entries are counted by tier, which only the warp walk does)
-    // the default chooses: where injections leave gaps the few wide walks set the
-    // sweep's time, and a step on a block is faster from the first row past a warp's
-    // lanes on (613 bp query: 0.76 ms from 32 entries, 0.79 from 64, 1.09 from 128);
-    // where they are dense every task walks a wide row and warps are the better use of
-    // the chip (1 M residues, BLOSUM62, sweep: from 128 entries 127 ms, 512: 104,
-    // 1,024: 69, never: 84), until the tasks run out (AE_LEAF_WIDE_TAIL)
     const bool choose = opt.leaf_wide_auto != 0 && opt.leaf_wide_rows == AE_LEAF_WIDE_DEFAULT;
-    const int32_t wide = choose ? 32 : opt.leaf_wide_rows;
-    const int32_t esc_min = (g_arena || opt.tier_stats) ? 0 : wide;
+    const int32_t esc_min = (g_arena || opt.tier_stats) ? 0 : opt.leaf_wide_rows;
     const int32_t esc_max = esc_min > 0 ? AE_LEAF_WIDE_SLOTS : 0;
     // (a search with small row buffers has little room for its workspace)
     const int64_t pool = std::min<int64_t>(AE_LEAF_WIDE_POOL, 1024 * (int64_t)opt.leaf_capacity);
@@ -1393,9 +1398,14 @@ void Search::leaf_phase(int64_t ninj) {
         la.tiers = opt.tier_stats ? 1 : 0;
         la.few = esc_max == 0 ? 1 : 0;
         la.stats = ptr<DevStats>(w->stats);
-        la.esc_min = esc_max > 0 ? esc_min : 0;
-        la.esc_dense = choose && la.esc_min > 0 ? 1024 : la.esc_min;
-        la.esc_tail = std::min(la.esc_dense, choose ? AE_LEAF_WIDE_TAIL : la.esc_min);
+        la.esc_by_density = choose && esc_max > 0 ? 1 : 0;
+        la.esc_min[0] = la.esc_last[0] = esc_max > 0 ? esc_min : 0;
+        if (la.esc_by_density) {
+            la.esc_min[0] = AE_LEAF_WIDE_SPARSE;
+            la.esc_min[1] = AE_LEAF_WIDE_DENSE;
+            la.esc_last[0] = 32;
+            la.esc_last[1] = AE_LEAF_WIDE_TAIL;
+        }
         la.esc_max = esc_max;
         if (esc_max > 0) {
             la.esc_count = ptr<unsigned long long>(w->esc_count);

@@ -870,7 +870,7 @@ __global__ void __launch_bounds__(128, E == 1 ? AE_LEAF_MINB : 2) k_leaf(LeafArg
     const uint64_t jmask = (1ull << a.bj) - 1ull;
     unsigned long long st_rows = 0, st_ent = 0, st_t0 = 0, st_t1 = 0, st_t2 = 0, st_reused = 0;
     bool overflow = false;
-    bool tail = false;   // every task is taken
+    bool tail = a.nseg <= a.nwarps;   // every task is taken (few tasks: at once)
 
     while (!overflow) {
         // one lane reads the counter and the overflow flag, which other warps write meanwhile:
@@ -903,10 +903,10 @@ __global__ void __launch_bounds__(128, E == 1 ? AE_LEAF_MINB : 2) k_leaf(LeafArg
             nk_qid = In.qid;
             nk_e = In.e;
         }
-        // row length at which the walk moves to a block
-        int32_t esc_at = a.esc_min;
-        if (a.esc_min != a.esc_dense && leaf_dense(a, nk_qid)) esc_at = a.esc_dense;
-        if (tail) esc_at = min(esc_at, a.esc_tail);
+        // row length at which the walk moves to a block, now and once the tasks are taken
+        const int dense = a.esc_by_density && leaf_dense(a, nk_qid);
+        const int32_t esc_last = a.esc_last[dense];
+        int32_t esc_at = tail ? esc_last : a.esc_min[dense];
         while (true) {
             if (rlen == 0 && k < kend) {
                 // ---- jump to a lone injected row: it is already a finished row
@@ -1299,11 +1299,11 @@ __global__ void __launch_bounds__(128, E == 1 ? AE_LEAF_MINB : 2) k_leaf(LeafArg
             seg_width = max(seg_width, (unsigned long long)nlen);
             // once every task is taken, warps fall idle while the last wide walks go on, and
             // a block each is the better use of the chip from narrower rows on
-            if (rlen > a.esc_tail && esc_at > a.esc_tail && (seg_steps & 7) == 0) {
+            if (rlen > esc_last && esc_at > esc_last && (seg_steps & 7) == 0) {
                 unsigned long long taken = 0;   // read once for the whole warp: the branches below are its
                 if (lane == 0) taken = *(volatile unsigned long long *)a.next_seg;
                 tail = __shfl_sync(FULL, taken, 0) >= (unsigned long long)a.nseg;
-                if (tail) esc_at = a.esc_tail;
+                if (tail) esc_at = esc_last;
             }
             if (esc_at > 0 && rlen > esc_at) {
                 // a wide row goes on on a whole block (k_leaf_wide), with the rest of
@@ -2163,7 +2163,7 @@ void ae_leaf_sweep(const LeafArgs &a, int blocks, int threads, cudaStream_t st) 
     ++g_launches;
     if (a.few) k_leaf<2><<<blocks, threads, 0, st>>>(a);
     else k_leaf<1><<<blocks, threads, 0, st>>>(a);
-    if (a.esc_min > 0 && a.esc_max > 0) {   // the walks handed on to blocks
+    if (a.esc_max > 0) {   // the walks handed on to blocks
         ++g_launches;
         cudaFuncSetAttribute(k_leaf_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WideSmem));
         k_leaf_wide<<<a.wide_blocks, WIDE_T, sizeof(WideSmem), st>>>(a);
