@@ -511,7 +511,7 @@ struct Search {
     void dna_chain(int64_t &F, int &cur, int64_t &cur_ent, int64_t &lf_ent_base, int64_t &lf_node_base,
                    int64_t &rh_base, int &depth, int levels);
     void dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_base, int64_t &lf_node_base,
-                   int64_t &rh_base, const WorkItem *d_items);
+                   int64_t &rh_base);
     void run_batch_split(const std::vector<WorkItem> &items);
     void compact_hits(int64_t from);
     void leaf_phase(int64_t ninj);
@@ -661,7 +661,7 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
                 dna_chain(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base, depth, chain);
                 continue;
             }
-            dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base, d_items);
+            dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base);
             cur ^= 1;
             ++depth;
             stats.levels++;
@@ -892,13 +892,26 @@ constexpr int32_t AE_LEAF_WIDE_DEFAULT = 128;
 constexpr int AE_CHAIN_MAX = 8;
 
 // Average parent-row length up to which a level's rows are packed over the
-// lanes; longer rows are spread one entry per lane.  Per level (before the
-// packed kernel's last tuning, which took another tenth) of the 100 Mbp
-// text with queries of 10 kbp to 1 Mbp (packed against the walk it replaces):
-// rows of 158 entries 2.4 ms against 6.3, 57: 3.3 / 6.2, 59 (2.0 M nodes):
-// 8.3 / 10.7, 30: 10.6 / 11.8, 13: 20.2 / 15.8, 7.2: 26.2 / 38.8, 5.0: 41.8 /
-// 56.5, 2.3: 13.8 / 26.9, 1.5: 3.5 / 7.3; rows of 441 stay with the spread
-// layout (3.1 ms)
+// lanes; longer rows are spread one entry per lane or, in levels of few nodes, take a
+// block each.  Row time of single levels, 100 Mbp text, random queries (ms):
+//                                              packed   walk  spread  block
+//   1 M letters,  16 k nodes of 610 entries     0.78    5.5    1.88   2.09
+//   8 queries,    33 k nodes of 441             0.92   11.2    2.97
+//   1 M letters, 262 k nodes of 220             3.0     5.2    8.2
+//   8 queries,   131 k nodes of 158             1.75    5.6    8.0
+//   8 queries,   2.0 M nodes of 59              6.9     9.9   17.4
+//   1 M letters, 4.2 M nodes of 41             10.0     8.0   16.4
+//   8 queries,   7.6 M nodes of 30             10.4    11.8   20.2
+//   1 M letters,  46 M nodes of 19             23.7    19.0   45.2
+//   1 M letters,  16 M nodes of 17.6           12.2    21.2   20.2
+//   8 queries,    27 M nodes of 13             20.0    15.5   32.4
+//   8 queries,   239 M nodes of 7.5            52.8    54.4  113.4
+//   8 queries,   303 M nodes of 3.0            27.3    44.9   60.5
+// So the average length alone does not tell the two or three levels of a search where the
+// walk wins a fifth (the ones whose rows first branch) from those where it takes half
+// as long again; over a whole search packed rows win.  The line at 300 lies below where
+// the packed layout stops paying: at 610 and 441 entries it is the fastest as well, at
+// 3,900 (1,024 nodes) the block is (0.58 against 1.06).
 #ifndef AE_PACK_ROW_AVG
 #define AE_PACK_ROW_AVG 300
 #endif
@@ -1015,7 +1028,7 @@ void Search::dna_chain(int64_t &F, int &cur, int64_t &cur_ent, int64_t &lf_ent_b
         if (c.overflow) throw ae_error{AE_ECUDA};
         if (F <= 0) break;
         if (c.retry) {
-            dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base, nullptr);
+            dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base);
         } else {
             if (trace())
                 fprintf(stderr, "[ae level] dna packed nodes %lld (chain) entries %lld triples %lld -> frontier %lld nodes "
@@ -1053,8 +1066,7 @@ void Search::dna_chain(int64_t &F, int &cur, int64_t &cur_ent, int64_t &lf_ent_b
 // capacity the arenas are grown to those totals and the level is run again.
 // Nodes and arenas have the layout of the general route.
 void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_base, int64_t &lf_node_base,
-                       int64_t &rh_base, const WorkItem *d_items) {
-    (void)d_items;
+                       int64_t &rh_base) {
     const int nxt = cur ^ 1;
     // nodes per task: 32 (one per lane) unless the level is too small to give
     // every resident warp a few tasks
@@ -1196,7 +1208,7 @@ void Search::dna_level(int64_t &F, int cur, int64_t &cur_ent, int64_t &lf_ent_ba
             // batch's next ones in the other layouts, which write their rows without gaps
             if (e.st != AE_ENOMEM || !packed) throw;
             no_pack = true;
-            dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base, d_items);
+            dna_level(F, cur, cur_ent, lf_ent_base, lf_node_base, rh_base);
             return;
         }
         run();

@@ -26,18 +26,6 @@ void ae_letter_lut(int32_t alphabet, uint8_t lut[256]) {
     for (int c = 0; c < s; ++c) lut[(uint8_t)a[c]] = (uint8_t)c;
 }
 
-// ASCII -> codes; returns 0 on success, -1 on a letter outside the alphabet.
-int ae_encode_letters(const uint8_t *ascii, int64_t n, int32_t alphabet, uint8_t *codes) {
-    uint8_t lut[256];
-    ae_letter_lut(alphabet, lut);
-    for (int64_t i = 0; i < n; ++i) {
-        uint8_t c = lut[ascii[i]];
-        if (c == 255) return -1;
-        codes[i] = c;
-    }
-    return 0;
-}
-
 // ------------------------------------------------------------------ SA-IS
 // Suffix array by induced sorting (Nong, Zhang & Chan, "Two efficient
 // algorithms for linear time suffix array construction", 2009).  s[0..N) has

@@ -160,7 +160,6 @@ struct HostIndex {
 };
 
 int ae_alphabet_sigma(int32_t alphabet);
-int ae_encode_letters(const uint8_t *ascii, int64_t n, int32_t alphabet, uint8_t *codes);
 void ae_letter_lut(int32_t alphabet, uint8_t lut[256]);
 void ae_host_index_free(HostIndex *h);
 // ready(k) waits until array k is there (false: it could not be had)
