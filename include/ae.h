@@ -176,9 +176,9 @@ typedef struct {
                                  entries continues on a whole thread block (each step spread over
                                  its threads) instead of one warp; 0: never.  With the
                                  default, 128, and leaf_wide_auto 1 the library chooses: 256
-                                 while the sweep has tasks and 32 for the last walks (1,024 and
-                                 128 for a query whose injected rows lie at most positions).
-                                 The results are the same */
+                                 for a few walks while the GPU is full of them and 32 for the
+                                 last ones (1,024 and 128 for a query whose injected rows lie at
+                                 most positions).  The results are the same */
 } ae_options;
 
 /* Fill *opt with the defaults: qprefix_seed 1, leaf_segment 0, item_columns

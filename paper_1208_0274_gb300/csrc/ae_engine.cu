@@ -856,23 +856,32 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
 // ae_options.leaf_wide_rows by default
 constexpr int32_t AE_LEAF_WIDE_DEFAULT = 128;
 
-// Row lengths at which a warp's walk moves to a block by default: while the sweep
-// has tasks (AE_LEAF_WIDE_SPARSE, _DENSE where the query's injections are dense), and
-// once they are all taken (32, AE_LEAF_WIDE_TAIL), which with fewer tasks than warps
-// they are at once.  With tasks left, warps are the better use of the chip and
-// blocks take only the widest walks: 4,000 / 20,000 reads of 150 letters, rows to 74
-// entries, sweep 7.6 / 45.7 ms with blocks from 32 entries on, 4.3 / 20.7 so; 16
-// queries at cheap gaps, rows to 406 entries, 1,020 against 481 (from 96 entries 509,
-// from 128 to 512 the same); dense protein, rows of hundreds of entries, from 128
-// entries 127, 512: 104, 1,024: 69, never: 84.  Without tasks the longest walk sets the
-// time, and a step on a block is faster from the first row past a warp's lanes on
-// (613 bp query 0.76 ms from 32 entries, 0.79 from 64, 1.09 from 128), for dense
-// injections from about 128 (69 -> 58 ms; from 40 to 400 entries the same).
+// Row lengths at which a warp's walk moves to a block by default: while more than
+// AE_LEAF_WIDE_LAST warps a block walk (AE_LEAF_WIDE_SPARSE, _DENSE where the query's
+// injections are dense; at most AE_LEAF_WIDE_EARLY walks a block), and after that (32,
+// AE_LEAF_WIDE_TAIL), which a search of few tasks is at once.
+// With the chip full of walking warps these are the better use of it and blocks take
+// only the widest walks.  20,000 reads of 150 letters, rows to 74 entries: sweep 45.7
+// ms with blocks from 32 entries on, 20.7 with blocks from 256 on and from 32 once
+// the tasks are taken, 16.9 so.  16 queries at cheap gaps, rows to 406 entries: 1,020 /
+// 481 / 397 (with 8 warps a block 399, 16: 423).  Dense protein, six queries: 127 from 128
+// entries on, 512: 104, 1,024: 69, never: 84.  A 900 k letter query against 100 kbp at
+// cheap gaps, 3,125 short walks of rows to 3,000 entries: 32.3 without the two limits,
+// 14.7 with them (8 warps a block 14.9, 16: 19.0).
+// With the chip nearly empty the longest walk sets the time, and a step on a block is
+// faster from the first row past a warp's lanes on (613 bp query 0.76 ms from 32
+// entries, 0.79 from 64, 1.09 from 128).
 #ifndef AE_LEAF_WIDE_DENSE
 #define AE_LEAF_WIDE_DENSE 1024
 #endif
 #ifndef AE_LEAF_WIDE_SPARSE
 #define AE_LEAF_WIDE_SPARSE 256
+#endif
+#ifndef AE_LEAF_WIDE_EARLY
+#define AE_LEAF_WIDE_EARLY 4
+#endif
+#ifndef AE_LEAF_WIDE_LAST
+#define AE_LEAF_WIDE_LAST 4
 #endif
 #ifndef AE_LEAF_WIDE_TAIL
 #define AE_LEAF_WIDE_TAIL 128
@@ -1419,6 +1428,8 @@ void Search::leaf_phase(int64_t ninj) {
             la.esc_last[1] = AE_LEAF_WIDE_TAIL;
         }
         la.esc_max = esc_max;
+        la.esc_early = la.esc_by_density ? std::min(AE_LEAF_WIDE_EARLY * wide_blocks, esc_max) : esc_max;
+        la.last_warps = AE_LEAF_WIDE_LAST * wide_blocks;
         if (esc_max > 0) {
             la.esc_count = ptr<unsigned long long>(w->esc_count);
             la.esc = ptr<EscWalk>(w->esc);

@@ -837,7 +837,7 @@ __device__ __forceinline__ int64_t task_start(const LeafArgs &a, int lane, int64
 // its segment, to a slot of k_leaf_wide (a block of threads per walk); when
 // the slots are taken the warp carries on itself.
 // A step is a chain of scans and dependent loads, so the resident warps set the
-// rate: 6 blocks per SM at one entry per lane (E = 1; 80 registers, some spilled)
+// rate: 6 blocks per SM at one entry per lane (E = 1; 80 registers, 228 bytes of spills)
 // against 3 at two entries (162 registers, 38 % of the issue slots used; 526
 // warp instructions per 32 entries).  Sweeps of a protein batch, a 1 M-letter query
 // and a batch with cheap gaps: 51.7 / 22.9 / 11.3 ms against 58.5 / 28.8 / 16.1
@@ -870,7 +870,7 @@ __global__ void __launch_bounds__(128, E == 1 ? AE_LEAF_MINB : 2) k_leaf(LeafArg
     const uint64_t jmask = (1ull << a.bj) - 1ull;
     unsigned long long st_rows = 0, st_ent = 0, st_t0 = 0, st_t1 = 0, st_t2 = 0, st_reused = 0;
     bool overflow = false;
-    bool tail = a.nseg <= a.nwarps;   // every task is taken (few tasks: at once)
+    bool tail = a.nseg <= a.last_warps;   // few warps still walk
 
     while (!overflow) {
         // one lane reads the counter and the overflow flag, which other warps write meanwhile:
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(128, E == 1 ? AE_LEAF_MINB : 2) k_leaf(LeafArg
             nk_qid = In.qid;
             nk_e = In.e;
         }
-        // row length at which the walk moves to a block, now and once the tasks are taken
+        // row length at which the walk moves to a block, now and once few warps still walk
         const int dense = a.esc_by_density && leaf_dense(a, nk_qid);
         const int32_t esc_last = a.esc_last[dense];
         int32_t esc_at = tail ? esc_last : a.esc_min[dense];
@@ -1297,12 +1297,13 @@ __global__ void __launch_bounds__(128, E == 1 ? AE_LEAF_MINB : 2) k_leaf(LeafArg
             ++st_rows;
             ++seg_steps;
             seg_width = max(seg_width, (unsigned long long)nlen);
-            // once every task is taken, warps fall idle while the last wide walks go on, and
-            // a block each is the better use of the chip from narrower rows on
+            // when tasks run out, warps fall idle while the last wide walks go on, and a block
+            // each is the better use of the chip from narrower rows on.  A warp that finds no
+            // task has counted next_seg past nseg.
             if (rlen > esc_last && esc_at > esc_last && (seg_steps & 7) == 0) {
                 unsigned long long taken = 0;   // read once for the whole warp: the branches below are its
                 if (lane == 0) taken = *(volatile unsigned long long *)a.next_seg;
-                tail = __shfl_sync(FULL, taken, 0) >= (unsigned long long)a.nseg;
+                tail = (int64_t)__shfl_sync(FULL, taken, 0) >= a.nseg + max(a.nwarps - a.last_warps, 0);
                 if (tail) esc_at = esc_last;
             }
             if (esc_at > 0 && rlen > esc_at) {
@@ -1314,7 +1315,8 @@ __global__ void __launch_bounds__(128, E == 1 ? AE_LEAF_MINB : 2) k_leaf(LeafArg
                     // read first so that they cannot wrap)
                     slot = *(volatile unsigned long long *)a.esc_count;
                     at = *(volatile unsigned long long *)(a.esc_count + 1);
-                    if (slot < (unsigned long long)a.esc_max && at + rlen <= (unsigned long long)a.esc_pool_cap) {
+                    if (slot < (unsigned long long)(tail ? a.esc_max : a.esc_early) &&
+                        at + rlen <= (unsigned long long)a.esc_pool_cap) {
                         at = atomicAdd(a.esc_count + 1, (unsigned long long)rlen);
                         slot = at + rlen <= (unsigned long long)a.esc_pool_cap ? atomicAdd(a.esc_count, 1ull)
                                                                                : (unsigned long long)a.esc_max;

@@ -265,15 +265,16 @@ struct LeafArgs {
     int32_t tiers;                // 1: count entries by cost tier
     int32_t few;                  // 1: few warps run, each as fast as it can (two row entries per lane)
     DevStats *stats;
-    // walks whose row grows past esc_min[0] entries (0: never), or esc_last[0] once all
-    // tasks are taken, continue on a whole block (k_leaf_wide) with the rest of their
-    // task's injections; with esc_by_density [1] are the lengths for queries whose
-    // injections are dense.  esc[slot] is the walk's state, its row lies in the pool at esc[slot].row.  esc_count counts
+    // walks whose row grows past esc_min[0] entries (0: never), or esc_last[0] once at most
+    // last_warps warps still have a task, continue on a whole block (k_leaf_wide) with the
+    // rest of their task's injections; with esc_by_density [1] are the lengths for queries
+    // whose injections are dense.  At most esc_early go before that, esc_max in all.
+    // esc[slot] is the walk's state, its row lies in the pool at esc[slot].row.  esc_count counts
     // the slots taken, the pool's entries taken and the walks the blocks have
     // taken; the first two may pass esc_max and esc_pool_cap: a walk that finds no
     // room stays on its warp.  Each of the wide_blocks blocks has 6 * wide_cap
     // words of row buffers at wide_rows.
-    int32_t esc_min[2], esc_last[2], esc_by_density, esc_max;
+    int32_t esc_min[2], esc_last[2], esc_by_density, esc_early, esc_max, last_warps;
     int64_t esc_pool_cap;
     unsigned long long *esc_count;
     struct EscWalk *esc;
