@@ -825,17 +825,17 @@ __device__ __forceinline__ int64_t task_start(const LeafArgs &a, int lane, int64
     return a.ninj;
 }
 
-// One warp per segment of `seg` consecutive injections (sorted by query and
-// text end).  The warp carries a row R along text positions p, p+1, ...:
+// One warp per task, a run of consecutive injections (sorted by query and text
+// end; k_leaf_cuts).  The warp carries a row R along text positions p, p+1, ...:
 //   candidates of row p+1 = the vertical and diagonal slots generated from R
 //   with letter T[p+1], merged by maximum with every injected row at p+1;
 //   then the horizontal-gap finish of Section 2.2 gives row p+1.
 // The walk jumps to the next injection when R has no live entry.  Rows live
 // in per-warp global scratch (cap entries per buffer); a row that outgrows it
 // sets leaf_overflow and the host reruns with a larger cap.
-// A walk whose row grows past esc_min entries is handed on, with the rest of
-// its segment, to a slot of k_leaf_wide (a block of threads per walk); when
-// the slots are taken the warp carries on itself.
+// A walk whose row grows wide (LeafArgs says when) is handed on, with the rest of its
+// task, to k_leaf_wide (a block of threads per walk); without a slot or room for its
+// row the warp carries on itself.
 // A step is a chain of scans and dependent loads, so the resident warps set the
 // rate: 6 blocks per SM at one entry per lane (E = 1; 80 registers, 228 bytes of spills)
 // against 3 at two entries (162 registers, 38 % of the issue slots used; 526
