@@ -514,7 +514,7 @@ __device__ __forceinline__ bool leaf_dense(const LeafArgs &a, int32_t q) {
 //   a span before.  A row lives about as long as its query, so a longer task only
 //   walks one row after the other that could be walked side by side, as in a
 //   tandem repeat that the query holds one copy of (3,000 copies of 171 letters,
-//   613 bp query: sweep 17.3 ms without, 10.6 with this cut),
+//   613 bp query: sweep 17.3 ms without, 13.5 with this cut),
 // - at every multiple of seg if the query's injections are dense.
 // Cut at multiples of 32 injections instead, six homologous reads wrote 13 times
 // the hit records (sweep 100 ms against 17).  One warp per multiple.
