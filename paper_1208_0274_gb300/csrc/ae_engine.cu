@@ -173,7 +173,7 @@ struct Workspace {
     // point hits of the whole search
     DevBuf hkey, hscore, hcount, hk1, hv1;
     // leaf sweep scratch; walks handed on to blocks (state, count, row buffers)
-    DevBuf scratch, next_seg, esc, esc_count, esc_pool, wide_rows, cuts, qrange;
+    DevBuf scratch, next_seg, esc, esc_count, esc_pool, wide_rows, qrange;
     // walk layout of the DNA row kernel: per warp and lane, the count phase's child rows
     DevBuf stage;
     // output
@@ -207,7 +207,7 @@ struct Workspace {
                 &aM[1], &aGa[0], &aGa[1], &nodes[0], &nodes[1], &cnt[0], &cnt[1], &cnt[2], &cnt[3],
                 &cnt[4], &off[0], &off[1], &off[2], &off[3], &off[4], &totals, &scan_tmp, &lj, &lM,
                 &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hkey, &hscore, &hcount, &hk1,
-                &hv1, &scratch, &next_seg, &esc, &esc_count, &esc_pool, &wide_rows, &cuts, &qrange, &stage, &uniq, &uflags, &uoff, &qcount, &stats, &stats_keep, &segs, &ctr, &chain, &seg_cnt, &seg_hit,
+                &hv1, &scratch, &next_seg, &esc, &esc_count, &esc_pool, &wide_rows, &qrange, &stage, &uniq, &uflags, &uoff, &qcount, &stats, &stats_keep, &segs, &ctr, &chain, &seg_cnt, &seg_hit,
                 &task_first, &task_tot, &task_off, &task_tmp, &task_sum, &res, &res_key};
     }
 
@@ -230,7 +230,7 @@ struct Workspace {
     void trim_batch() {
         DevBuf *drop[] = {&aj[0], &aj[1], &aM[0], &aM[1], &aGa[0], &aGa[1], &nodes[0], &nodes[1], &cnt[0], &cnt[1],
                           &cnt[2], &cnt[3], &cnt[4], &off[0], &off[1], &off[2], &off[3], &off[4], &scan_tmp, &lj,
-                          &lM, &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hk1, &hv1, &scratch, &esc_pool, &wide_rows, &cuts,
+                          &lM, &lGa, &inj, &rhits, &sk0, &sv0, &sk1, &sv1, &sort_tmp, &hk1, &hv1, &scratch, &esc_pool, &wide_rows,
                           &uniq,
                           &uflags, &uoff, &segs, &seg_cnt, &seg_hit, &task_first, &task_tot, &task_off, &task_tmp,
                           &res, &res_key};
@@ -581,14 +581,14 @@ void Search::run_batch(const std::vector<WorkItem> &items) {
         ensure(w->sv0, npos * 4, st);
         ensure(w->sk1, npos * 8, st);
         ensure(w->sv1, npos * 4, st);
-        ensure(w->sort_tmp, ae_sort_tmp_words(npos) * 8, st);
+        ensure(w->sort_tmp, ae_sort_tmp_words(npos, !g_arena) * 8, st);
         prof.mark(K_OTHER);
         ae_seed_keys(sa, ptr<uint64_t>(w->sk0), ptr<uint32_t>(w->sv0), st);
         prof.mark(K_OTHER);
         const int key_bits = (sigma == 4 ? 2 : 5) * d0 + bits_for(nitems);
         prof.mark(K_SORT);
         int which = ae_radix_sort(ptr<uint64_t>(w->sk0), ptr<uint32_t>(w->sv0), ptr<uint64_t>(w->sk1),
-                                  ptr<uint32_t>(w->sv1), npos, key_bits, ptr<uint64_t>(w->sort_tmp), st);
+                                  ptr<uint32_t>(w->sv1), npos, key_bits, ptr<uint64_t>(w->sort_tmp), st, !g_arena);
         prof.mark(K_SORT);
         uint64_t *keys = which ? ptr<uint64_t>(w->sk1) : ptr<uint64_t>(w->sk0);
         uint32_t *vals = which ? ptr<uint32_t>(w->sv1) : ptr<uint32_t>(w->sv0);
@@ -1296,12 +1296,12 @@ void Search::compact_hits(int64_t from) {
     if (N <= 1) return;
     ensure(w->hk1, N * 8, st);
     ensure(w->hv1, N * 4, st);
-    ensure(w->sort_tmp, ae_sort_tmp_words(N) * 8, st);
+    ensure(w->sort_tmp, ae_sort_tmp_words(N, !g_arena) * 8, st);
     uint64_t *k0 = ptr<uint64_t>(w->hkey) + from;
     uint32_t *v0 = reinterpret_cast<uint32_t *>(ptr<int32_t>(w->hscore) + from);
     prof.mark(K_SORT);
     int which = ae_radix_sort(k0, v0, ptr<uint64_t>(w->hk1), ptr<uint32_t>(w->hv1), N, be + bj + bq,
-                              ptr<uint64_t>(w->sort_tmp), st);
+                              ptr<uint64_t>(w->sort_tmp), st, !g_arena);
     prof.mark(K_SORT);
     const uint64_t *keys = which ? ptr<uint64_t>(w->hk1) : k0;
     const int32_t *scores = which ? ptr<int32_t>(w->hv1) : reinterpret_cast<int32_t *>(v0);
@@ -1335,12 +1335,12 @@ void Search::leaf_phase(int64_t ninj) {
     ensure(w->sv0, ninj * 4, st);
     ensure(w->sk1, ninj * 8, st);
     ensure(w->sv1, ninj * 4, st);
-    ensure(w->sort_tmp, ae_sort_tmp_words(ninj) * 8, st);
+    ensure(w->sort_tmp, ae_sort_tmp_words(ninj, !g_arena) * 8, st);
     prof.mark(K_SORT);
     ae_inject_keys(ptr<Inject>(w->inj), ninj, ptr<uint64_t>(w->sk0), ptr<uint32_t>(w->sv0), st);
     int which = ae_radix_sort(ptr<uint64_t>(w->sk0), ptr<uint32_t>(w->sv0), ptr<uint64_t>(w->sk1),
                               ptr<uint32_t>(w->sv1), ninj, 32 + bits_for(std::max(nq - 1, 1)),
-                              ptr<uint64_t>(w->sort_tmp), st);
+                              ptr<uint64_t>(w->sort_tmp), st, !g_arena);
     prof.mark(K_SORT);
     const uint32_t *order = which ? ptr<uint32_t>(w->sv1) : ptr<uint32_t>(w->sv0);
     const uint64_t *keys = which ? ptr<uint64_t>(w->sk1) : ptr<uint64_t>(w->sk0);
@@ -1439,11 +1439,16 @@ void Search::leaf_phase(int64_t ninj) {
             la.wide_cap = w->wide_cap;
             la.wide_blocks = wide_blocks;
         }
-        ensure(w->cuts, (size_t)la.nseg * 4, st);
-        if (!one_query) ensure(w->qrange, sizeof(uint2) * (size_t)nq, st);
-        la.qrange = one_query ? nullptr : ptr<uint2>(w->qrange);
-        if (attempt == 0) ae_leaf_cuts(la, keys, ptr<uint2>(w->qrange), ptr<uint32_t>(w->cuts), st);
-        la.cuts = ptr<uint32_t>(w->cuts);
+        // the sort's other buffers hold the cuts and (one range a query, so mostly) the ranges
+        uint32_t *cuts = which ? ptr<uint32_t>(w->sv0) : ptr<uint32_t>(w->sv1);
+        uint2 *qrange = nullptr;
+        if (!one_query) {
+            if (ninj < nq) ensure(w->qrange, sizeof(uint2) * (size_t)nq, st);
+            qrange = ninj < nq ? ptr<uint2>(w->qrange) : which ? ptr<uint2>(w->sk0) : ptr<uint2>(w->sk1);
+        }
+        la.qrange = qrange;
+        if (attempt == 0) ae_leaf_cuts(la, keys, qrange, cuts, st);
+        la.cuts = cuts;
         prof.mark(K_LEAF);
         ++stats.leaf_sweeps;
         const auto t_sweep = std::chrono::steady_clock::now();
@@ -1553,11 +1558,11 @@ int64_t Search::finish(ae_hit **out_dev, std::vector<int64_t> &counts) {
     }
     ensure(w->hk1, N * 8, st);
     ensure(w->hv1, N * 4, st);
-    ensure(w->sort_tmp, ae_sort_tmp_words(N) * 8, st);
+    ensure(w->sort_tmp, ae_sort_tmp_words(N, !g_arena) * 8, st);
     prof.mark(K_SORT);
     int which = ae_radix_sort(ptr<uint64_t>(w->hkey), reinterpret_cast<uint32_t *>(w->hscore.p),
                               ptr<uint64_t>(w->hk1), ptr<uint32_t>(w->hv1), N, be + bj + bq,
-                              ptr<uint64_t>(w->sort_tmp), st);
+                              ptr<uint64_t>(w->sort_tmp), st, !g_arena);
     prof.mark(K_SORT);
     const uint64_t *keys = which ? ptr<uint64_t>(w->hk1) : ptr<uint64_t>(w->hkey);
     const int32_t *scores = which ? ptr<int32_t>(w->hv1) : ptr<int32_t>(w->hscore);

@@ -2048,9 +2048,9 @@ void ae_scan_u32(const uint32_t *const *in, uint64_t *const *out, int W, int64_t
     }
 }
 
-int64_t ae_sort_tmp_words(int64_t N) {
+int64_t ae_sort_tmp_words(int64_t N, bool halves) {
     // enough for any number of pairs up to N (short lists take smaller tiles)
-    const int64_t half = std::min<int64_t>(N, AE_RS_SPLIT);
+    const int64_t half = halves ? std::min<int64_t>(N, AE_RS_SPLIT) : 0;
     const int64_t ntiles = std::max((N + RS_TILE - 1) / RS_TILE, (half + RS_TILE / 2 - 1) / (RS_TILE / 2));
     int64_t h = 256 * ntiles;
     // hist (u32, packed two per word) + offsets (u64) + scan tmp
@@ -2083,7 +2083,7 @@ int rs_passes(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_t N,
 }
 
 int ae_radix_sort(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_t N, int bits, uint64_t *tmp,
-                  cudaStream_t st) {
+                  cudaStream_t st, bool halves) {
     if (N <= 1 || bits <= 0) return 0;
     if (N <= RS_SMALL) {
         ++g_launches;
@@ -2092,7 +2092,7 @@ int ae_radix_sort(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_
         k_rs_small<<<1, RS_ST, smem, st>>>(k0, v0, (int)N, bits);
         return 0;
     }
-    return N <= AE_RS_SPLIT ? rs_passes<RS_I / 2>(k0, v0, k1, v1, N, bits, tmp, st)
+    return halves && N <= AE_RS_SPLIT ? rs_passes<RS_I / 2>(k0, v0, k1, v1, N, bits, tmp, st)
                             : rs_passes<RS_I>(k0, v0, k1, v1, N, bits, tmp, st);
 }
 

@@ -18,10 +18,11 @@ void ae_scan_u32(const uint32_t *const *in, uint64_t *const *out, int W, int64_t
 
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of the
 // key.  Ping-pong buffers k0/v0 (input) and k1/v1; returns 0 if the result
-// ended in k0/v0, 1 if in k1/v1.  tmp must hold ae_sort_tmp_words(N) u64.
-int64_t ae_sort_tmp_words(int64_t N);
+// ended in k0/v0, 1 if in k1/v1.  tmp must hold ae_sort_tmp_words(N, halves) u64; with `halves` short
+// lists take smaller tiles, which need more of it.
+int64_t ae_sort_tmp_words(int64_t N, bool halves = true);
 int ae_radix_sort(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_t N, int bits,
-                  uint64_t *tmp, cudaStream_t st);
+                  uint64_t *tmp, cudaStream_t st, bool halves = true);
 
 // Suffix array of the n codes at d_codes (read backwards with `reversed`)
 // followed by a unique smallest sentinel, into d_sa[0..n] (device), by prefix
